@@ -182,7 +182,7 @@ struct mk_ctx {
   size_t scan_cap = 0;
   double *d_partials = nullptr;
   size_t partials_cap = 0;  // doubles
-  mk_stats_out *d_stats = nullptr, *h_stats = nullptr;
+  mk_stats_out *h_stats = nullptr;  // pinned; k_finalize writes it
   int64_t *h_total = nullptr;  // pinned
   int skewer_threads = 256;
   // launch configurations chosen by the autotuner, per kernel variant
@@ -439,8 +439,9 @@ int ensure_zbin(mk_ctx *ctx, const mk_stat_bins *b) {
   return MK_OK;
 }
 
-int read_error_word(mk_ctx *ctx) {
-  CK(cudaMemcpyAsync(ctx->h_err, ctx->d_err, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream));
+// Wait for the stream, then report (and clear) the device errors that the
+// work before left in h_err.
+int sync_error_word(mk_ctx *ctx) {
   CK(cudaStreamSynchronize(ctx->stream));
   const int e = *ctx->h_err;
   if (e) {
@@ -467,6 +468,25 @@ int time_end(mk_ctx *ctx) {
 }
 
 // persistent grids: as many resident CTAs as the SMs hold
+int read_error_word(mk_ctx *ctx) {
+  CK(cudaMemcpyAsync(ctx->h_err, ctx->d_err, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream));
+  return sync_error_word(ctx);
+}
+
+// statistics and error word into page-locked host memory (k_finalize writes
+// them there itself)
+int enqueue_finalize(mk_ctx *ctx, const double *partials, int nparts, const mk_stat_bins *b) {
+  CK(launch_finalize(partials, nparts, b->n_z, b->n_k, b->n_fft, ctx->d_err, ctx->h_stats, ctx->h_err, ctx->stream));
+  return MK_OK;
+}
+
+// the statistics of the enqueued work, once the stream is idle
+int take_stats(mk_ctx *ctx, mk_stats_out *h_out) {
+  const int rc = sync_error_word(ctx);
+  if (rc == MK_OK) std::memcpy(h_out, ctx->h_stats, sizeof(mk_stats_out));
+  return rc;
+}
+
 // (at most ctx->grid_cap CTAs when a cap is set)
 int capped(mk_ctx *ctx, int grid) { return ctx->grid_cap > 0 && grid > ctx->grid_cap ? ctx->grid_cap : grid; }
 
@@ -563,15 +583,6 @@ SkewerParams skewer_params(mk_ctx *ctx, const mk_box *box, const mk_skewer *d_sk
   return S;
 }
 
-int finish_stats(mk_ctx *ctx, int nparts, const mk_stat_bins *b, mk_stats_out *h_out) {
-  CK(launch_finalize(ctx->d_partials, nparts, b->n_z, b->n_k, b->n_fft, ctx->d_stats, ctx->stream));
-  CK(cudaMemcpyAsync(ctx->h_stats, ctx->d_stats, sizeof(mk_stats_out), cudaMemcpyDeviceToHost, ctx->stream));
-  int rc = read_error_word(ctx);  // synchronises
-  if (rc) return rc;
-  std::memcpy(h_out, ctx->h_stats, sizeof(mk_stats_out));
-  return MK_OK;
-}
-
 }  // namespace
 
 // ====================================================================== C ABI
@@ -607,7 +618,6 @@ int mk_create(mk_ctx **out, int device, void *cuda_stream, const mk_cosmo *cosmo
         cudaMalloc(&ctx->d_err, sizeof(int)) != cudaSuccess || cudaMemset(ctx->d_err, 0, sizeof(int)) != cudaSuccess ||
         cudaMallocHost(&ctx->h_err, sizeof(int)) != cudaSuccess ||
         cudaMallocHost(&ctx->h_total, sizeof(int64_t)) != cudaSuccess ||
-        cudaMalloc(&ctx->d_stats, sizeof(mk_stats_out)) != cudaSuccess ||
         cudaMallocHost(&ctx->h_stats, sizeof(mk_stats_out)) != cudaSuccess) {
       rc = MK_ENOMEM;
       break;
@@ -646,7 +656,6 @@ void mk_destroy(mk_ctx *ctx) {
   cudaFree(ctx->d_segoff);
   cudaFree(ctx->d_scan_ws);
   cudaFree(ctx->d_partials);
-  cudaFree(ctx->d_stats);
   cudaFreeHost(ctx->h_stats);
   if (ctx->graph) cudaGraphExecDestroy(ctx->graph);
   if (ctx->ev0) cudaEventDestroy(ctx->ev0);
@@ -890,7 +899,8 @@ int stats_pass(mk_ctx *ctx, const mk_skewer_params *params, const mk_skewer *d_s
   if ((rc = time_begin(ctx))) return rc;
   CK(launch_stats(P, bins->n_fft, grid, threads, ctx->stream));
   if ((rc = time_end(ctx))) return rc;
-  return finish_stats(ctx, grid, bins, h_out);
+  if ((rc = enqueue_finalize(ctx, ctx->d_partials, grid, bins))) return rc;
+  return take_stats(ctx, h_out);
 }
 }  // namespace
 
@@ -976,12 +986,7 @@ int mk_run(mk_ctx *ctx, const mk_box *box, const mk_qso *d_qso, int64_t n_qso, c
     if (timed && (r = time_begin(ctx))) return r;
     CK(launch_skewer(S, params->n_fft, variant, c.minb, grid, c.threads, ctx->stream));
     if (timed && (r = time_end(ctx))) return r;
-    if (stats) {
-      CK(launch_finalize(ctx->d_partials, grid, bins->n_z, bins->n_k, bins->n_fft, ctx->d_stats, ctx->stream));
-      CK(cudaMemcpyAsync(ctx->h_stats, ctx->d_stats, sizeof(mk_stats_out), cudaMemcpyDeviceToHost, ctx->stream));
-      CK(cudaMemcpyAsync(ctx->h_err, ctx->d_err, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream));
-    }
-    return MK_OK;
+    return stats ? enqueue_finalize(ctx, ctx->d_partials, grid, bins) : MK_OK;
   };
   auto ensure_partials = [&](int grid) -> int {
     if (!stats) return MK_OK;
@@ -1066,12 +1071,7 @@ int mk_run(mk_ctx *ctx, const mk_box *box, const mk_qso *d_qso, int64_t n_qso, c
   } else {
     if ((rc = enqueue(cfg, grid, true))) return rc;
   }
-  if (!stats) return MK_OK;
-  CK(cudaStreamSynchronize(ctx->stream));
-  const int e = *ctx->h_err;
-  if (e) return read_error_word(ctx);
-  std::memcpy(h_out, ctx->h_stats, sizeof(mk_stats_out));
-  return MK_OK;
+  return stats ? take_stats(ctx, h_out) : MK_OK;
 }
 
 namespace {
@@ -1191,14 +1191,9 @@ int mk_run_host(mk_ctx *ctx, const mk_box *box, const mk_qso *h_qso, int64_t n_q
       CK(cudaEventRecord(ctx->ev_copy[c][k], ctx->copy_st[c]));
     }
   }
-  if (stats) {
-    CK(launch_finalize(ctx->d_partials, grid * K, bins->n_z, bins->n_k, bins->n_fft, ctx->d_stats, s0));
-    CK(cudaMemcpyAsync(ctx->h_stats, ctx->d_stats, sizeof(mk_stats_out), cudaMemcpyDeviceToHost, s0));
-  }
+  if (stats && (rc = enqueue_finalize(ctx, ctx->d_partials, grid * K, bins))) return rc;
   for (int c = 0; c < MK_HOST_COPY_STREAMS; ++c) CK(cudaStreamWaitEvent(s0, ctx->ev_copy[c][K - 1], 0));
-  if ((rc = read_error_word(ctx))) return rc;  // synchronises s0, after every copy
-  if (stats) std::memcpy(h_out, ctx->h_stats, sizeof(mk_stats_out));
-  return MK_OK;
+  return stats ? take_stats(ctx, h_out) : read_error_word(ctx);  // synchronises s0, after every copy
 }
 
 int mk_launch_config(mk_ctx *ctx, int32_t n_fft, int32_t layout, int32_t big_box, uint32_t flags,
@@ -1274,7 +1269,20 @@ extern "C" int mk_stats_merge(const mk_stats_out *parts, int32_t n_parts, const 
       tot.n_seg[zb] += parts[p].n_seg[zb];
     }
   const double per_bin = static_cast<double>(bins->n_fft / 2) / bins->n_k;
-  for (int zb = 0; zb < bins->n_z; ++zb) finalize_bin(&tot, zb, bins->n_k, per_bin);
+  for (int zb = 0; zb < bins->n_z; ++zb) {
+    mk_stats_bin b{};
+    std::memcpy(b.sums, tot.sums[zb], sizeof(b.sums));
+    std::memcpy(b.p1d_sum, tot.p1d_sum[zb], sizeof(b.p1d_sum));
+    b.n_seg = tot.n_seg[zb];
+    finalize_bin_scalars(&b);
+    for (int k = 0; k < bins->n_k; ++k) finalize_bin_p1d(&b, k, per_bin);
+    tot.mean_flux[zb] = b.mean_flux;
+    tot.sigma_f[zb] = b.sigma_f;
+    tot.b_f[zb] = b.b_f;
+    tot.beta_f[zb] = b.beta_f;
+    std::memcpy(tot.p1d_f[zb], b.p1d_f, sizeof(b.p1d_f));
+    std::memcpy(tot.p1d_df[zb], b.p1d_df, sizeof(b.p1d_df));
+  }
   std::memcpy(out, &tot, sizeof(tot));
   return MK_OK;
 }
@@ -1282,8 +1290,8 @@ extern "C" int mk_stats_merge(const mk_stats_out *parts, int32_t n_parts, const 
 // ====================================================================== statistics without allocation
 // Scratch of mk_stats_static: one fixed array in the library's device memory
 // instead of the context's growable workspace.  Layout, in 256-byte aligned
-// pieces: the device copy of the result, segment counts, segment offsets,
-// scan tile sums, then per-CTA FP64 partial sums in the remaining space.
+// pieces: segment counts, segment offsets, scan tile sums, then per-CTA FP64
+// partial sums in the remaining space.
 static __device__ __align__(256) unsigned char g_stats_scratch[MK_STATIC_SCRATCH_BYTES];
 
 namespace {
@@ -1341,12 +1349,11 @@ extern "C" int mk_stats_static(mk_ctx *ctx, const mk_skewer_params *params, cons
   unsigned char *base = nullptr;
   if ((rc = stats_scratch_address(ctx, &base))) return rc;
 
-  const size_t off_cnt = align256(sizeof(mk_stats_out));
+  const size_t off_cnt = 0;
   const size_t off_seg = off_cnt + align256(sizeof(int64_t) * MK_STATIC_MAX_SKEWERS);
   const size_t off_tiles = off_seg + align256(sizeof(int64_t) * (MK_STATIC_MAX_SKEWERS + 1));
   const size_t off_part = off_tiles + align256(scan_workspace_bytes(MK_STATIC_MAX_SKEWERS));
   if (off_part >= MK_STATIC_SCRATCH_BYTES) return fail(ctx, MK_EINVAL, "static scratch layout overflow");
-  mk_stats_out *d_out = reinterpret_cast<mk_stats_out *>(base);
   int64_t *d_cnt = reinterpret_cast<int64_t *>(base + off_cnt);
   int64_t *d_seg = reinterpret_cast<int64_t *>(base + off_seg);
   void *d_tiles = base + off_tiles;
@@ -1388,11 +1395,8 @@ extern "C" int mk_stats_static(mk_ctx *ctx, const mk_skewer_params *params, cons
   if ((rc = time_begin(ctx))) return rc;
   CK(launch_stats(P, bins->n_fft, grid, threads, ctx->stream));
   if ((rc = time_end(ctx))) return rc;
-  CK(launch_finalize(d_part, grid, bins->n_z, bins->n_k, bins->n_fft, d_out, ctx->stream));
-  CK(cudaMemcpyAsync(ctx->h_stats, d_out, sizeof(mk_stats_out), cudaMemcpyDeviceToHost, ctx->stream));
-  if ((rc = read_error_word(ctx))) return rc;  // synchronises
-  std::memcpy(h_out, ctx->h_stats, sizeof(mk_stats_out));
-  return MK_OK;
+  if ((rc = enqueue_finalize(ctx, d_part, grid, bins))) return rc;
+  return take_stats(ctx, h_out);
 }
 
 // ====================================================================== internal accessors

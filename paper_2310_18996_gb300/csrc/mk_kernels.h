@@ -93,7 +93,9 @@ enum BoxPass : int {
   kBoxInvXOut = 5  // inverse FFT along x, lines written into the output layout (or in place)
 };
 cudaError_t launch_box_pass(const BoxPassParams &P, int mode, int sms, cudaStream_t st);
-cudaError_t launch_finalize(const double *partials, int nparts, int n_z, int n_k, int n_fft, mk_stats_out *out,
-                            cudaStream_t st);
+// Sums the partials in a fixed order into *out and copies the error word to
+// *err_out; both are page-locked host memory, valid once the stream is idle.
+cudaError_t launch_finalize(const double *partials, int nparts, int n_z, int n_k, int n_fft, const int *err,
+                            mk_stats_out *out, int *err_out, cudaStream_t st);
 
 }  // namespace mk

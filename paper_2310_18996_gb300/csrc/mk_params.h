@@ -46,20 +46,27 @@ struct StatLayout {
   __host__ __device__ int size() const { return n_z * (MK_NSUM + n_k + 1); }
 };
 
-// Derived statistics of z bin zb from its raw sums (out->sums[zb],
-// p1d_sum[zb], n_seg[zb]), which the caller has filled: F-bar, sigma_F,
-// P1D_F per mode, P1D_F / F-bar^2, and b_F, beta_F from the least-squares
-// fit F ~ F0 + k_d delta + k_e eta (Sec. 2.6, Sec. 4.1).  per_bin: modes per k
-// bin, (n_fft / 2) / n_k.  The finalize kernel and the host-side merge of
-// per-rank sums (mk_stats_merge) both use it.
-__host__ __device__ inline void finalize_bin(mk_stats_out *out, int zb, int n_k, double per_bin) {
-  const double *s = out->sums[zb];
+// One z bin of mk_stats_out.
+struct mk_stats_bin {
+  double sums[MK_NSUM], p1d_sum[MK_MAX_KBINS], n_seg;
+  double mean_flux, sigma_f, b_f, beta_f;
+  double p1d_f[MK_MAX_KBINS], p1d_df[MK_MAX_KBINS];
+};
+
+// Derived statistics of a z bin from its raw sums (sums, p1d_sum, n_seg), the
+// rest of the bin being zero: F-bar, sigma_F, and b_F, beta_F from the
+// least-squares fit F ~ F0 + k_d delta + k_e eta (Sec. 2.6, Sec. 4.1); then, per
+// k bin, P1D_F per mode and P1D_F / F-bar^2.  per_bin: modes per k bin,
+// (n_fft / 2) / n_k.  The finalize kernel and the host-side merge of per-rank
+// sums (mk_stats_merge) both use them.
+__host__ __device__ inline void finalize_bin_scalars(mk_stats_bin *b) {
+  const double *s = b->sums;
   const double n = s[0];
   if (n <= 0.0) return;
   const double fbar = s[1] / n;
-  out->mean_flux[zb] = fbar;
+  b->mean_flux = fbar;
   const double varf = s[2] / n - fbar * fbar;
-  out->sigma_f[zb] = varf > 0.0 ? sqrt(varf) : 0.0;
+  b->sigma_f = varf > 0.0 ? sqrt(varf) : 0.0;
   const double md = s[3] / n, me = s[4] / n;
   const double cdd = s[5] / n - md * md, cee = s[6] / n - me * me, cde = s[7] / n - md * me;
   const double vfd = s[8] / n - fbar * md, vfe = s[9] / n - fbar * me;
@@ -67,16 +74,15 @@ __host__ __device__ inline void finalize_bin(mk_stats_out *out, int zb, int n_k,
   if (det != 0.0) {
     const double kd = (cee * vfd - cde * vfe) / det;
     const double ke = (cdd * vfe - cde * vfd) / det;
-    out->b_f[zb] = kd / fbar;
-    out->beta_f[zb] = kd != 0.0 ? ke / kd : 0.0;
+    b->b_f = kd / fbar;
+    b->beta_f = kd != 0.0 ? ke / kd : 0.0;
   }
-  const double ns = out->n_seg[zb];
-  if (ns > 0.0) {
-    for (int k = 0; k < n_k; ++k) {
-      out->p1d_f[zb][k] = out->p1d_sum[zb][k] / (ns * per_bin);
-      out->p1d_df[zb][k] = out->p1d_f[zb][k] / (fbar * fbar);
-    }
-  }
+}
+
+__host__ __device__ inline void finalize_bin_p1d(mk_stats_bin *b, int k, double per_bin) {
+  if (b->sums[0] <= 0.0 || b->n_seg <= 0.0) return;
+  b->p1d_f[k] = b->p1d_sum[k] / (b->n_seg * per_bin);
+  b->p1d_df[k] = b->p1d_f[k] / (b->mean_flux * b->mean_flux);
 }
 
 // Everything the fused / split skewer kernels read.
