@@ -158,12 +158,16 @@ struct mk_ctx {
   double *d_zpix = nullptr, *d_cumz = nullptr;
   float *d_gpix = nullptr;
   float4 *d_pixtab = nullptr;
-  int16_t *d_zbin = nullptr, *d_segzbin = nullptr;
-  int32_t *d_bin_end = nullptr;  // MK_MAX_ZBINS + 2 entries
+  // z-bin tables, one set for fine pixels and one for rebinned ones
+  struct ZTables {
+    int16_t *zbin = nullptr, *segzbin = nullptr;
+    int32_t *bin_end = nullptr;  // MK_MAX_ZBINS + 2 entries
+    bool valid = false;
+    mk_stat_bins bins{};
+    int32_t rebin = 0;
+  } zt[2];
   bool pixtab_valid = false;
   mk_fgpa_nodes nodes_key{};
-  bool zbin_valid = false;
-  mk_stat_bins bins_key{};
   // small-scale amplitudes and twiddles
   float *d_amp = nullptr;
   std::vector<double> amp_key;
@@ -286,28 +290,32 @@ int ensure_pixel_tables(mk_ctx *ctx, double dr) {
   cudaFree(ctx->d_cumz);
   cudaFree(ctx->d_gpix);
   cudaFree(ctx->d_pixtab);
-  cudaFree(ctx->d_zbin);
-  cudaFree(ctx->d_segzbin);
+  for (auto &z : ctx->zt) {
+    cudaFree(z.zbin);
+    cudaFree(z.segzbin);
+    z.zbin = z.segzbin = nullptr;
+    z.valid = false;
+  }
   cudaFree(ctx->d_zwin);
   ctx->d_zwin = nullptr;
   ctx->d_zpix = ctx->d_cumz = nullptr;
   ctx->d_gpix = nullptr;
   ctx->d_pixtab = nullptr;
-  ctx->d_zbin = ctx->d_segzbin = nullptr;
   if (cudaMalloc(&ctx->d_zpix, sizeof(double) * jmax) != cudaSuccess ||
       cudaMalloc(&ctx->d_cumz, sizeof(double) * (jmax + 1)) != cudaSuccess ||
       cudaMalloc(&ctx->d_gpix, sizeof(float) * jmax) != cudaSuccess ||
-      cudaMalloc(&ctx->d_pixtab, sizeof(float4) * jmax) != cudaSuccess ||
-      cudaMalloc(&ctx->d_zbin, sizeof(int16_t) * jmax) != cudaSuccess ||
-      cudaMalloc(&ctx->d_segzbin, sizeof(int16_t) * jmax) != cudaSuccess)
+      cudaMalloc(&ctx->d_pixtab, sizeof(float4) * jmax) != cudaSuccess)
     return fail(ctx, MK_ENOMEM, "pixel tables");
+  for (auto &z : ctx->zt)
+    if (cudaMalloc(&z.zbin, sizeof(int16_t) * jmax) != cudaSuccess ||
+        cudaMalloc(&z.segzbin, sizeof(int16_t) * jmax) != cudaSuccess)
+      return fail(ctx, MK_ENOMEM, "pixel tables");
   CK(cudaMemcpy(ctx->d_zpix, z.data(), sizeof(double) * jmax, cudaMemcpyHostToDevice));
   CK(cudaMemcpy(ctx->d_cumz, cz.data(), sizeof(double) * (jmax + 1), cudaMemcpyHostToDevice));
   CK(cudaMemcpy(ctx->d_gpix, g.data(), sizeof(float) * jmax, cudaMemcpyHostToDevice));
   ctx->dr = dr;
   ctx->j_max = jmax;
   ctx->pixtab_valid = false;
-  ctx->zbin_valid = false;
   return MK_OK;
 }
 
@@ -425,17 +433,23 @@ int ensure_pixtab(mk_ctx *ctx, const mk_fgpa_nodes *nd) {
   return MK_OK;
 }
 
-int ensure_zbin(mk_ctx *ctx, const mk_stat_bins *b) {
-  if (ctx->zbin_valid && std::memcmp(&ctx->bins_key, b, sizeof(*b)) == 0) return MK_OK;
-  if (!ctx->d_bin_end) {
-    ++ctx->generation;
-    CK(cudaMalloc(&ctx->d_bin_end, sizeof(int32_t) * (MK_MAX_ZBINS + 2)));
-  }
-  CK(launch_zbin(ctx->d_zpix, ctx->d_cumz, ctx->j_max, b->z_lo, b->dz, b->n_z, b->n_fft, ctx->d_zbin,
-                 ctx->d_segzbin, ctx->stream));
-  CK(launch_bin_end(ctx->d_zbin, ctx->j_max, b->n_z, ctx->d_bin_end, ctx->stream));
-  ctx->bins_key = *b;
-  ctx->zbin_valid = true;
+// The z-bin tables of `b` for output pixels of `rebin` fine pixels.  Both sets
+// get their memory at once, so that a later call with another rebin only runs
+// kernels.
+int ensure_zbin(mk_ctx *ctx, const mk_stat_bins *b, int rebin) {
+  mk_ctx::ZTables &z = ctx->zt[rebin > 1];
+  if (z.valid && z.rebin == rebin && std::memcmp(&z.bins, b, sizeof(*b)) == 0) return MK_OK;
+  for (auto &q : ctx->zt)
+    if (!q.bin_end) {
+      ++ctx->generation;
+      CK(cudaMalloc(&q.bin_end, sizeof(int32_t) * (MK_MAX_ZBINS + 2)));
+    }
+  CK(launch_zbin(ctx->d_zpix, ctx->d_cumz, ctx->j_max, b->z_lo, b->dz, b->n_z, b->n_fft, rebin, z.zbin, z.segzbin,
+                 ctx->stream));
+  CK(launch_bin_end(z.zbin, ctx->j_max, b->n_z, z.bin_end, ctx->stream));
+  z.bins = *b;
+  z.rebin = rebin;
+  z.valid = true;
   return MK_OK;
 }
 
@@ -454,20 +468,6 @@ int sync_error_word(mk_ctx *ctx) {
   return MK_OK;
 }
 
-int time_begin(mk_ctx *ctx) {
-  if (ctx->timing) CK(cudaEventRecord(ctx->ev0, ctx->stream));
-  return MK_OK;
-}
-
-int time_end(mk_ctx *ctx) {
-  if (ctx->timing) {
-    CK(cudaEventRecord(ctx->ev1, ctx->stream));
-    ctx->timed = true;
-  }
-  return MK_OK;
-}
-
-// persistent grids: as many resident CTAs as the SMs hold
 int read_error_word(mk_ctx *ctx) {
   CK(cudaMemcpyAsync(ctx->h_err, ctx->d_err, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream));
   return sync_error_word(ctx);
@@ -487,6 +487,20 @@ int take_stats(mk_ctx *ctx, mk_stats_out *h_out) {
   return rc;
 }
 
+int time_begin(mk_ctx *ctx) {
+  if (ctx->timing) CK(cudaEventRecord(ctx->ev0, ctx->stream));
+  return MK_OK;
+}
+
+int time_end(mk_ctx *ctx) {
+  if (ctx->timing) {
+    CK(cudaEventRecord(ctx->ev1, ctx->stream));
+    ctx->timed = true;
+  }
+  return MK_OK;
+}
+
+// persistent grids: as many resident CTAs as the SMs hold
 // (at most ctx->grid_cap CTAs when a cap is set)
 int capped(mk_ctx *ctx, int grid) { return ctx->grid_cap > 0 && grid > ctx->grid_cap ? ctx->grid_cap : grid; }
 
@@ -566,7 +580,7 @@ SkewerParams skewer_params(mk_ctx *ctx, const mk_box *box, const mk_skewer *d_sk
   S.box_e = box->e;
   S.lgn = box->lgn;
   S.pixtab = ctx->d_pixtab;
-  S.zbin = ctx->d_zbin;
+  S.zbin = ctx->zt[0].zbin;
   S.cumz = ctx->d_cumz;
   S.amp = ctx->d_amp;
   S.ps_nodes = ctx->ps_nodes;
@@ -575,8 +589,8 @@ SkewerParams skewer_params(mk_ctx *ctx, const mk_box *box, const mk_skewer *d_sk
   S.tw = ctx->d_tw[tw_slot(p->n_fft)];
   S.seed = p->seed;
   S.j_max = ctx->j_max;
-  S.segzbin = ctx->d_segzbin;
-  S.bin_end = ctx->d_bin_end;
+  S.segzbin = ctx->zt[0].segzbin;
+  S.bin_end = ctx->zt[0].bin_end;
   S.err = ctx->d_err;
   S.dr = p->dr;
   S.p1d_scale = static_cast<float>(p->dr / p->n_fft);
@@ -644,9 +658,11 @@ void mk_destroy(mk_ctx *ctx) {
   cudaFree(ctx->d_cumz);
   cudaFree(ctx->d_gpix);
   cudaFree(ctx->d_pixtab);
-  cudaFree(ctx->d_zbin);
-  cudaFree(ctx->d_segzbin);
-  cudaFree(ctx->d_bin_end);
+  for (auto &z : ctx->zt) {
+    cudaFree(z.zbin);
+    cudaFree(z.segzbin);
+    cudaFree(z.bin_end);
+  }
   cudaFree(ctx->d_amp);
   cudaFree(ctx->d_zwin);
   cudaFree(ctx->d_pk);
@@ -859,7 +875,7 @@ int stats_pass(mk_ctx *ctx, const mk_skewer_params *params, const mk_skewer *d_s
   if ((d_delta == nullptr) != (d_eta == nullptr)) return fail(ctx, MK_EINVAL, "d_delta and d_eta go together");
   CK(cudaSetDevice(ctx->device));
   if ((rc = ensure_pixel_tables(ctx, params->dr)) || (rc = ensure_counts(ctx, n_sk)) ||
-      (rc = ensure_twiddles(ctx, bins->n_fft)) || (rc = ensure_zbin(ctx, bins)))
+      (rc = ensure_twiddles(ctx, bins->n_fft)) || (rc = ensure_zbin(ctx, bins, rebin)))
     return rc;
   if (nodes && (rc = ensure_pixtab(ctx, nodes))) return rc;
   const int threads = 256;
@@ -880,18 +896,15 @@ int stats_pass(mk_ctx *ctx, const mk_skewer_params *params, const mk_skewer *d_s
   P.delta = d_delta;
   P.eta = d_eta;
   P.rebin = rebin;
-  P.zbin = ctx->d_zbin;
-  P.segzbin = ctx->d_segzbin;
-  P.bin_end = ctx->d_bin_end;
+  const mk_ctx::ZTables &zt = ctx->zt[rebin > 1];
+  P.zbin = zt.zbin;
+  P.segzbin = zt.segzbin;
+  P.bin_end = zt.bin_end;
   P.p1d_scale = static_cast<float>(rebin * params->dr / bins->n_fft);
-  P.cumz = ctx->d_cumz;
   P.tw = ctx->d_tw[tw_slot(bins->n_fft)];
   P.j_max = ctx->j_max;
   P.n_z = bins->n_z;
   P.n_k = bins->n_k;
-  P.z_lo = bins->z_lo;
-  P.dz = bins->dz;
-  P.dr = params->dr;
   P.partials = ctx->d_partials;
   P.err = ctx->d_err;
   P.wait_test = ctx->wait_test;
@@ -954,7 +967,7 @@ int mk_run(mk_ctx *ctx, const mk_box *box, const mk_qso *d_qso, int64_t n_qso, c
       (rc = ensure_twiddles(ctx, params->n_fft)) || (rc = ensure_amp(ctx, params)) ||
       (rc = ensure_pixtab(ctx, nodes)))
     return rc;
-  if (stats && (rc = ensure_zbin(ctx, bins))) return rc;
+  if (stats && (rc = ensure_zbin(ctx, bins, 1))) return rc;
   const StatLayout L{stats ? bins->n_z : 0, stats ? bins->n_k : 0};
 
   // the launch shape: tuned, or tune now, or the default
@@ -1112,7 +1125,7 @@ int mk_run_host(mk_ctx *ctx, const mk_box *box, const mk_qso *h_qso, int64_t n_q
       (rc = ensure_twiddles(ctx, params->n_fft)) || (rc = ensure_amp(ctx, params)) ||
       (rc = ensure_pixtab(ctx, nodes)) || (rc = ensure_host_path(ctx)))
     return rc;
-  if (stats && (rc = ensure_zbin(ctx, bins))) return rc;
+  if (stats && (rc = ensure_zbin(ctx, bins, 1))) return rc;
   const size_t nq = static_cast<size_t>(n_qso);
   if ((rc = grow(ctx, &ctx->d_hq, &ctx->hq_cap, sizeof(mk_qso) * (nq ? nq : 1))) ||
       (rc = grow(ctx, &ctx->d_hsk, &ctx->hsk_cap, sizeof(mk_skewer) * (nq ? nq : 1))) ||
@@ -1341,11 +1354,11 @@ extern "C" int mk_stats_static(mk_ctx *ctx, const mk_skewer_params *params, cons
   // the z-bin tables: the per-pixel ones come with the pixel tables, the
   // bin-end table with the first allocating statistics call; rebuilding them
   // for other bins only runs kernels into that memory
-  if (!ctx->d_bin_end)
+  if (!ctx->zt[0].bin_end)
     return fail(ctx, MK_EINVAL,
                 "no z-bin tables on this context: run an allocating statistics call (mk_stats, mk_flux_stats, "
                 "or mk_run with MK_STATS) first");
-  if ((rc = ensure_zbin(ctx, bins))) return rc;
+  if ((rc = ensure_zbin(ctx, bins, rebin))) return rc;
   unsigned char *base = nullptr;
   if ((rc = stats_scratch_address(ctx, &base))) return rc;
 
@@ -1378,18 +1391,15 @@ extern "C" int mk_stats_static(mk_ctx *ctx, const mk_skewer_params *params, cons
   P.delta = d_delta;
   P.eta = d_eta;
   P.rebin = rebin;
-  P.zbin = ctx->d_zbin;
-  P.segzbin = ctx->d_segzbin;
-  P.bin_end = ctx->d_bin_end;
+  const mk_ctx::ZTables &zt = ctx->zt[rebin > 1];
+  P.zbin = zt.zbin;
+  P.segzbin = zt.segzbin;
+  P.bin_end = zt.bin_end;
   P.p1d_scale = static_cast<float>(rebin * params->dr / bins->n_fft);
-  P.cumz = ctx->d_cumz;
   P.tw = ctx->d_tw[tw_slot(bins->n_fft)];
   P.j_max = ctx->j_max;
   P.n_z = bins->n_z;
   P.n_k = bins->n_k;
-  P.z_lo = bins->z_lo;
-  P.dz = bins->dz;
-  P.dr = params->dr;
   P.partials = d_part;
   P.err = ctx->d_err;
   if ((rc = time_begin(ctx))) return rc;

@@ -713,35 +713,6 @@ __device__ __forceinline__ float reduce_scatter16(float (&v)[16], int lane) {
   return v[0] + __shfl_xor_sync(0xffffffffu, v[0], 16);
 }
 
-// Warp reduce-scatter of 32 values: lane l holds the warp total of v[l].
-__device__ __forceinline__ float reduce_scatter32(float (&v)[32], int lane) {
-#pragma unroll
-  for (int s = 16; s >= 1; s >>= 1) {
-#pragma unroll
-    for (int i = 0; i < s; ++i) {
-      const bool up = lane & s;
-      const float send = up ? v[i] : v[i + s];
-      const float keep = up ? v[i + s] : v[i];
-      v[i] = keep + __shfl_xor_sync(0xffffffffu, send, s);
-    }
-  }
-  return v[0];
-}
-
-// Pixel sums of one pixel: n, F, F^2, d, e, d^2, e^2, d e, F d, F e.
-__device__ __forceinline__ void add_pixel(float *a, float f, float d, float e) {
-  a[0] += 1.f;
-  a[1] += f;
-  a[2] = fmaf(f, f, a[2]);
-  a[3] += d;
-  a[4] += e;
-  a[5] = fmaf(d, d, a[5]);
-  a[6] = fmaf(e, e, a[6]);
-  a[7] = fmaf(d, e, a[7]);
-  a[8] = fmaf(f, d, a[8]);
-  a[9] = fmaf(f, e, a[9]);
-}
-
 // Pixel sums of one thread for one z bin, in the StatLayout order
 // n, F, F^2, d, e, d^2, e^2, d e, F d, F e; the (d, e) pairs run packed.
 struct PixelSums {
@@ -773,42 +744,6 @@ __device__ __forceinline__ void flush_bin_sums(const WarpAcc &W, int n_z, int zb
                  0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
   const float s = reduce_scatter16(v, lane);
   if (lane < MK_NSUM && zb >= 0 && zb < n_z) kahan_add(W.sums[zb * MK_NSUM + lane], s);
-}
-
-// Flush the thread sums of bins zf (a0) and zf + 1 (a1) into the warp
-// accumulators (warp-uniform call).
-__device__ __forceinline__ void flush_pixel_sums(const WarpAcc &W, int n_z, int zf, bool two, const float *a0,
-                                                 const float *a1, int lane) {
-  if (!two) {
-    float v[16];
-#pragma unroll
-    for (int i = 0; i < 16; ++i) v[i] = i < MK_NSUM ? a0[i] : 0.f;
-    const float s = reduce_scatter16(v, lane);
-    if (lane < MK_NSUM && zf >= 0 && zf < n_z) kahan_add(W.sums[zf * MK_NSUM + lane], s);
-  } else {
-    float v[32];
-#pragma unroll
-    for (int i = 0; i < 32; ++i) v[i] = i < MK_NSUM ? a0[i] : (i < 2 * MK_NSUM ? a1[i - MK_NSUM] : 0.f);
-    const float s = reduce_scatter32(v, lane);
-    const int b = zf + (lane >= MK_NSUM ? 1 : 0);
-    if (lane < 2 * MK_NSUM && b >= 0 && b < n_z) kahan_add(W.sums[b * MK_NSUM + lane % MK_NSUM], s);
-  }
-}
-
-// Pixel sums of bins beyond zf + 1 (only when a segment spans three or more
-// bins): the lanes that need it take turns adding into the warp accumulators.
-__device__ __forceinline__ void add_pixel_slow(const WarpAcc &W, int zb, float f, float d, float e) {
-  float a[MK_NSUM] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-  add_pixel(a, f, d, e);
-  const unsigned active = __activemask();
-  const int lane = threadIdx.x & 31;
-  for (int l = 0; l < 32; ++l) {
-    if (((active >> l) & 1u) && l == lane) {
-#pragma unroll
-      for (int i = 0; i < MK_NSUM; ++i) kahan_add(W.sums[zb * MK_NSUM + i], a[i]);
-    }
-    __syncwarp(active);
-  }
 }
 
 // Add the 4 mode powers of thread t (modes 4t+1..4t+4) to the P1D bins of z

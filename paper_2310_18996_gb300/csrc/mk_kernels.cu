@@ -218,12 +218,14 @@ __device__ __forceinline__ int16_t bin_of(double z, double z_lo, double dz, int 
 // of the segment of n_seg output pixels starting at J (n_z where they leave
 // the tables).
 __global__ void k_zbin(const double *__restrict__ zpix, const double *__restrict__ cumz, int32_t j_max,
-                       double z_lo, double dz, int n_z, int n_seg, int16_t *zbin, int16_t *segzbin) {
+                       double z_lo, double dz, int n_z, int n_seg, int R, int16_t *zbin, int16_t *segzbin) {
   const int j = blockIdx.x * blockDim.x + threadIdx.x;
   if (j >= j_max) return;
-  zbin[j] = bin_of(zpix[j], z_lo, dz, n_z);
-  segzbin[j] = (j + n_seg <= j_max) ? bin_of((cumz[j + n_seg] - cumz[j]) / n_seg, z_lo, dz, n_z)
-                                    : static_cast<int16_t>(n_z);
+  const int16_t out = static_cast<int16_t>(n_z);
+  zbin[j] = R == 1 ? bin_of(zpix[j], z_lo, dz, n_z)
+                   : (j + R <= j_max ? bin_of((cumz[j + R] - cumz[j]) / R, z_lo, dz, n_z) : out);
+  const int64_t span = static_cast<int64_t>(n_seg) * R;
+  segzbin[j] = j + span <= j_max ? bin_of((cumz[j + span] - cumz[j]) / static_cast<double>(span), z_lo, dz, n_z) : out;
 }
 
 // bin_end[k + 1] for k = -1 .. n_z: the first J whose z bin exceeds k (zbin is
@@ -443,8 +445,8 @@ cudaError_t launch_pixtab(const double *zpix, const float *gpix, int32_t j_max, 
 }
 
 cudaError_t launch_zbin(const double *zpix, const double *cumz, int32_t j_max, double z_lo, double dz, int n_z,
-                        int n_seg, int16_t *zbin, int16_t *segzbin, cudaStream_t st) {
-  k_zbin<<<blocks_for(j_max, 256), 256, 0, st>>>(zpix, cumz, j_max, z_lo, dz, n_z, n_seg, zbin, segzbin);
+                        int n_seg, int rebin, int16_t *zbin, int16_t *segzbin, cudaStream_t st) {
+  k_zbin<<<blocks_for(j_max, 256), 256, 0, st>>>(zpix, cumz, j_max, z_lo, dz, n_z, n_seg, rebin, zbin, segzbin);
   return cudaGetLastError();
 }
 

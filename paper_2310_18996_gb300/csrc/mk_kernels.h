@@ -20,7 +20,7 @@ cudaError_t launch_scan(const int64_t *a, const int64_t *b, int64_t n, int64_t *
 cudaError_t launch_pixtab(const double *zpix, const float *gpix, int32_t j_max, const NodeParams &nd,
                           float4 *pixtab, cudaStream_t st);
 cudaError_t launch_zbin(const double *zpix, const double *cumz, int32_t j_max, double z_lo, double dz, int n_z,
-                        int n_seg, int16_t *zbin, int16_t *segzbin, cudaStream_t st);
+                        int n_seg, int rebin, int16_t *zbin, int16_t *segzbin, cudaStream_t st);
 cudaError_t launch_pack(const float *d, const float *e, int64_t n, float *out, int sms, cudaStream_t st);
 cudaError_t launch_pack_tensor(const float *d, const float *e6, int lgn, float *out, int sms, cudaStream_t st);
 cudaError_t launch_pack_halo(const float *d, const float *e, int lgn, float *out, int sms, cudaStream_t st);

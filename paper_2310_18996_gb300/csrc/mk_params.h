@@ -129,14 +129,12 @@ struct StatParams {
   const float *delta, *eta;  // fine fields or NULL
   const float4 *pixtab;      // tuning pass: FGPA table; the flux is computed from delta, eta
   int32_t rebin;
-  const int16_t *zbin;
-  const int16_t *segzbin;
-  const int32_t *bin_end;  // first pixel J past each z bin (index zbin + 1), as in SkewerParams
-  const double *cumz;
+  const int16_t *zbin;     // per J: z bin of the output pixel (rebin fine pixels) starting there
+  const int16_t *segzbin;  // per J: z bin of the segment of N output pixels starting there
+  const int32_t *bin_end;  // first J past each z bin of zbin (index zbin + 1), as in SkewerParams
   const float2 *tw;
   int32_t j_max;
   int32_t n_z, n_k;
-  double z_lo, dz, dr;
   float p1d_scale;  // rebin dr / N
   double *partials;
   int *err;

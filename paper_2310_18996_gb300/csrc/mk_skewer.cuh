@@ -260,6 +260,14 @@ __global__ void __launch_bounds__(256, MINB) k_skewer(SkewerParams P) {
 }
 
 // =================================================================== statistics kernel
+// Statistics of output pixels of R = P.rebin fine pixels: of stored flux, or
+// (rebin 1, pixtab set) of the FGPA of stored fields.  The pixel sums stay in
+// registers across segments while the warp's pixels stay in one z bin and are
+// flushed at the bin's end, as in k_skewer; an output pixel's z bin comes from
+// the tables of mean z over R pixels (zbin, bin_end) for every R.  (With R > 1
+// the bin once came from an FP64 division per pixel, and this GPU's FP64 pipe
+// was the bound: flux and statistics of 1.4e8 fine pixels at R = 3 took 3.28 ms
+// then and 1.19 ms with the tables.)
 template <int N>
 __global__ void __launch_bounds__(256, 2) k_stats(StatParams P) {
   constexpr int T = N / 8;
@@ -284,8 +292,6 @@ __global__ void __launch_bounds__(256, 2) k_stats(StatParams P) {
   int64_t i = u < uend ? upper_index(P.segoff, P.n_sk, u) : 0;
   const int R = P.rebin;
   const int wlo0 = t & ~31;  // first team pixel of this warp
-  // R = 1: pixel sums in registers across segments while the warp's pixels
-  // stay in one z bin, flushed at the bin's end (as in k_skewer)
   PixelSums acc;
   acc.zero();
   int zc = -2;
@@ -305,60 +311,71 @@ __global__ void __launch_bounds__(256, 2) k_stats(StatParams P) {
     }
     const int64_t k0 = static_cast<int64_t>(s) * N;
     const int npx = static_cast<int>(min(static_cast<int64_t>(N), nout - k0));
-    auto zbin_of = [&](int64_t kk) -> int {
-      const int64_t J = sk.j_lo + kk * R;
-      if (R == 1) return __ldg(P.zbin + J);
-      const double fz = floor(((P.cumz[J + R] - P.cumz[J]) / R - P.z_lo) / P.dz);
-      return fz < 0.0 ? -1 : (fz >= P.n_z ? P.n_z : static_cast<int>(fz));
+    const int jb = sk.j_lo + static_cast<int>(k0 * R);
+    const int zs0 = __ldg(P.zbin + jb);
+    if (zs0 != zc) {
+      if (zc != -2) flush_bin_sums(W, P.n_z, zc, acc, lane);
+      acc.zero();
+      zc = zs0;
+    }
+    // segment pixel where bin zc ends
+    auto bin_stop = [&]() -> int {
+      const int d = __ldg(P.bin_end + zc + 1) - jb;
+      return R == 1 ? d : (d + R - 1) / R;
     };
-    if (R == 1) {
-      const int jb = sk.j_lo + static_cast<int>(k0);
-      const int zs = __ldg(P.zbin + jb);
-      if (zs != zc) {
-        if (zc != -2) flush_bin_sums(W, P.n_z, zc, acc, lane);
-        acc.zero();
-        zc = zs;
+    int pend = bin_stop();
+    // warp-uniform: this warp's pixels of the segment all lie before pend
+    const bool one_bin = min(T * 7 + wlo0 + 32, npx) <= pend;
+    // issue every load of the thread's 8 pixels before any use
+    float dv[8], ev[8], fv[8];
+    float4 tb[8];
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      const int p = t + T * q;
+      const bool ok = p < npx;
+      const int64_t kk = k0 + (ok ? p : 0);
+      dv[q] = ev[q] = 0.f;
+      if (R == 1 && ok && P.delta) {
+        dv[q] = __ldg(P.delta + sk.offset + kk);
+        ev[q] = __ldg(P.eta + sk.offset + kk);
       }
-      int pend = __ldg(P.bin_end + zc + 1) - jb;  // segment pixel where bin zc ends
-      // warp-uniform: this warp's pixels of the segment all lie before pend
-      const bool one_bin = min(T * 7 + wlo0 + 32, npx) <= pend;
-      if (npx == N && one_bin && P.pixtab) {
-        // tuning pass over a full segment inside one z bin: no bounds or bin checks
-        const float *dp = P.delta + sk.offset + k0 + t, *ep = P.eta + sk.offset + k0 + t;
-        const float4 *tp = P.pixtab + sk.j_lo + k0 + t;
-        float dv[8], ev[8];
-        float4 tb[8];
-#pragma unroll
-        for (int q = 0; q < 8; ++q) {
-          dv[q] = __ldg(dp + T * q);
-          ev[q] = __ldg(ep + T * q);
-          tb[q] = __ldg(tp + T * q);
-        }
-#pragma unroll
-        for (int q = 0; q < 8; ++q) {
-          const float f = fgpa(tb[q], dv[q], ev[q]);
-          acc.add_sums(f, make_float2(dv[q], ev[q]));
-          fb[t + T * q] = f;
-        }
-        acc.n += 8.f;
+      if (P.pixtab) {
+        tb[q] = __ldg(P.pixtab + sk.j_lo + kk);
+        fv[q] = 0.f;
       } else {
-      // streaming case: issue every load of the thread's 8 pixels before any use
-      float dv[8], ev[8], fv[8];
-      float4 tb[8];
+        fv[q] = ok ? __ldg(P.flux + o + kk) : 0.f;
+      }
+    }
+    if (R > 1 && P.delta) {  // the mean of R fine pixels; fine pixel r of all 8 at a time
+      const float *dp = P.delta + sk.offset + k0 * R, *ep = P.eta + sk.offset + k0 * R;
+#pragma unroll 2
+      for (int r = 0; r < R; ++r) {
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+          const int p = t + T * q;
+          if (p < npx) {
+            dv[q] += __ldg(dp + p * R + r);
+            ev[q] += __ldg(ep + p * R + r);
+          }
+        }
+      }
+      const float fr = static_cast<float>(R);
 #pragma unroll
       for (int q = 0; q < 8; ++q) {
-        const int p = t + T * q;
-        const bool ok = p < npx;
-        const int64_t kk = k0 + (ok ? p : 0);
-        dv[q] = (ok && P.delta) ? __ldg(P.delta + sk.offset + kk) : 0.f;
-        ev[q] = (ok && P.delta) ? __ldg(P.eta + sk.offset + kk) : 0.f;
-        if (P.pixtab) {
-          tb[q] = __ldg(P.pixtab + sk.j_lo + kk);
-          fv[q] = 0.f;
-        } else {
-          fv[q] = ok ? __ldg(P.flux + o + kk) : 0.f;
-        }
+        dv[q] /= fr;
+        ev[q] /= fr;
       }
+    }
+    if (npx == N && one_bin) {
+      // a full segment inside one z bin: no bounds or bin checks
+#pragma unroll
+      for (int q = 0; q < 8; ++q) {
+        const float f = P.pixtab ? fgpa(tb[q], dv[q], ev[q]) : fv[q];
+        acc.add_sums(f, make_float2(dv[q], ev[q]));
+        fb[t + T * q] = f;
+      }
+      acc.n += 8.f;
+    } else {
 #pragma unroll
       for (int q = 0; q < 8; ++q) {
         const int p = t + T * q;
@@ -379,54 +396,15 @@ __global__ void __launch_bounds__(256, 2) k_stats(StatParams P) {
             flush_bin_sums(W, P.n_z, zc, acc, lane);
             acc.zero();
             ++zc;
-            pend = __ldg(P.bin_end + zc + 1) - jb;
+            pend = bin_stop();
           }
           if (todo) acc.add(f, x);
         }
         fb[p] = f;
       }
-      }
-    } else {
-      const int zf = zbin_of(k0), zl = zbin_of(k0 + npx - 1);
-      float a0[MK_NSUM], a1[MK_NSUM];
-#pragma unroll
-      for (int q = 0; q < MK_NSUM; ++q) a0[q] = a1[q] = 0.f;
-#pragma unroll 2
-      for (int q = 0; q < 8; ++q) {
-        const int p = t + T * q;
-        float f = 0.f;
-        if (p < npx) {
-          const int64_t kk = k0 + p;
-          float ds = 0.f, es = 0.f;
-          if (P.delta) {
-            for (int r = 0; r < R; ++r) {
-              ds += P.delta[sk.offset + kk * R + r];
-              es += P.eta[sk.offset + kk * R + r];
-            }
-            ds /= static_cast<float>(R);
-            es /= static_cast<float>(R);
-          }
-          f = P.flux[o + kk];
-          const int zb = zbin_of(kk);
-          if (zb == zf) add_pixel(a0, f, ds, es);
-          else if (zb == zf + 1) add_pixel(a1, f, ds, es);
-          else if (zb >= 0 && zb < P.n_z) add_pixel_slow(W, zb, f, ds, es);
-        }
-        fb[p] = f;
-      }
-      flush_pixel_sums(W, P.n_z, zf, zl > zf, a0, a1, lane);
     }
     if (npx == N) {
-      int zs;
-      if (R == 1) {
-        zs = __ldg(P.segzbin + sk.j_lo + k0);
-      } else {
-        const int64_t J0 = sk.j_lo + k0 * R;
-        const double zm =
-            (P.cumz[J0 + static_cast<int64_t>(N) * R] - P.cumz[J0]) / (static_cast<double>(N) * R);
-        const double fz = floor((zm - P.z_lo) / P.dz);
-        zs = fz < 0.0 ? -1 : (fz >= P.n_z ? P.n_z : static_cast<int>(fz));
-      }
+      const int zs = __ldg(P.segzbin + jb);
       if (zs >= 0 && zs < P.n_z) {
         forward_packed_fft<N>(buf, tws, t, team);
         float pk[4];
@@ -437,7 +415,7 @@ __global__ void __launch_bounds__(256, 2) k_stats(StatParams P) {
     }
     team_sync<T>(team);
   }
-  if (R == 1 && zc != -2) flush_bin_sums(W, P.n_z, zc, acc, lane);
+  if (zc != -2) flush_bin_sums(W, P.n_z, zc, acc, lane);
   flush_warp_partials(smem, nwarps, wbytes, P.n_z, P.n_k, P.partials);
 }
 
