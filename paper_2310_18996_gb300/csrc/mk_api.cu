@@ -21,6 +21,7 @@ namespace {
 constexpr double kCH = 2997.92458;  // c/H0 [Mpc/h]
 constexpr double kZMax = 12.0;      // redshift range of the tables
 constexpr double kDcStep = 1.0 / 512.0;
+constexpr int kPixPad = 2048;    // entries past the FGPA table that masked lanes of a last segment may read
 constexpr double kZrStep = 1.0;  // Mpc/h, spacing of the z(r) starting table
 
 // ------------------------------------------------------------------ host cosmology
@@ -304,8 +305,9 @@ int ensure_pixel_tables(mk_ctx *ctx, double dr) {
   if (cudaMalloc(&ctx->d_zpix, sizeof(double) * jmax) != cudaSuccess ||
       cudaMalloc(&ctx->d_cumz, sizeof(double) * (jmax + 1)) != cudaSuccess ||
       cudaMalloc(&ctx->d_gpix, sizeof(float) * jmax) != cudaSuccess ||
-      cudaMalloc(&ctx->d_pixtab, sizeof(float4) * jmax) != cudaSuccess)
+      cudaMalloc(&ctx->d_pixtab, sizeof(float4) * (jmax + kPixPad)) != cudaSuccess)
     return fail(ctx, MK_ENOMEM, "pixel tables");
+  CK(cudaMemset(ctx->d_pixtab + jmax, 0, sizeof(float4) * kPixPad));
   for (auto &z : ctx->zt)
     if (cudaMalloc(&z.zbin, sizeof(int16_t) * jmax) != cudaSuccess ||
         cudaMalloc(&z.segzbin, sizeof(int16_t) * jmax) != cudaSuccess)
@@ -504,23 +506,29 @@ int time_end(mk_ctx *ctx) {
 // (at most ctx->grid_cap CTAs when a cap is set)
 int capped(mk_ctx *ctx, int grid) { return ctx->grid_cap > 0 && grid > ctx->grid_cap ? ctx->grid_cap : grid; }
 
-int skewer_grid(mk_ctx *ctx, int n_fft, int variant, int lgn, LaunchCfg cfg, const mk_stat_bins *bins) {
-  return capped(ctx, ctx->sms * skewer_blocks_per_sm(n_fft, variant, lgn, cfg.minb, cfg.threads,
+int skewer_grid(mk_ctx *ctx, int n_fft, int variant, int cap, LaunchCfg cfg, const mk_stat_bins *bins) {
+  return capped(ctx, ctx->sms * skewer_blocks_per_sm(n_fft, variant, cap, cfg.minb, cfg.threads,
                                                      bins ? bins->n_z : 0, bins ? bins->n_k : 0, bins != nullptr));
 }
 
 // default launch: 256-thread CTAs with the register budget of three per SM
 // (85 registers; measured fastest on GB300 for N = 256)
-LaunchCfg default_cfg(int n_fft) {
-  (void)n_fft;
-  return LaunchCfg{256, 3};
-}
+LaunchCfg default_cfg() { return LaunchCfg{256, 3}; }
 
 // kernel variant: the box layout, plus kGauss7Variant for the Gaussian kernel,
-// plus kPsNodesVariant for P_s tables at several redshifts
+// plus kPsNodesVariant for P_s tables at several redshifts, plus
+// kPixelGatherVariant where pixels are too long for the cells
 int kernel_variant(const mk_box *box, const mk_skewer_params *p) {
   return box->desc.layout | (p->interp == MK_INTERP_GAUSS7 ? kGauss7Variant : 0) |
-         (p->p_s_nodes >= 2 ? kPsNodesVariant : 0);
+         (p->p_s_nodes >= 2 ? kPsNodesVariant : 0) |
+         (p->interp == MK_INTERP_TRILINEAR && !use_cells(p->dr, box->desc.cell) ? kPixelGatherVariant : 0);
+}
+
+// cells the sight line of a pair of segments may cross (0: the kernel gathers per pixel)
+int run_cells(const mk_box *box, const mk_skewer_params *p) {
+  return p->interp == MK_INTERP_TRILINEAR && use_cells(p->dr, box->desc.cell)
+             ? cell_capacity(p->n_fft, p->dr / box->desc.cell)
+             : 0;
 }
 
 int check_interp(mk_ctx *ctx, const mk_box *box, const mk_skewer_params *p) {
@@ -552,8 +560,7 @@ GeomParams geom_params(mk_ctx *ctx, const mk_box *box, const mk_skewer_params *p
   for (int d = 0; d < 3; ++d) G.origin[d] = box->desc.origin[d];
   G.cell = box->desc.cell;
   G.j_max = ctx->j_max;
-  G.n_fft = p->n_fft;
-  G.rebin = 0;
+  G.unit_px = 2 * p->n_fft;
   return G;
 }
 
@@ -579,9 +586,9 @@ SkewerParams skewer_params(mk_ctx *ctx, const mk_box *box, const mk_skewer *d_sk
   S.box_d = box->d;
   S.box_e = box->e;
   S.lgn = box->lgn;
+  S.cell_cap = run_cells(box, p);
   S.pixtab = ctx->d_pixtab;
   S.zbin = ctx->zt[0].zbin;
-  S.cumz = ctx->d_cumz;
   S.amp = ctx->d_amp;
   S.ps_nodes = ctx->ps_nodes;
   for (int k = 0; k < MK_MAX_NODES; ++k) S.ps_z[k] = ctx->ps_z[k];
@@ -592,7 +599,6 @@ SkewerParams skewer_params(mk_ctx *ctx, const mk_box *box, const mk_skewer *d_sk
   S.segzbin = ctx->zt[0].segzbin;
   S.bin_end = ctx->zt[0].bin_end;
   S.err = ctx->d_err;
-  S.dr = p->dr;
   S.p1d_scale = static_cast<float>(p->dr / p->n_fft);
   return S;
 }
@@ -819,9 +825,9 @@ int mk_make_skewers(mk_ctx *ctx, const mk_box *box, const mk_qso *d_qso, int64_t
   S.flux_out = nullptr;
   S.capacity = capacity_px;
   S.do_stats = 0;
-  const LaunchCfg cfg = default_cfg(params->n_fft);
   const int variant = kernel_variant(box, params);
-  const int grid = skewer_grid(ctx, params->n_fft, variant, box->lgn, cfg, nullptr);
+  const LaunchCfg cfg = default_cfg();
+  const int grid = skewer_grid(ctx, params->n_fft, variant, S.cell_cap, cfg, nullptr);
   if ((rc = time_begin(ctx))) return rc;
   CK(launch_skewer(S, params->n_fft, variant, cfg.minb, grid, cfg.threads, ctx->stream));
   return time_end(ctx);
@@ -973,7 +979,7 @@ int mk_run(mk_ctx *ctx, const mk_box *box, const mk_qso *d_qso, int64_t n_qso, c
   // the launch shape: tuned, or tune now, or the default
   const int variant = kernel_variant(box, params);
   const uint64_t key = tune_key(params->n_fft, variant, box->lgn, flags);
-  LaunchCfg cfg = default_cfg(params->n_fft);
+  LaunchCfg cfg = default_cfg();
   auto it = ctx->tuned.find(key);
   if (it != ctx->tuned.end()) cfg = it->second;
 
@@ -987,8 +993,6 @@ int mk_run(mk_ctx *ctx, const mk_box *box, const mk_qso *d_qso, int64_t n_qso, c
   if (stats) {
     S.n_z = bins->n_z;
     S.n_k = bins->n_k;
-    S.z_lo = bins->z_lo;
-    S.dz = bins->dz;
   }
 
   // enqueue geometry, the fused kernel and (with statistics) their readback
@@ -1017,7 +1021,7 @@ int mk_run(mk_ctx *ctx, const mk_box *box, const mk_qso *d_qso, int64_t n_qso, c
     float best = 1e30f;
     for (const LaunchCfg &c : cand) {
       if (c.threads < params->n_fft / 8) continue;  // a team must fit in a CTA
-      const int grid = skewer_grid(ctx, params->n_fft, variant, box->lgn, c, stats ? bins : nullptr);
+      const int grid = skewer_grid(ctx, params->n_fft, variant, S.cell_cap, c, stats ? bins : nullptr);
       if ((rc = ensure_partials(grid))) break;
       if ((rc = enqueue_geometry(ctx, G, d_qso, n_qso, d_sk, d_offsets))) break;
       S.partials = ctx->d_partials;
@@ -1041,7 +1045,7 @@ int mk_run(mk_ctx *ctx, const mk_box *box, const mk_qso *d_qso, int64_t n_qso, c
     ctx->tuned[key] = cfg;
   }
 
-  const int grid = skewer_grid(ctx, params->n_fft, variant, box->lgn, cfg, stats ? bins : nullptr);
+  const int grid = skewer_grid(ctx, params->n_fft, variant, S.cell_cap, cfg, stats ? bins : nullptr);
   if ((rc = ensure_partials(grid))) return rc;
 
   if (flags & MK_GRAPH) {
@@ -1154,11 +1158,11 @@ int mk_run_host(mk_ctx *ctx, const mk_box *box, const mk_qso *h_qso, int64_t n_q
     if ((rc = grow(ctx, &ctx->d_stage[b], &ctx->stage_cap[b], sizeof(float) * static_cast<size_t>(maxc)))) return rc;
 
   const uint32_t kflags = MK_STORE_FLUX | (stats ? MK_STATS : 0u);
-  LaunchCfg cfg = default_cfg(params->n_fft);
   const int variant = kernel_variant(box, params);
+  LaunchCfg cfg = default_cfg();
   auto it = ctx->tuned.find(tune_key(params->n_fft, variant, box->lgn, kflags));
   if (it != ctx->tuned.end()) cfg = it->second;
-  const int grid = skewer_grid(ctx, params->n_fft, variant, box->lgn, cfg, stats ? bins : nullptr);
+  const int grid = skewer_grid(ctx, params->n_fft, variant, run_cells(box, params), cfg, stats ? bins : nullptr);
   const StatLayout L{stats ? bins->n_z : 0, stats ? bins->n_k : 0};
   if (stats && (rc = grow(ctx, reinterpret_cast<void **>(&ctx->d_partials), &ctx->partials_cap,
                           sizeof(double) * static_cast<size_t>(grid) * K * L.size())))
@@ -1168,8 +1172,6 @@ int mk_run_host(mk_ctx *ctx, const mk_box *box, const mk_qso *h_qso, int64_t n_q
   if (stats) {
     S.n_z = bins->n_z;
     S.n_k = bins->n_k;
-    S.z_lo = bins->z_lo;
-    S.dz = bins->dz;
   }
 
   // slices: compute on s0 into staging buffer k % 2, copy out on the copy
@@ -1213,7 +1215,7 @@ int mk_launch_config(mk_ctx *ctx, int32_t n_fft, int32_t layout, int32_t big_box
                      int32_t *threads, int32_t *occupancy) {
   if (!ctx || !threads || !occupancy) return MK_EINVAL;
   if (!skewer_fft(n_fft)) return fail(ctx, MK_EINVAL, "bad n_fft");
-  LaunchCfg c = default_cfg(n_fft);
+  LaunchCfg c = default_cfg();
   auto it = ctx->tuned.find(tune_key(n_fft, layout, big_box ? 11 : 10, flags));
   if (it != ctx->tuned.end()) c = it->second;
   *threads = c.threads;

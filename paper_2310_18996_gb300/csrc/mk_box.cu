@@ -184,7 +184,8 @@ __global__ void __launch_bounds__(BoxSmem<N2, REG>::THREADS, 2) k_box_pass(BoxPa
         const uint64_t q = static_cast<uint64_t>(v0 + i) >> 2;
         const u32x4 w = philox4x32_10(u32x4{static_cast<uint32_t>(q), static_cast<uint32_t>(q >> 32), 0u, 0u},
                                       P.key0, P.key1);
-        const float r0 = sqrt_pos(2.0f * neg_log_uniform(w.x)), r1 = sqrt_pos(2.0f * neg_log_uniform(w.z));
+        const float2 nl = neg_log_uniform2(w.x, w.z);
+        const float r0 = sqrt_pos(2.0f * nl.x), r1 = sqrt_pos(2.0f * nl.y);
         const float2 p0 = unit_phase(w.y), p1 = unit_phase(w.w);
         const int c = i / M, e = i % M;  // 4 | M: the 4 voxels share a line
         float2 *b = lines + c * LS + e;

@@ -8,8 +8,6 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
-#include <type_traits>
-
 #include "mk_params.h"
 
 namespace mk {
@@ -41,30 +39,6 @@ __device__ __forceinline__ float lg2_approx(float x) {
   float y;
   asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
   return y;
-}
-
-// -ln(u) for u = (x + 1/2) 2^-32, branch-free and accurate in relative terms
-// over the whole range.  Below 1/2 the SFU log2 is accurate to ~2^-22
-// relative (|log2 u| >= 1).  Above, u = 1 - d with d = (~x + 1/2) 2^-32 known
-// exactly, and -ln(1 - d) = 2 atanh(s), s = d/(2 - d) <= 1/3, summed from the
-// Gregory series 2 (s + s^3/3 + ... + s^17/17) (truncation < 1e-10).
-__device__ __forceinline__ float neg_log_uniform(uint32_t x) {
-  const float u = (__uint2float_rn(x) + 0.5f) * 0x1p-32f;
-  const float lo = -0.69314718055994531f * lg2_approx(u);
-  const float d = (__uint2float_rn(~x) + 0.5f) * 0x1p-32f;
-  const float s = __fdividef(d, 2.0f - d);
-  const float s2 = s * s;
-  float p = 1.0f / 17.0f;
-  p = fmaf(p, s2, 1.0f / 15.0f);
-  p = fmaf(p, s2, 1.0f / 13.0f);
-  p = fmaf(p, s2, 1.0f / 11.0f);
-  p = fmaf(p, s2, 1.0f / 9.0f);
-  p = fmaf(p, s2, 1.0f / 7.0f);
-  p = fmaf(p, s2, 1.0f / 5.0f);
-  p = fmaf(p, s2, 1.0f / 3.0f);
-  p = fmaf(p, s2, 1.0f);
-  const float hi = 2.0f * s * p;
-  return (x & 0x80000000u) ? hi : lo;
 }
 
 // (cos, sin)(2 pi u), u = (x + 1/2) 2^-32: the angle is taken in (-pi, pi)
@@ -122,6 +96,31 @@ __device__ __forceinline__ float2 f2fma(float2 a, float2 b, float2 c) {
 // a + t (b - a) per half, t the same for both: the scalar lerp's rounding
 __device__ __forceinline__ float2 f2lerp(float2 a, float2 b, float t) {
   return f2fma(make_float2(t, t), f2sub(b, a), a);
+}
+
+// ------------------------------------------------------------------ normals from Philox words
+// -ln(u) for u = (x + 1/2) 2^-32 of two words, branch-free and accurate in
+// relative terms over the whole range.  Below 1/2 the SFU log2 is accurate to
+// ~2^-22 relative (|log2 u| >= 1).  Above, u = 1 - d with d = (~x + 1/2) 2^-32
+// known exactly, and -ln(1 - d) = 2 atanh(s), s = d/(2 - d) <= 1/3, with
+// atanh(s)/s a polynomial in s^2 of degree 5 interpolated at the Chebyshev
+// points of [0, 1/9] (relative error 1e-9).  The two words run as packed pairs:
+// the polynomial once for both.
+__device__ __forceinline__ float2 neg_log_uniform2(uint32_t x0, uint32_t x1) {
+  const float2 half = make_float2(0.5f, 0.5f), scale = make_float2(0x1p-32f, 0x1p-32f);
+  const float2 u = f2mul(f2add(make_float2(__uint2float_rn(x0), __uint2float_rn(x1)), half), scale);
+  const float2 d = f2mul(f2add(make_float2(__uint2float_rn(~x0), __uint2float_rn(~x1)), half), scale);
+  const float2 s = make_float2(__fdividef(d.x, 2.0f - d.x), __fdividef(d.y, 2.0f - d.y));
+  const float2 s2 = f2mul(s, s);
+  float2 p = make_float2(0.12196954f, 0.12196954f);
+  p = f2fma(p, s2, make_float2(0.10699280f, 0.10699280f));
+  p = f2fma(p, s2, make_float2(0.14310104f, 0.14310104f));
+  p = f2fma(p, s2, make_float2(0.19999355f, 0.19999355f));
+  p = f2fma(p, s2, make_float2(0.33333340f, 0.33333340f));
+  p = f2fma(p, s2, make_float2(1.0f, 1.0f));
+  const float2 hi = f2mul(f2add(s, s), p);
+  const float lo0 = -0.69314718055994531f * lg2_approx(u.x), lo1 = -0.69314718055994531f * lg2_approx(u.y);
+  return make_float2((x0 & 0x80000000u) ? hi.x : lo0, (x1 & 0x80000000u) ? hi.y : lo1);
 }
 
 // ------------------------------------------------------------------ team barrier
@@ -318,32 +317,6 @@ __device__ __forceinline__ void fft_finish256(float2 *buf, float2 (&v)[4], const
   __syncwarp();
 }
 
-// Inverse real FFT of the Hermitian modes Y_0..Y_M held in buf (already
-// scaled by 1/N); on return the float view holds the N real outputs at plain
-// indices (pixel p at float p).
-template <int N>
-__device__ __forceinline__ void inverse_real_fft(float2 *buf, const float2 *tws, int t, int team) {
-  constexpr int T = Fft<N>::T;
-  constexpr int M = Fft<N>::M;
-  float2 v[4];
-  // N = 256: k = t + 32 r at lay_a(t) + 34 r, M - k at lay_a(32 - t) + 34 (3 - r)
-  const int ka = N == 256 ? lay_a(t) : 0, kb = N == 256 ? lay_a(32 - t) : 0;
-#pragma unroll
-  for (int r = 0; r < 4; ++r) {
-    const int k = t + r * T;
-    const float2 yk = buf[N == 256 ? ka + 34 * r : sw(k)];
-    const float2 ym = cconj(buf[N == 256 ? kb + 34 * (3 - r) : sw(M - k)]);
-    // Z_k = (Y_k + conj Y_{M-k}) + i (Y_k - conj Y_{M-k}) e^{+2 pi i k/N}
-    v[r] = cadd(cadd(yk, ym), cmul_i<1>(cmul(csub(yk, ym), cconj(tws[(TwTab<N>::U + r) * T + t]))));
-  }
-  dft4<1>(v[0], v[1], v[2], v[3]);
-  if constexpr (N == 256) {
-    fft_finish256<1, true>(buf, v, tws, t);
-  } else {
-    fft_finish<N, 1, true>(buf, v, tws, t, team);
-  }
-}
-
 // Forward complex FFT of the N reals in the float view of buf (plain
 // indices, pixel p at float p); on return buf holds Z_0..Z_{M-1} through the
 // swizzle.
@@ -387,43 +360,6 @@ __device__ __forceinline__ void power_of_modes(const float2 *buf, const float2 *
   }
 }
 
-// ------------------------------------------------------------------ small-scale modes
-// Y_m = X_m / N for m = 0..M into buf (Philox words -> Box-Muller):
-// X_m = A_m sqrt(-ln u1) e^{2 pi i u2} (= A (e1 + i e2)/sqrt 2), X_M = A e1.
-// Counter c serves modes 2c (words 0, 1) and 2c + 1 (words 2, 3); the words
-// of counter 0 that mode 0 (X_0 = 0) would use serve the Nyquist mode M.
-// ZNODES: amp and amp_hi hold (A_m / N)^2 at two z nodes, mixed with weight
-// w_hi; otherwise amp holds A_m / N and amp_hi is unused.
-template <int N, bool ZNODES>
-__device__ __forceinline__ void small_scale_modes(float2 *buf, const float *__restrict__ amp,
-                                                  const float *__restrict__ amp_hi, float w_hi, uint32_t seg,
-                                                  uint64_t id, uint32_t seed, int t) {
-  constexpr int T = Fft<N>::T;
-  constexpr int M = Fft<N>::M;
-  const uint32_t id_lo = static_cast<uint32_t>(id), id_hi = static_cast<uint32_t>(id >> 32);
-#pragma unroll
-  for (int q = 0; q < 2; ++q) {
-    const uint32_t c = t + q * T;  // modes 2c, 2c+1 (< M)
-    const u32x4 w = philox4x32_10(u32x4{c, seg, id_hi, 0u}, seed, id_lo);
-    const bool nyq = (c == 0);
-    const int m0 = nyq ? M : 2 * c, m1 = 2 * c + 1;
-    float s0 = __ldg(amp + m0), s1 = __ldg(amp + m1);
-    if (ZNODES) {  // interpolate P_s between the nodes, then the root
-      s0 = sqrtf(fmaf(w_hi, __ldg(amp_hi + m0) - s0, s0));
-      s1 = sqrtf(fmaf(w_hi, __ldg(amp_hi + m1) - s1, s1));
-    }
-    const float2 p0 = unit_phase(w.y), p1 = unit_phase(w.w);
-    const float a0 = s0 * sqrt_pos((nyq ? 2.0f : 1.0f) * neg_log_uniform(w.x));
-    const float a1 = s1 * sqrt_pos(neg_log_uniform(w.z));
-    // N = 256 (layout LA): mode 2c + e, c = t + 32 q, at lay_a(2t) + e + 68 q
-    const int i0 = N != 256 ? sw(m0) : (nyq ? lay_a(M) : lay_a(2 * t) + 68 * q);
-    const int i1 = N != 256 ? sw(m1) : lay_a(2 * t) + 1 + 68 * q;
-    buf[i0] = make_float2(a0 * p0.x, nyq ? 0.f : a0 * p0.y);
-    buf[i1] = make_float2(a1 * p1.x, a1 * p1.y);
-  }
-  if (t == 0) buf[0] = make_float2(0.f, 0.f);  // sw(0) = lay_a(0) = 0
-}
-
 // ------------------------------------------------------------------ fixed-point gather
 // Positions are Q20.44 cell coordinates (minus 1/2, so that integer values
 // fall on cell centres).  The kernels add kRoundQ to a skewer's start so that
@@ -441,108 +377,6 @@ __device__ __forceinline__ float weight_of(int64_t p) {
 }
 
 __device__ __forceinline__ float lerpf(float a, float b, float t) { return fmaf(t, b - a, a); }
-
-// Trilinear (delta, eta) at fixed-point coordinate (px, py, pz).  BIG: box
-// with more than 2^30 cells (64-bit indices).
-//   MK_BOX_PLANAR / MK_BOX_INTERLEAVED: n^3 cells, periodic indices.
-//   MK_BOX_PADDED: (delta, eta) pairs on (n+1)^3 points whose last plane,
-//   row and column repeat index 0, so the 8 corners sit at fixed offsets
-//   from the base corner and no index wraps.
-//   MK_BOX_HALO: pairs on (n+6)^3 points, a periodic margin of 3 on every
-//   side; the same fixed offsets from base index (x+3, y+3, z+3).
-// FIXLGN > 0 (padded layout, 32-bit indices): the box side is 2^FIXLGN, so
-// the row and plane strides are constants and the eight loads take immediate
-// offsets from one pointer (placed mid-way between the two planes, so that
-// every offset stays within the immediate range).
-template <int LAYOUT, bool BIG, int FIXLGN = 0>
-__device__ __forceinline__ float2 gather(const float *__restrict__ d, const float *__restrict__ e, int lgn,
-                                         int64_t px, int64_t py, int64_t pz) {
-  const int mask = FIXLGN > 0 ? (1 << FIXLGN) - 1 : (1 << lgn) - 1;
-  const int x0 = cell_of(px, mask), y0 = cell_of(py, mask), z0 = cell_of(pz, mask);
-  const float tx = weight_of(px), ty = weight_of(py), tz = weight_of(pz);
-  using I = typename std::conditional<BIG, int64_t, int32_t>::type;
-  float2 v[8];
-  if constexpr (FIXLGN > 0) {
-    static_assert(LAYOUT == MK_BOX_PADDED && !BIG, "fixed strides serve the padded layout with 32-bit indices");
-    constexpr int n1 = (1 << FIXLGN) + 1, plane = n1 * n1, half = plane / 2;
-    const float2 *mid = reinterpret_cast<const float2 *>(d) + (z0 * plane + y0 * n1 + x0 + half);
-    const float2 *a00 = mid - half, *a01 = a00 + n1;
-    const float2 *a10 = mid + (plane - half), *a11 = a10 + n1;
-    v[0] = __ldg(a00); v[1] = __ldg(a00 + 1);
-    v[2] = __ldg(a01); v[3] = __ldg(a01 + 1);
-    v[4] = __ldg(a10); v[5] = __ldg(a10 + 1);
-    v[6] = __ldg(a11); v[7] = __ldg(a11 + 1);
-  } else if constexpr (LAYOUT == MK_BOX_PADDED || LAYOUT == MK_BOX_HALO) {
-    constexpr int h = LAYOUT == MK_BOX_HALO ? 3 : 0;
-    const I n1 = mask + 1 + (LAYOUT == MK_BOX_HALO ? 6 : 1);
-    const float2 *a00 =
-        reinterpret_cast<const float2 *>(d) + ((static_cast<I>(z0 + h) * n1 + (y0 + h)) * n1 + (x0 + h));
-    const float2 *a01 = a00 + n1, *a10 = a00 + n1 * n1;
-    const float2 *a11 = a10 + n1;
-    v[0] = __ldg(a00); v[1] = __ldg(a00 + 1);
-    v[2] = __ldg(a01); v[3] = __ldg(a01 + 1);
-    v[4] = __ldg(a10); v[5] = __ldg(a10 + 1);
-    v[6] = __ldg(a11); v[7] = __ldg(a11 + 1);
-  } else {
-    const int x1 = (x0 + 1) & mask, y1 = (y0 + 1) & mask, z1 = (z0 + 1) & mask;
-    using U = typename std::conditional<BIG, size_t, uint32_t>::type;
-    const U zz0 = static_cast<U>(z0) << (2 * lgn), zz1 = static_cast<U>(z1) << (2 * lgn);
-    const U yy0 = static_cast<U>(y0) << lgn, yy1 = static_cast<U>(y1) << lgn;
-    const U r00 = zz0 | yy0, r10 = zz0 | yy1, r01 = zz1 | yy0, r11 = zz1 | yy1;
-    if constexpr (LAYOUT == MK_BOX_INTERLEAVED) {
-      const float2 *b = reinterpret_cast<const float2 *>(d);
-      v[0] = __ldg(b + (r00 | x0)); v[1] = __ldg(b + (r00 | x1));
-      v[2] = __ldg(b + (r10 | x0)); v[3] = __ldg(b + (r10 | x1));
-      v[4] = __ldg(b + (r01 | x0)); v[5] = __ldg(b + (r01 | x1));
-      v[6] = __ldg(b + (r11 | x0)); v[7] = __ldg(b + (r11 | x1));
-    } else {
-      const U idx[8] = {r00 | x0, r00 | x1, r10 | x0, r10 | x1, r01 | x0, r01 | x1, r11 | x0, r11 | x1};
-#pragma unroll
-      for (int k = 0; k < 8; ++k) v[k] = make_float2(__ldg(d + idx[k]), __ldg(e + idx[k]));
-    }
-  }
-  // x, then y, then z; delta and eta as one packed pair
-  const float2 c0 = f2lerp(v[0], v[1], tx), c1 = f2lerp(v[2], v[3], tx);
-  const float2 c2 = f2lerp(v[4], v[5], tx), c3 = f2lerp(v[6], v[7], tx);
-  return f2lerp(f2lerp(c0, c1, ty), f2lerp(c2, c3, ty), tz);
-}
-
-// Trilinear (delta, eta_par) from an MK_BOX_TENSOR box: all seven fields are
-// interpolated (x, then y, then z, on packed pairs) and the velocity-gradient
-// tensor is contracted with the sight line, eta_par = u_p u_q eta_pq (Eq. eta);
-// uu = {ux^2, uy^2, uz^2, 2 ux uy, 2 ux uz, 2 uy uz}.
-struct F7 {
-  float2 a, b, c;  // (delta, xx), (yy, zz), (xy, xz)
-  float d;         // yz
-};
-__device__ __forceinline__ F7 lerp7(const F7 &p, const F7 &q, float t) {
-  return F7{f2lerp(p.a, q.a, t), f2lerp(p.b, q.b, t), f2lerp(p.c, q.c, t), lerpf(p.d, q.d, t)};
-}
-// the two points (x0, x0 + 1) of a row, lerped in x
-__device__ __forceinline__ F7 tensor_row(const float4 *r, float tx) {
-  const float4 a0 = __ldg(r), b0 = __ldg(r + 1), a1 = __ldg(r + 2), b1 = __ldg(r + 3);
-  const F7 p{make_float2(a0.x, a0.y), make_float2(a0.z, a0.w), make_float2(b0.x, b0.y), b0.z};
-  const F7 q{make_float2(a1.x, a1.y), make_float2(a1.z, a1.w), make_float2(b1.x, b1.y), b1.z};
-  return lerp7(p, q, tx);
-}
-
-template <bool BIG>
-__device__ __forceinline__ float2 gather_tensor(const float *__restrict__ d, int lgn, int64_t px, int64_t py,
-                                                int64_t pz, const float (&uu)[6]) {
-  const int mask = (1 << lgn) - 1;
-  const int x0 = cell_of(px, mask), y0 = cell_of(py, mask), z0 = cell_of(pz, mask);
-  const float tx = weight_of(px), ty = weight_of(py), tz = weight_of(pz);
-  using I = typename std::conditional<BIG, int64_t, int32_t>::type;
-  const I n1 = mask + 2;
-  const float4 *b = reinterpret_cast<const float4 *>(d);
-  const I i00 = (static_cast<I>(z0) * n1 + y0) * n1 + x0;
-  const F7 c0 = tensor_row(b + 2 * i00, tx), c1 = tensor_row(b + 2 * (i00 + n1), tx);
-  const F7 c2 = tensor_row(b + 2 * (i00 + n1 * n1), tx), c3 = tensor_row(b + 2 * (i00 + n1 * n1 + n1), tx);
-  const F7 v = lerp7(lerp7(c0, c1, ty), lerp7(c2, c3, ty), tz);
-  const float eta = fmaf(uu[0], v.a.y, fmaf(uu[1], v.b.x, fmaf(uu[2], v.b.y,
-                    fmaf(uu[3], v.c.x, fmaf(uu[4], v.c.y, uu[5] * v.d)))));
-  return make_float2(v.a.x, eta);
-}
 
 // Normalised 1D weights of the Gaussian-kernel average (Sec. 2.3) along one
 // axis: voxels c - 3 .. c + 3 around the voxel c containing the point, whose
@@ -578,7 +412,6 @@ __device__ __forceinline__ void gauss7_weights(float f, float (&w)[7]) {
 // MK_BOX_HALO box, as three nested 1D contractions (the weights are
 // separable): per z plane, 7 x-rows of 7 pairs contracted with the x weights,
 // then with the y weights; the z weights come as a running product.
-template <bool BIG>
 __device__ __forceinline__ float2 gather_gauss7(const float *__restrict__ d, int lgn, int64_t px, int64_t py,
                                                 int64_t pz) {
   const int mask = (1 << lgn) - 1;
@@ -591,10 +424,9 @@ __device__ __forceinline__ float2 gather_gauss7(const float *__restrict__ d, int
   float qz, qiz, invz;
   gauss7_axis(weight_of(hz), qz, qiz, invz);
   float pz_run = qiz * qiz * qiz * invz;
-  using I = typename std::conditional<BIG, int64_t, int32_t>::type;
-  const I n6 = mask + 7;
+  const int64_t n6 = mask + 7;
   // voxel (c - 3) per axis sits at halo index c
-  const float2 *row = reinterpret_cast<const float2 *>(d) + ((static_cast<I>(cz) * n6 + cy) * n6 + cx);
+  const float2 *row = reinterpret_cast<const float2 *>(d) + ((cz * n6 + cy) * n6 + cx);
   float2 acc = make_float2(0.f, 0.f);
 #pragma unroll 1
   for (int k = 0; k < 7; ++k) {
@@ -618,44 +450,33 @@ __device__ __forceinline__ float2 gather_gauss7(const float *__restrict__ d, int
 // Prefetch into L2 the four voxel rows (y0|y1, z0|z1) that the trilinear
 // stencil at (px, py, pz) reads, for the paired layouts (each row's two
 // corners x0, x0 + 1 are adjacent).
-template <int LAYOUT, bool BIG>
+template <int LAYOUT>
 __device__ __forceinline__ void prefetch_stencil(const float *__restrict__ d, int lgn, int64_t px, int64_t py,
                                                  int64_t pz) {
   if constexpr (LAYOUT == MK_BOX_PLANAR) return;
-  if constexpr (LAYOUT == MK_BOX_TENSOR) {
-    const int mask = (1 << lgn) - 1;
-    const int x0 = cell_of(px, mask), y0 = cell_of(py, mask), z0 = cell_of(pz, mask);
-    using I = typename std::conditional<BIG, int64_t, int32_t>::type;
-    const I n1 = mask + 2;
-    const float4 *b = reinterpret_cast<const float4 *>(d);
-    const I i00 = (static_cast<I>(z0) * n1 + y0) * n1 + x0;
-    const I rows[4] = {i00, i00 + n1, i00 + n1 * n1, i00 + n1 * n1 + n1};
-#pragma unroll
-    for (int r = 0; r < 4; ++r) asm volatile("prefetch.global.L2 [%0];" ::"l"(b + 2 * rows[r]));
-    return;
-  }
   const int mask = (1 << lgn) - 1;
   const int x0 = cell_of(px, mask), y0 = cell_of(py, mask), z0 = cell_of(pz, mask);
-  using I = typename std::conditional<BIG, int64_t, int32_t>::type;
-  const float2 *b = reinterpret_cast<const float2 *>(d);
-  const float2 *a[4];
-  if constexpr (LAYOUT == MK_BOX_PADDED || LAYOUT == MK_BOX_HALO) {
+  constexpr int kRecord = LAYOUT == MK_BOX_TENSOR ? 32 : 8;  // bytes
+  int64_t row[4];
+  if constexpr (LAYOUT == MK_BOX_PADDED || LAYOUT == MK_BOX_HALO || LAYOUT == MK_BOX_TENSOR) {
     constexpr int h = LAYOUT == MK_BOX_HALO ? 3 : 0;
-    const I n1 = mask + 1 + (LAYOUT == MK_BOX_HALO ? 6 : 1);
-    a[0] = b + ((static_cast<I>(z0 + h) * n1 + (y0 + h)) * n1 + (x0 + h));
-    a[1] = a[0] + n1;
-    a[2] = a[0] + n1 * n1;
-    a[3] = a[2] + n1;
+    const int64_t n1 = mask + 1 + (LAYOUT == MK_BOX_HALO ? 6 : 1);
+    row[0] = ((z0 + h) * n1 + (y0 + h)) * n1 + (x0 + h);
+    row[1] = row[0] + n1;
+    row[2] = row[0] + n1 * n1;
+    row[3] = row[2] + n1;
   } else {
     const int y1 = (y0 + 1) & mask, z1 = (z0 + 1) & mask;
-    using U = typename std::conditional<BIG, size_t, uint32_t>::type;
-    a[0] = b + ((static_cast<U>(z0) << (2 * lgn)) | (static_cast<U>(y0) << lgn) | x0);
-    a[1] = b + ((static_cast<U>(z0) << (2 * lgn)) | (static_cast<U>(y1) << lgn) | x0);
-    a[2] = b + ((static_cast<U>(z1) << (2 * lgn)) | (static_cast<U>(y0) << lgn) | x0);
-    a[3] = b + ((static_cast<U>(z1) << (2 * lgn)) | (static_cast<U>(y1) << lgn) | x0);
+    const int64_t a = static_cast<int64_t>(z0) << (2 * lgn), b = static_cast<int64_t>(z1) << (2 * lgn);
+    const int64_t c = static_cast<int64_t>(y0) << lgn, e = static_cast<int64_t>(y1) << lgn;
+    row[0] = a | c | x0;
+    row[1] = a | e | x0;
+    row[2] = b | c | x0;
+    row[3] = b | e | x0;
   }
+  const char *base = reinterpret_cast<const char *>(d);
 #pragma unroll
-  for (int r = 0; r < 4; ++r) asm volatile("prefetch.global.L2 [%0];" ::"l"(a[r]));
+  for (int r = 0; r < 4; ++r) asm volatile("prefetch.global.L2 [%0];" ::"l"(base + kRecord * row[r]));
 }
 
 // ------------------------------------------------------------------ FGPA
@@ -697,22 +518,6 @@ __device__ __forceinline__ void kahan_add(float2 &acc, float x) {
   acc.x = t;
 }
 
-// Warp reduce-scatter of 16 values: afterwards lanes l and l + 16 hold the
-// warp total of v[l & 15].
-__device__ __forceinline__ float reduce_scatter16(float (&v)[16], int lane) {
-#pragma unroll
-  for (int s = 8; s >= 1; s >>= 1) {
-#pragma unroll
-    for (int i = 0; i < s; ++i) {
-      const bool up = lane & s;
-      const float send = up ? v[i] : v[i + s];
-      const float keep = up ? v[i + s] : v[i];
-      v[i] = keep + __shfl_xor_sync(0xffffffffu, send, s);
-    }
-  }
-  return v[0] + __shfl_xor_sync(0xffffffffu, v[0], 16);
-}
-
 // Pixel sums of one thread for one z bin, in the StatLayout order
 // n, F, F^2, d, e, d^2, e^2, d e, F d, F e; the (d, e) pairs run packed.
 struct PixelSums {
@@ -738,31 +543,48 @@ struct PixelSums {
 };
 
 // Add the warp's PixelSums of bin zb to the warp accumulators (warp-uniform
-// call; bins outside [0, n_z) are dropped).
+// call; bins outside [0, n_z) are dropped).  A rolled butterfly: it runs about
+// once a pair of segments, and its code (60 instructions; 260 for a
+// reduce-scatter of unrolled steps) shares the instruction cache with the
+// segment loop it interrupts.
 __device__ __forceinline__ void flush_bin_sums(const WarpAcc &W, int n_z, int zb, const PixelSums &a, int lane) {
-  float v[16] = {a.n, a.f, a.ff, a.m1.x, a.m1.y, a.m2.x, a.m2.y, a.de, a.fm.x, a.fm.y,
-                 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-  const float s = reduce_scatter16(v, lane);
+  float v[MK_NSUM] = {a.n, a.f, a.ff, a.m1.x, a.m1.y, a.m2.x, a.m2.y, a.de, a.fm.x, a.fm.y};
+#pragma unroll 1
+  for (int s = 16; s >= 1; s >>= 1) {
+#pragma unroll
+    for (int i = 0; i < MK_NSUM; ++i) v[i] += __shfl_xor_sync(0xffffffffu, v[i], s);
+  }
+  float s = v[0];
+#pragma unroll
+  for (int i = 1; i < MK_NSUM; ++i) s = lane == i ? v[i] : s;
   if (lane < MK_NSUM && zb >= 0 && zb < n_z) kahan_add(W.sums[zb * MK_NSUM + lane], s);
 }
 
+// P1D bins of a thread's 4 modes 4t+1 .. 4t+4 (m modes, n_k equal bins), worked
+// out once per kernel.
+struct P1dBins {
+  int per_bin, group, slot;  // modes per bin, threads of a warp that share a bin (0: several bins per thread), bin of mode 4t+1
+  bool writer;
+  __device__ __forceinline__ P1dBins(int m, int n_k, int t) {
+    per_bin = m / max(n_k, 1);
+    group = per_bin >= 4 ? min(per_bin / 4, 32) : 0;
+    slot = (4 * t) / max(per_bin, 1);
+    writer = group > 0 && (t & (group - 1)) == 0;
+  }
+};
+
 // Add the 4 mode powers of thread t (modes 4t+1..4t+4) to the P1D bins of z
 // bin zb (warp-uniform call).  Every bin slot of a warp has one writer.
-template <int N>
-__device__ __forceinline__ void accumulate_p1d(const WarpAcc &W, int n_k, const float (&pk)[4], float scale,
-                                               int zb, int t) {
-  constexpr int M = Fft<N>::M;
-  const int per_bin = M / n_k;
-  const int lane = t & 31;
-  if (per_bin >= 4) {
+__device__ __forceinline__ void accumulate_p1d(const WarpAcc &W, int n_k, const P1dBins &B, const float (&pk)[4],
+                                               float scale, int zb) {
+  float2 *row = W.p1d + zb * n_k;
+  if (B.group > 0) {
     float s = (pk[0] + pk[1]) + (pk[2] + pk[3]);
-    const int group = per_bin / 4;  // threads sharing a bin
-    const int g32 = group < 32 ? group : 32;
-    for (int o = 1; o < g32; o <<= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    if ((lane & (g32 - 1)) == 0) kahan_add(W.p1d[zb * n_k + (4 * t) / per_bin], s * scale);
+    for (int o = 1; o < B.group; o <<= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (B.writer) kahan_add(row[B.slot], s * scale);
   } else {
 #pragma unroll
-    for (int r = 0; r < 4; ++r) kahan_add(W.p1d[zb * n_k + ((4 * t + r) * n_k) / M], pk[r] * scale);
+    for (int r = 0; r < 4; ++r) kahan_add(row[B.slot + r / B.per_bin], pk[r] * scale);
   }
 }
 

@@ -90,8 +90,8 @@ __global__ void k_geometry(const mk_qso *__restrict__ q, int64_t nq, GeomParams 
     }
   }
   sk[i] = s;
-  cnt_px[i] = P.rebin > 0 ? s.n / P.rebin : s.n;
-  cnt_seg[i] = P.n_fft > 0 ? (s.n + P.n_fft - 1) / P.n_fft : 0;
+  cnt_px[i] = s.n;
+  cnt_seg[i] = (s.n + P.unit_px - 1) / P.unit_px;
 }
 
 // =================================================================== scan
@@ -513,12 +513,8 @@ cudaError_t launch_seg_counts(const int64_t *off, int64_t n, int n_fft, int64_t 
   }                                            \
   return FAIL;
 
-size_t skewer_smem_bytes(int n_fft, int threads, int n_z, int n_k, bool stats) {
-  MK_SWITCH(smem_bytes(threads, n_z, n_k, stats), 0)
-}
-
-int skewer_blocks_per_sm(int n_fft, int variant, int lgn, int minb, int threads, int n_z, int n_k, bool stats) {
-  MK_SWITCH(blocks_per_sm(variant, lgn, minb, threads, n_z, n_k, stats), 1)
+int skewer_blocks_per_sm(int n_fft, int variant, int cap, int minb, int threads, int n_z, int n_k, bool stats) {
+  MK_SWITCH(blocks_per_sm(variant, cap, minb, threads, n_z, n_k, stats), 1)
 }
 
 cudaError_t launch_skewer(const SkewerParams &P, int n_fft, int variant, int minb, int grid, int threads,

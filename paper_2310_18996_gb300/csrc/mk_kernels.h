@@ -9,6 +9,15 @@ namespace mk {
 
 constexpr int kGauss7Variant = 16;   // kernel variant bit of MK_INTERP_GAUSS7
 constexpr int kPsNodesVariant = 32;  // kernel variant bit of P_s tables at several redshifts
+constexpr int kPixelGatherVariant = 64;  // kernel variant bit of trilinear gathers per pixel (see use_cells)
+
+// Whether a trilinear run reads its box through the cells of the sight line
+// (plan_cells in mk_pair.cuh) or gathers pixel by pixel.  Up to dr/cell = 0.1
+// (the paper's is 0.091) a pair's cells fit three rounds of one cell per thread
+// and the shared memory of three CTAs per SM.  At 0.091 the fused kernel takes
+// 1.07 ms per 1.37e8 pixels through the cells and 1.46 ms gathering (N = 256;
+// 1.53 and 2.60 ms on a tensor box, 1.78 and 2.17 ms at N = 1024).
+inline bool use_cells(double dr, double cell) { return dr <= 0.1 * cell; }
 
 cudaError_t launch_geometry(const mk_qso *q, int64_t nq, const GeomParams &P, mk_skewer *sk, int64_t *cnt_px,
                             int64_t *cnt_seg, int *err, cudaStream_t st);
@@ -31,7 +40,7 @@ cudaError_t launch_pick(const int64_t *off, int64_t n, int k, int64_t *out, cuda
 cudaError_t launch_bin_end(const int16_t *zbin, int32_t j_max, int n_z, int32_t *bin_end, cudaStream_t st);
 cudaError_t launch_out_counts(const mk_skewer *sk, int64_t n, int rebin, int64_t *cnt, cudaStream_t st);
 cudaError_t launch_seg_counts(const int64_t *off, int64_t n, int n_fft, int64_t *cnt, cudaStream_t st);
-int skewer_blocks_per_sm(int n_fft, int variant, int lgn, int minb, int threads, int n_z, int n_k, bool stats);
+int skewer_blocks_per_sm(int n_fft, int variant, int cap, int minb, int threads, int n_z, int n_k, bool stats);
 // The tuning pass (FGPA table set, rebin 1, 16-byte aligned fields) runs the
 // staged kernel k_tune_stats; every other statistics pass runs k_stats.
 inline bool tune_kernel(const void *pixtab, const float *delta, const float *eta, int rebin) {
@@ -39,9 +48,9 @@ inline bool tune_kernel(const void *pixtab, const float *delta, const float *eta
          ((reinterpret_cast<uintptr_t>(delta) | reinterpret_cast<uintptr_t>(eta)) & 15) == 0;
 }
 int stats_blocks_per_sm(int n_fft, int threads, int n_z, int n_k, bool tune);
-size_t skewer_smem_bytes(int n_fft, int threads, int n_z, int n_k, bool stats);
 // variant: box layout, plus kGauss7Variant for the Gaussian-kernel interpolation,
-// plus kPsNodesVariant for z-dependent P_s (built for register budget 3 only);
+// plus kPsNodesVariant for z-dependent P_s (built for register budget 3 only),
+// plus kPixelGatherVariant (budget 3 only); cap: cells of a run (P.cell_cap);
 // minb: register budget of the instance, that of minb 256-thread CTAs per SM
 // (2, 3 or 4)
 cudaError_t launch_skewer(const SkewerParams &P, int n_fft, int variant, int minb, int grid, int threads,
@@ -51,8 +60,7 @@ cudaError_t launch_skewer(const SkewerParams &P, int n_fft, int variant, int min
 // per length (256, 512, 1024, 2048) in mk_skewer_<N>.cu.
 template <int N>
 struct SkewerUnit {
-  static size_t smem_bytes(int threads, int n_z, int n_k, bool stats);
-  static int blocks_per_sm(int variant, int lgn, int minb, int threads, int n_z, int n_k, bool stats);
+  static int blocks_per_sm(int variant, int cap, int minb, int threads, int n_z, int n_k, bool stats);
   static cudaError_t launch(const SkewerParams &P, int variant, int minb, int grid, int threads, cudaStream_t st);
   static int stats_blocks_per_sm(int threads, int n_z, int n_k, bool tune);
   static cudaError_t launch_stats(const StatParams &P, int grid, int threads, cudaStream_t st);

@@ -1,0 +1,487 @@
+// Building blocks of the kernels that work on a pair of segments: the N-point
+// complex FFT that carries two real segments, and the cells of a run of pixels.
+//
+// A team of T = N/8 threads owns the pair (2i, 2i + 1) of segments of N pixels
+// of one skewer; thread t holds pixels t + T r, r = 0..7, of both.
+#pragma once
+
+#include "mk_device.cuh"
+
+namespace mk {
+
+// ------------------------------------------------------------------ FFT plan
+// Radix-8 Stockham passes (sub-transform lengths 1, 8, 64) and one pass of
+// radix F.  Eight points a thread stay in registers between the exchanges, and
+// both ends of the transform sit at t + T r, the pixels of the thread: neither
+// end needs shared memory.  Two real segments as the real and imaginary parts
+// of one complex transform need no real-FFT untangling, and a radix-8 pass
+// halves the exchanges of the radix-4 passes on N/2 points that went before:
+// two for the pair at N = 256 instead of four for each segment.
+template <int N>
+struct PairFft {
+  static constexpr int T = N / 8;
+  static constexpr int P8 = N == 256 ? 2 : 3;
+  static constexpr int F = N == 256 ? 4 : (N == 512 ? 1 : (N == 1024 ? 2 : 4));
+  static_assert(N == 256 || N == 512 || N == 1024 || N == 2048, "unsupported N");
+  // complex slots of the exchange buffer (layout LB: 8 of padding per 64)
+  static constexpr int BUF = N + N / 8;
+  // twiddles (forward sign), shared by the CTA's teams: pass 1 (7 x 8 entries,
+  // e^{-2 pi i r j / 64}), pass 2 (7 x 64 entries, e^{-2 pi i r j / 512}, P8 = 3),
+  // last pass (slot (i, q), i < 8 / F, q = 1..F-1: e^{-2 pi i q (t + T i) / N}, T entries each)
+  static constexpr int TW1 = 0;
+  static constexpr int TW2 = 56;
+  static constexpr int TWF = P8 == 3 ? TW2 + 7 * 64 : TW2;
+  static constexpr int TWN = TWF + (8 / F) * (F - 1) * T;
+  static constexpr size_t TW_BYTES = sizeof(float2) * TWN;
+};
+
+// tab[k] = e^{-2 pi i k/N}, k < N (FP64-rounded table in global memory).
+// Called by every thread of the CTA; ends with a CTA barrier.
+template <int N>
+__device__ __forceinline__ void fill_pair_twiddles(float2 *tws, const float2 *__restrict__ tab) {
+  using P = PairFft<N>;
+  for (int i = threadIdx.x; i < P::TWN; i += blockDim.x) {
+    int k;
+    if (i < P::TW2) {
+      k = (i / 8 + 1) * (i % 8) * (N / 64);
+    } else if (i < P::TWF) {
+      k = ((i - P::TW2) / 64 + 1) * ((i - P::TW2) % 64) * (N / 512);
+    } else {
+      const int s = (i - P::TWF) / P::T, t = (i - P::TWF) % P::T;
+      k = (P::F > 1) ? (s % (P::F - 1) + 1) * (t + P::T * (s / (P::F > 1 ? P::F - 1 : 1))) : 0;
+    }
+    tws[i] = tab[k & (N - 1)];
+  }
+  __syncthreads();
+}
+
+// 8-point forward DFT in place, natural order
+__device__ __forceinline__ void dft8(float2 (&v)[8]) {
+  constexpr float kH = 0.70710678118654752f;
+  float2 a0 = f2add(v[0], v[4]), b0 = f2sub(v[0], v[4]);
+  float2 a1 = f2add(v[1], v[5]), b1 = f2sub(v[1], v[5]);
+  float2 a2 = f2add(v[2], v[6]), b2 = f2sub(v[2], v[6]);
+  float2 a3 = f2add(v[3], v[7]), b3 = f2sub(v[3], v[7]);
+  // b1 (1 - i) / sqrt 2, -i b2, b3 (-1 - i) / sqrt 2
+  b1 = f2mul(make_float2(b1.x + b1.y, b1.y - b1.x), make_float2(kH, kH));
+  b3 = f2mul(make_float2(b3.y - b3.x, -b3.x - b3.y), make_float2(kH, kH));
+  b2 = cmul_i<-1>(b2);
+  dft4<-1>(a0, a1, a2, a3);
+  dft4<-1>(b0, b1, b2, b3);
+  v[0] = a0; v[2] = a1; v[4] = a2; v[6] = a3;
+  v[1] = b0; v[3] = b1; v[5] = b2; v[7] = b3;
+}
+
+// N-point forward complex FFT of a team, v[r] at index t + T r on both ends, natural
+// order.  buf: BUF complex slots, free when the call starts after a team
+// barrier; its contents are undefined on return, and a barrier is needed before
+// others write it.  Layouts: LA(i) = i + i/16 after pass 0, LB(i) = i + 8 (i/64)
+// after pass 1, plain after pass 2: every access is a lane base plus a
+// compile-time offset and its half warps hit 16 distinct 8-byte slots.
+template <int N>
+__device__ __forceinline__ void pair_fft(float2 *buf, float2 (&v)[8], const float2 *tws, int t, int team) {
+  using P = PairFft<N>;
+  constexpr int T = P::T;
+  dft8(v);
+  {
+    float2 *w = buf + 8 * t + (t >> 1);
+#pragma unroll
+    for (int r = 0; r < 8; ++r) w[r] = v[r];
+  }
+  team_sync<T>(team);
+  {
+    const float2 *p = buf + t + (t >> 4);
+#pragma unroll
+    for (int r = 0; r < 8; ++r) v[r] = p[(T + T / 16) * r];
+  }
+#pragma unroll
+  for (int r = 1; r < 8; ++r) {
+    const float2 w = tws[P::TW1 + 8 * (r - 1) + (t & 7)];
+    v[r] = cmul(v[r], w);
+  }
+  dft8(v);
+  team_sync<T>(team);
+  {
+    float2 *w = buf + (t >> 3) * 72 + (t & 7);
+#pragma unroll
+    for (int r = 0; r < 8; ++r) w[8 * r] = v[r];
+  }
+  team_sync<T>(team);
+  if constexpr (N == 256) {
+    const float2 *p = buf + t;
+#pragma unroll
+    for (int r = 0; r < 8; ++r) v[r] = p[32 * r + 8 * (r >> 1)];
+  } else {
+    const float2 *p = buf + t + 8 * (t >> 6);
+#pragma unroll
+    for (int r = 0; r < 8; ++r) v[r] = p[(T + T / 8) * r];
+  }
+  if constexpr (P::P8 == 3) {
+#pragma unroll
+    for (int r = 1; r < 8; ++r) {
+      const float2 w = tws[P::TW2 + 64 * (r - 1) + (t & 63)];
+      v[r] = cmul(v[r], w);
+    }
+    dft8(v);  // N = 512: index t + 64 r, done
+    if constexpr (P::F > 1) {
+      team_sync<T>(team);
+      float2 *w = buf + (t >> 6) * 512 + (t & 63);
+#pragma unroll
+      for (int r = 0; r < 8; ++r) w[64 * r] = v[r];
+      team_sync<T>(team);
+#pragma unroll
+      for (int r = 0; r < 8; ++r) v[r] = buf[t + T * r];
+    }
+  }
+  if constexpr (P::F == 2) {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const float2 w = tws[P::TWF + i * T + t];
+      const float2 b = cmul(v[i + 4], w), a = v[i];
+      v[i] = f2add(a, b);
+      v[i + 4] = f2sub(a, b);
+    }
+  } else if constexpr (P::F == 4) {
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+#pragma unroll
+      for (int q = 1; q < 4; ++q) {
+        const float2 w = tws[P::TWF + (3 * i + q - 1) * T + t];
+        v[i + 2 * q] = cmul(v[i + 2 * q], w);
+      }
+      dft4<-1>(v[i], v[i + 2], v[i + 4], v[i + 6]);
+    }
+  }
+}
+
+// Powers |X_k|^2 of the two real segments (real part: a, imaginary part: b) for
+// k = 4t + 1 .. 4t + 4 from the transform v of a + i b: with Z_k and Z_{N-k},
+// |A_k|^2 = |Z_k + conj Z_{N-k}|^2 / 4, |B_k|^2 = |Z_k - conj Z_{N-k}|^2 / 4.
+// The factor 1/4 is left to the caller.  Starts and ends with a team barrier.
+template <int N>
+__device__ __forceinline__ void pair_powers(float2 *buf, const float2 (&v)[8], int t, int team, float (&pa)[4],
+                                            float (&pb)[4]) {
+  constexpr int T = PairFft<N>::T;
+  team_sync<T>(team);
+  {
+    float2 *w = buf + t + (t >> 4);
+#pragma unroll
+    for (int r = 0; r < 8; ++r) w[(T + T / 16) * r] = v[r];
+  }
+  team_sync<T>(team);
+  const float2 *up = buf + 4 * t + (t >> 2);                          // LA(4t)
+  const float2 *dn = buf + 4 * (2 * T - t - 1) + ((2 * T - t - 1) >> 2);  // LA(N - 4t - 4)
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    const float2 zk = j < 3 ? up[1 + j] : buf[4 * (t + 1) + ((t + 1) >> 2)];
+    const float2 zm = dn[3 - j];
+    const float2 s = f2add(zk, zm), d = f2sub(zk, zm);
+    pa[j] = fmaf(s.x, s.x, d.y * d.y);
+    pb[j] = fmaf(d.x, d.x, s.y * s.y);
+  }
+  team_sync<T>(team);
+}
+
+// ------------------------------------------------------------------ small-scale modes
+// Y_m = X_m / N of the modes 2c (y0) and 2c + 1 (y1) of one segment (Philox
+// words -> Box-Muller): X_m = A_m sqrt(-ln u1) e^{2 pi i u2} (= A (e1 + i e2)/sqrt 2).
+// Counter c serves modes 2c (words 0, 1) and 2c + 1 (words 2, 3); the words of
+// counter 0 that mode 0 (X_0 = 0) would use serve the Nyquist mode, X = A e1,
+// which y0 holds for c = 0.
+// ZNODES: amp and amp_hi hold (A_m / N)^2 at two z nodes, mixed with weight
+// w_hi; otherwise amp holds A_m / N and amp_hi is unused.
+template <int N, bool ZNODES>
+__device__ __forceinline__ void small_scale_modes(uint32_t c, const float *__restrict__ amp,
+                                                  const float *__restrict__ amp_hi, float w_hi, uint32_t seg,
+                                                  uint64_t id, uint32_t seed, float2 &y0, float2 &y1) {
+  const u32x4 w = philox4x32_10(u32x4{c, seg, static_cast<uint32_t>(id >> 32), 0u}, seed, static_cast<uint32_t>(id));
+  const bool nyq = (c == 0);
+  const int m0 = nyq ? N / 2 : 2 * c, m1 = 2 * c + 1;
+  float s0 = __ldg(amp + m0), s1 = __ldg(amp + m1);
+  if (ZNODES) {  // interpolate P_s between the nodes, then the root
+    s0 = sqrtf(fmaf(w_hi, __ldg(amp_hi + m0) - s0, s0));
+    s1 = sqrtf(fmaf(w_hi, __ldg(amp_hi + m1) - s1, s1));
+  }
+  const float2 p0 = unit_phase(w.y), p1 = unit_phase(w.w);
+  const float2 nl = neg_log_uniform2(w.x, w.z);
+  const float a0 = s0 * sqrt_pos((nyq ? 2.0f : 1.0f) * nl.x);
+  const float a1 = s1 * sqrt_pos(nl.y);
+  y0 = make_float2(a0 * p0.x, nyq ? 0.f : a0 * p0.y);
+  y1 = make_float2(a1 * p1.x, a1 * p1.y);
+}
+
+// The modes 2c, 2c + 1 of the pair (a, b) into the input of its transform.  The
+// inverse FFT of Z = A + i B is the forward FFT of Z with its index reversed, so
+// that one copy of the transform serves both directions: Z_m = A + i B goes to
+// index N - m and Z_{N-m} = conj A + i conj B to index m.  The upper half sits one
+// slot up, so that both pairs are stored 16 bytes at a time.
+template <int N>
+__device__ __forceinline__ void store_mode_pair(float2 *buf, int c, float2 a0, float2 a1, float2 b0, float2 b1) {
+  float2 z0 = make_float2(a0.x - b0.y, a0.y + b0.x), y0 = make_float2(a0.x + b0.y, b0.x - a0.y);
+  const float2 z1 = make_float2(a1.x - b1.y, a1.y + b1.x), y1 = make_float2(a1.x + b1.y, b1.x - a1.y);
+  if (c == 0) {
+    buf[N / 2 + 1] = make_float2(a0.x, b0.x);  // the Nyquist mode (real in each segment)
+    z0 = y0 = make_float2(0.f, 0.f);
+  }
+  *reinterpret_cast<float4 *>(buf + 2 * c) = make_float4(y0.x, y0.y, y1.x, y1.y);
+  *reinterpret_cast<float4 *>(buf + N - 2 * c) = make_float4(z1.x, z1.y, z0.x, z0.y);
+}
+template <int N>
+__device__ __forceinline__ void load_modes(const float2 *buf, float2 (&v)[8], int t) {
+  constexpr int T = N / 8;
+#pragma unroll
+  for (int r = 0; r < 8; ++r) v[r] = buf[t + T * r + (r >= 4 ? 1 : 0)];
+}
+
+// ------------------------------------------------------------------ cells of a run of pixels
+// A sight line crosses a cell in ~1/(dr/cell) pixels (11 at the paper's sizes),
+// and inside a cell the trilinear interpolant along the line is a cubic in the
+// pixel number.  So the team finds the cells of its run of up to 2N pixels,
+// one thread per cell reads the 8 corners and expands the cubic of (delta,
+// eta) about the cell's first pixel, and each pixel then takes two 16-byte
+// shared-memory reads and three packed FMAs instead of eight global loads and
+// seven lerps.
+//
+// Positions along a run are 2^-35 cells: frac + s q at pixel q, with s < 2^32 for
+// steps below 1/8 of a cell, one 32 x 32 + 64-bit multiply-add each; the step's
+// rounding moves a position by at most 2^-36 cells a pixel (the weights have 23
+// bits).  The same arithmetic decides which cell a pixel is in and where it is
+// inside it, so a pixel next to a face may take either cell but always with the
+// weight that belongs to it.  A decreasing coordinate runs on its complement,
+// which increases and crosses cells at the same pixels.
+struct alignas(16) LineAxis {
+  uint64_t frac;  // position of pixel 0 inside its cell, plus the rounding of the weights
+  uint32_t s;     // |step|
+  int32_t c0;     // cell of pixel 0
+  float inv;      // 1 / s
+  float slope;    // signed step in cells
+  int32_t sign;   // +1, or -1 for a decreasing coordinate
+  int32_t n;      // crossings up to the last pixel
+};
+struct CellPlan {
+  float4 *a, *b;   // cubic: a = (c0, c1), b = (c2, c3), each (delta, eta)
+  float *first;    // first pixel of the cell
+  uint2 *mask;     // per 32 pixels: {a bit for each first pixel of a cell, bits before}
+  LineAxis *line;  // x, y, z
+  static constexpr size_t kLineBytes = 3 * sizeof(LineAxis);
+};
+
+// Cell plan of a run of npx pixels from pixel j0 of a skewer: lines, masks and
+// first pixels; returns the number of cells (the same in every thread).  Starts
+// with the plan's memory free and ends with a team barrier.  A run has at most
+// cell_capacity() <= 3 T cells (see use_cells).
+template <int N>
+__device__ __forceinline__ int plan_cells(const CellPlan &C, const mk_skewer *rec, int j0, int npx, int t,
+                                          int team) {
+  constexpr int T = N / 8, WORDS = N / 16;
+  if (t < WORDS) C.mask[t] = make_uint2(0u, 0u);
+  if (t < 3) {
+    const int64_t step = rec->step[t], p = rec->p0[t] + j0 * step;
+    const bool neg = step < 0;
+    LineAxis A;
+    A.frac = ((static_cast<uint64_t>(neg ? ~p : p) & ((uint64_t(1) << 44) - 1)) >> 9) + (1u << 11);
+    A.s = static_cast<uint32_t>(((neg ? -step : step) + 256) >> 9);
+    A.c0 = static_cast<int32_t>(p >> 44);
+    A.inv = __fdividef(1.0f, static_cast<float>(A.s));
+    A.slope = static_cast<float>(step) * 0x1p-44f;
+    A.sign = neg ? -1 : 1;
+    A.n = static_cast<int>((A.frac + static_cast<uint64_t>(A.s) * (npx - 1)) >> 35);
+    if (A.frac >> 35) {  // rounded up to the next cell (weight 0)
+      A.frac -= uint64_t(1) << 35;
+      A.c0 += A.sign;
+      A.n -= 1;
+    }
+    C.line[t] = A;
+  }
+  team_sync<T>(team);
+  const int nx = C.line[0].n, nxy = nx + C.line[1].n, total = nxy + C.line[2].n;
+  int *at = reinterpret_cast<int *>(C.a);  // (free until the cubics) first pixel past each crossing
+#pragma unroll (N == 256 ? 1 : 3)
+  for (int e = 0; e < 3; ++e) {
+    const int i = t + T * e;
+    if (i < total) {
+      const int ax = (i >= nx ? 1 : 0) + (i >= nxy ? 1 : 0);
+      const uint32_t k = 1 + i - (i >= nxy ? nxy : (i >= nx ? nx : 0));
+      const uint64_t frac = C.line[ax].frac;
+      const uint32_t s = C.line[ax].s;
+      // the smallest q with frac + q s >= k cells: the FP32 quotient is within
+      // 1e-3 of it, so q is its integer part or one or two more
+      const uint32_t q0 =
+          static_cast<uint32_t>(__ull2float_rn((static_cast<uint64_t>(k) << 35) - frac) * C.line[ax].inv);
+      const uint64_t v = frac + static_cast<uint64_t>(s) * q0;
+      const int q = static_cast<int>(q0) + (static_cast<uint32_t>(v >> 35) < k ? 1 : 0) +
+                    (static_cast<uint32_t>((v + s) >> 35) < k ? 1 : 0);
+      at[i] = q;
+      atomicOr(&C.mask[q >> 5].x, 1u << (q & 31));
+    }
+  }
+  team_sync<T>(team);
+  if (t < 32) {  // prefix counts of the words, WORDS / 32 a lane
+    constexpr int PER = WORDS < 32 ? 1 : WORDS / 32;
+    int c[PER], s = 0;
+#pragma unroll
+    for (int j = 0; j < PER; ++j) {
+      const int w = t * PER + j;
+      c[j] = w < WORDS ? __popc(C.mask[w].x) : 0;
+      s += c[j];
+    }
+    int run = s;
+#pragma unroll
+    for (int o = 1; o < (WORDS < 32 ? WORDS : 32); o <<= 1) {
+      const int v = __shfl_up_sync(0xffffffffu, run, o);
+      if (t >= o) run += v;
+    }
+    run -= s;
+#pragma unroll
+    for (int j = 0; j < PER; ++j) {
+      const int w = t * PER + j;
+      if (w < WORDS) C.mask[w].y = static_cast<uint32_t>(run);
+      run += c[j];
+    }
+  }
+  if (t == 0) C.first[0] = 0.f;
+  team_sync<T>(team);
+#pragma unroll (N == 256 ? 1 : 3)
+  for (int e = 0; e < 3; ++e) {
+    const int i = t + T * e;
+    if (i < total) {
+      const int q = at[i];
+      const uint2 m = C.mask[q >> 5];
+      C.first[m.y + __popc(m.x & (0xffffffffu >> (31 - (q & 31))))] = static_cast<float>(q);
+    }
+  }
+  const uint2 m = C.mask[WORDS - 1];
+  const int cells = static_cast<int>(m.y) + __popc(m.x) + 1;
+  team_sync<T>(team);
+  return cells;
+}
+
+// Sight-line weights of the velocity-gradient tensor (Eq. eta) from the step in
+// any unit: {ux^2, uy^2, uz^2, 2 ux uy, 2 ux uz, 2 uy uz} (MK_BOX_TENSOR only).
+template <int LAYOUT>
+__device__ __forceinline__ void tensor_weights(float ux, float uy, float uz, float (&uu)[6]) {
+  if constexpr (LAYOUT == MK_BOX_TENSOR) {
+    const float inv = rsqrtf(ux * ux + uy * uy + uz * uz);
+    const float vx = ux * inv, vy = uy * inv, vz = uz * inv;
+    uu[0] = vx * vx;
+    uu[1] = vy * vy;
+    uu[2] = vz * vz;
+    uu[3] = 2.f * vx * vy;
+    uu[4] = 2.f * vx * vz;
+    uu[5] = 2.f * vy * vz;
+  }
+}
+
+// (delta, eta) at the 8 corners of cell (x0, y0, z0); eta of MK_BOX_TENSOR is
+// the velocity-gradient tensor contracted with the sight line, uu = {ux^2,
+// uy^2, uz^2, 2 ux uy, 2 ux uz, 2 uy uz}.
+template <int LAYOUT>
+__device__ __forceinline__ void load_corners(const float *__restrict__ d, const float *__restrict__ e, int lgn, int x0,
+                                             int y0, int z0, const float (&uu)[6], float2 (&v)[8]) {
+  const int mask = (1 << lgn) - 1;
+  if constexpr (LAYOUT == MK_BOX_PADDED || LAYOUT == MK_BOX_HALO || LAYOUT == MK_BOX_TENSOR) {
+    constexpr int h = LAYOUT == MK_BOX_HALO ? 3 : 0;
+    const int64_t n1 = mask + 1 + (LAYOUT == MK_BOX_HALO ? 6 : 1);
+    const int64_t i00 = ((z0 + h) * n1 + (y0 + h)) * n1 + (x0 + h);
+    const int64_t row[4] = {i00, i00 + n1, i00 + n1 * n1, i00 + n1 * n1 + n1};
+    if constexpr (LAYOUT == MK_BOX_TENSOR) {
+      const float4 *b = reinterpret_cast<const float4 *>(d);
+#pragma unroll
+      for (int k = 0; k < 8; ++k) {
+        const float4 p = __ldg(b + 2 * (row[k >> 1] + (k & 1))), q = __ldg(b + 2 * (row[k >> 1] + (k & 1)) + 1);
+        const float eta = fmaf(uu[0], p.y, fmaf(uu[1], p.z, fmaf(uu[2], p.w,
+                          fmaf(uu[3], q.x, fmaf(uu[4], q.y, uu[5] * q.z)))));
+        v[k] = make_float2(p.x, eta);
+      }
+    } else {
+      const float2 *b = reinterpret_cast<const float2 *>(d);
+#pragma unroll
+      for (int k = 0; k < 8; ++k) v[k] = __ldg(b + row[k >> 1] + (k & 1));
+    }
+  } else {
+    const int x1 = (x0 + 1) & mask, y1 = (y0 + 1) & mask, z1 = (z0 + 1) & mask;
+    const size_t zz[2] = {static_cast<size_t>(z0) << (2 * lgn), static_cast<size_t>(z1) << (2 * lgn)};
+    const size_t yy[2] = {static_cast<size_t>(y0) << lgn, static_cast<size_t>(y1) << lgn};
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      const size_t i = zz[k >> 2] | yy[(k >> 1) & 1] | static_cast<size_t>((k & 1) ? x1 : x0);
+      v[k] = LAYOUT == MK_BOX_INTERLEAVED ? __ldg(reinterpret_cast<const float2 *>(d) + i)
+                                          : make_float2(__ldg(d + i), __ldg(e + i));
+    }
+  }
+}
+
+__device__ __forceinline__ float2 f2fma1(float a, float2 b, float2 c) { return f2fma(make_float2(a, a), b, c); }
+__device__ __forceinline__ float2 f2mul1(float a, float2 b) { return f2mul(make_float2(a, a), b); }
+
+// Trilinear (delta, eta) at one fixed-point position, for pixels too long for
+// the cells of a run to pay: lerps in x, then y, then z, the pair packed.
+template <int LAYOUT>
+__device__ __forceinline__ float2 gather(const float *__restrict__ d, const float *__restrict__ e, int lgn, int64_t px,
+                                         int64_t py, int64_t pz, const int64_t (&st)[3]) {
+  const int mask = (1 << lgn) - 1;
+  float2 v[8];
+  float uu[6];
+  tensor_weights<LAYOUT>(static_cast<float>(st[0]), static_cast<float>(st[1]), static_cast<float>(st[2]), uu);
+  load_corners<LAYOUT>(d, e, lgn, cell_of(px, mask), cell_of(py, mask), cell_of(pz, mask), uu, v);
+  const float tx = weight_of(px), ty = weight_of(py), tz = weight_of(pz);
+  const float2 c0 = f2lerp(v[0], v[1], tx), c1 = f2lerp(v[2], v[3], tx);
+  const float2 c2 = f2lerp(v[4], v[5], tx), c3 = f2lerp(v[6], v[7], tx);
+  return f2lerp(f2lerp(c0, c1, ty), f2lerp(c2, c3, ty), tz);
+}
+
+// The cubic of cell c: the trilinear interpolant of the corners along the line,
+// expanded in the pixel number from the cell's first pixel.  At that pixel it
+// is the lerp in x, then y, then z.
+template <int LAYOUT>
+__device__ __forceinline__ void expand_cell(const CellPlan &C, int c, const float *__restrict__ d,
+                                            const float *__restrict__ e, int lgn) {
+  const int mask = (1 << lgn) - 1;
+  const uint32_t q = static_cast<uint32_t>(C.first[c]);
+  int cell[3];
+  float w[3], sl[3];
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    const LineAxis A = C.line[k];
+    const uint64_t v = A.frac + static_cast<uint64_t>(A.s) * q;
+    cell[k] = (A.c0 + A.sign * static_cast<int>(v >> 35)) & mask;
+    // weight in the direction of travel, 23 bits; 1 - it against the axis
+    const float f = __uint_as_float(0x3F800000u | (static_cast<uint32_t>(v >> 12) & 0x7FFFFFu)) - 1.0f;
+    w[k] = A.sign > 0 ? f : 1.0f - f;
+    sl[k] = A.slope;
+  }
+  const float wx = w[0], wy = w[1], wz = w[2], sx = sl[0], sy = sl[1], sz = sl[2];
+  float2 v[8];
+  float uu[6];
+  tensor_weights<LAYOUT>(sx, sy, sz, uu);
+  load_corners<LAYOUT>(d, e, lgn, cell[0], cell[1], cell[2], uu, v);
+  float2 f0[2], f1[2], f2[2];
+#pragma unroll
+  for (int k = 0; k < 2; ++k) {
+    const float2 d0 = f2sub(v[4 * k + 1], v[4 * k]), d1 = f2sub(v[4 * k + 3], v[4 * k + 2]);
+    const float2 a0 = f2fma1(wx, d0, v[4 * k]), a1 = f2fma1(wx, d1, v[4 * k + 2]);
+    const float2 b0 = f2mul1(sx, d0), b1 = f2mul1(sx, d1);
+    const float2 da = f2sub(a1, a0), db = f2sub(b1, b0);
+    f0[k] = f2fma1(wy, da, a0);
+    f1[k] = f2fma1(wy, db, f2fma1(sy, da, b0));
+    f2[k] = f2mul1(sy, db);
+  }
+  const float2 g0 = f2sub(f0[1], f0[0]), g1 = f2sub(f1[1], f1[0]), g2 = f2sub(f2[1], f2[0]);
+  const float2 c0 = f2fma1(wz, g0, f0[0]);
+  const float2 c1 = f2fma1(wz, g1, f2fma1(sz, g0, f1[0]));
+  const float2 c2 = f2fma1(wz, g2, f2fma1(sz, g1, f2[0]));
+  const float2 c3 = f2mul1(sz, g2);
+  C.a[c] = make_float4(c0.x, c0.y, c1.x, c1.y);
+  C.b[c] = make_float4(c2.x, c2.y, c3.x, c3.y);
+}
+
+// (delta, eta) at pixel q of the run, m its mask word (uniform in the warp)
+__device__ __forceinline__ float2 eval_cell(const CellPlan &C, uint2 m, float q, uint32_t lanes_le) {
+  const int c = static_cast<int>(m.y) + __popc(m.x & lanes_le);
+  const float4 a = C.a[c], b = C.b[c];
+  const float x = q - C.first[c];
+  const float2 r = f2fma1(x, make_float2(b.z, b.w), make_float2(b.x, b.y));
+  return f2fma1(x, f2fma1(x, r, make_float2(a.z, a.w)), make_float2(a.x, a.y));
+}
+
+}  // namespace mk

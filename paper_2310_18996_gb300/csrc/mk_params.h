@@ -30,8 +30,7 @@ struct GeomParams {
   int32_t n_min, n_max;
   double origin[3], cell;
   int32_t j_max;  // pixel tables cover J < j_max
-  int32_t n_fft;  // segment length for the segment count (0: none)
-  int32_t rebin;  // > 0: write floor(n / rebin) counts instead (flux offsets)
+  int32_t unit_px;  // pixels of a work unit of the skewer kernel (a pair of segments)
 };
 
 using NodeParams = mk_fgpa_nodes;
@@ -88,18 +87,18 @@ __host__ __device__ inline void finalize_bin_p1d(mk_stats_bin *b, int k, double 
 // Everything the fused / split skewer kernels read.
 struct SkewerParams {
   const mk_skewer *sk;
-  const int64_t *segoff;  // exclusive prefix of segments per skewer, n_sk + 1
+  const int64_t *segoff;  // exclusive prefix of pairs of segments per skewer, n_sk + 1
   int64_t n_sk;
   // box
   const float *box_d;  // planar delta, or (delta, eta) pairs (interleaved, padded)
   const float *box_e;  // planar eta or NULL
   int32_t lgn;
+  int32_t cell_cap;  // cells a pair's sight line may cross (0: gathers per pixel)
   // tables
   const float4 *pixtab;  // per global pixel J: {G, a log2e, b log2e, c}
   const int16_t *zbin;     // per J: z bin, -1 below, n_z above
   const int16_t *segzbin;  // per J: z bin of the mean z of pixels J .. J+N-1
   const int32_t *bin_end;  // [k + 1], k = -1 .. n_z: first J with zbin > k (large beyond the tables)
-  const double *cumz;      // per J: sum_{J' < J} z_J'
   const float *amp;        // A_m / N, m = 0..N/2; with ps_nodes >= 2: (A_m / N)^2 per node, node-major
   int32_t ps_nodes;        // z-dependent small-scale power: tables at ps_z (>= 2), else one
   float ps_z[MK_MAX_NODES];
@@ -113,11 +112,17 @@ struct SkewerParams {
   // statistics
   int32_t do_stats;
   int32_t n_z, n_k;
-  double z_lo, dz, dr;
   float p1d_scale;   // dr / N
   double *partials;  // [gridDim.x][layout size]
   int *err;
 };
+
+// Cells the sight line of a run of 2n pixels can cross, a multiple of 4: at most
+// sqrt(3) dr/cell crossings a pixel (|ux| + |uy| + |uz| <= sqrt 3), one more
+// per axis for the start, and the first cell.
+inline int cell_capacity(int n, double dr_over_cell) {
+  return (static_cast<int>(1.7320508076 * dr_over_cell * (2 * n - 1)) + 5 + 3) / 4 * 4;
+}
 
 // Statistics pass over stored flux (any rebin).
 struct StatParams {

@@ -2,13 +2,13 @@
 // length is instantiated in its own translation unit (mk_skewer_<N>.cu).
 #pragma once
 
-#include "mk_device.cuh"
+#include "mk_pair.cuh"
 
 namespace mk {
 
 // =================================================================== shared-memory plan
-// Per CTA: per-warp statistic accumulators (when statistics are on), the
-// twiddle table, then one FFT buffer of N/2 + 2 complex values per team.
+// Statistics kernels, per CTA: per-warp statistic accumulators, the twiddle
+// table, then one FFT buffer of N/2 + 2 complex values per team.
 template <int N>
 struct TeamSmem {
   static constexpr int T = N / 8;
@@ -19,6 +19,30 @@ struct TeamSmem {
   __host__ __device__ static size_t bytes(int threads, int n_z, int n_k, bool stats) {
     return acc_bytes(threads, n_z, n_k, stats) + TwTab<N>::BYTES +
            static_cast<size_t>(threads / T) * BUF * sizeof(float2);
+  }
+};
+
+// Fused kernel, per CTA: per-warp accumulators (when statistics are on), the
+// twiddles, the ends of the z bins, then per team one area that is the FFT's
+// exchange buffer and, between the two transforms, the cubics of the pair's
+// cells; a stash of N floats; the skewer's record; and the line, the masks and
+// the cells' first pixels (cap, a multiple of 4, is 0 where pixels gather for
+// themselves).
+template <int N>
+struct PairSmem {
+  static constexpr int T = N / 8;
+  __host__ __device__ static size_t area_bytes(int cap) {
+    const size_t f = sizeof(float2) * PairFft<N>::BUF, c = 32 * static_cast<size_t>(cap);
+    return f > c ? f : c;
+  }
+  static constexpr size_t HEAD = (PairFft<N>::TW_BYTES + 15) / 16 * 16 + (sizeof(int32_t) * (MK_MAX_ZBINS + 2) + 15) / 16 * 16;
+  static constexpr int REC = 10;  // 8-byte words: the record, then the end of its pairs
+  __host__ __device__ static size_t team_bytes(int cap) {
+    return area_bytes(cap) + sizeof(float) * N + sizeof(uint64_t) * REC +
+           (cap > 0 ? CellPlan::kLineBytes + sizeof(uint2) * (N / 16) + sizeof(float) * cap : 0);
+  }
+  __host__ __device__ static size_t bytes(int threads, int n_z, int n_k, bool stats, int cap) {
+    return TeamSmem<N>::acc_bytes(threads, n_z, n_k, stats) + HEAD + static_cast<size_t>(threads / T) * team_bytes(cap);
   }
 };
 
@@ -64,20 +88,35 @@ __device__ __forceinline__ void flush_warp_partials(unsigned char *smem, int nwa
 }
 
 // =================================================================== fused skewer kernel
-// One team per segment of N pixels: small-scale modes -> inverse real FFT ->
-// per pixel gather, growth, FGPA, stores and pixel sums -> forward FFT of the
-// flux -> P1D.  Teams take contiguous ranges of segments (all segments cost
-// the same).  Pixel sums stay in registers, across segments, for as long as
-// the warp's pixels stay in one z bin: the warp flushes them to its shared
+// One team per pair of segments of N pixels of a skewer: cells of the pair's
+// sight line -> small-scale modes of both -> one inverse FFT -> per pixel the
+// cell's cubic, growth, FGPA, stores and pixel sums -> one forward FFT of both
+// fluxes -> P1D.  Pairs never straddle skewers, so a skewer's pixels do not
+// depend on how a catalogue is cut into launches.  Teams take contiguous ranges
+// of pairs.  Pixel sums stay in registers, across segments, for as long as the
+// warp's pixels stay in one z bin: the warp flushes them to its shared
 // accumulators when its pixels reach the end of the bin (bin_end) or a
 // segment starts in another bin.
-// INTERP: MK_INTERP_TRILINEAR, or MK_INTERP_GAUSS7 (LAYOUT must be MK_BOX_HALO).
+//
+// Bound by instruction issue: 6.4 warp instructions a pixel at 70 % of the issue
+// slots, DRAM ~10 B a pixel.  One radix-8 transform for two segments and one set
+// of corner loads per cell of the sight line take 1.07 ms per 1.37e8 pixels
+// (512^3 box, 100k quasars, N = 256) where a radix-4 transform per segment and a
+// gather of eight corners per pixel took 1.25 ms, and 1.53 against 2.19 ms on a
+// tensor box; a step of the 1024^3 box with 1M quasars went from 13.0 to 11.2 ms.
+// The loop over pairs has to fit the instruction cache: variants of it whose
+// pixel loops were unrolled further (4400 to 6000 instructions instead of 3600)
+// ran 10 to 50 % slower, stalled on fetches.
+//
+// CELLS: the trilinear interpolant from the cubics of the line's cells (needs
+// P.cell_cap); otherwise each pixel gathers for itself: INTERP ==
+// MK_INTERP_GAUSS7 (LAYOUT must be MK_BOX_HALO), or trilinear with pixels too
+// long for the cells to pay (see use_cells).
 // PSZ: P_s given at several redshifts (P.ps_nodes >= 2), interpolated per segment
-// FIXLGN > 0: a padded box of side 2^FIXLGN (constant strides in the gather)
-template <int N, int LAYOUT, bool BIG, int MINB, int INTERP = MK_INTERP_TRILINEAR, bool PSZ = false, int FIXLGN = 0>
+template <int N, int LAYOUT, int MINB, int INTERP, bool PSZ, bool CELLS>
 __global__ void __launch_bounds__(256, MINB) k_skewer(SkewerParams P) {
   constexpr int T = N / 8;
-  constexpr int BUF = TeamSmem<N>::BUF;
+  constexpr int kRows = 2;  // rows of T pixels per round of the pixel loop
   const int teams = blockDim.x / T;
   const int team = threadIdx.x / T, t = threadIdx.x % T, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int wlo0 = t & ~31;  // first team pixel of this warp
@@ -85,14 +124,27 @@ __global__ void __launch_bounds__(256, MINB) k_skewer(SkewerParams P) {
   extern __shared__ __align__(16) unsigned char smem[];
   const size_t wbytes = P.do_stats ? WarpAcc::bytes(P.n_z, P.n_k) : 0;
   float2 *tws = reinterpret_cast<float2 *>(smem + nwarps * wbytes);
-  float2 *buf = tws + TwTab<N>::SLOTS * T + team * BUF;
-  float *fb = reinterpret_cast<float *>(buf);
+  int32_t *bin_end = reinterpret_cast<int32_t *>(tws + (PairFft<N>::TW_BYTES + 15) / 16 * 2);
+  unsigned char *mine = smem + nwarps * wbytes + PairSmem<N>::HEAD + team * PairSmem<N>::team_bytes(P.cell_cap);
+  float2 *buf = reinterpret_cast<float2 *>(mine);
+  CellPlan C;
+  C.a = reinterpret_cast<float4 *>(mine);
+  C.b = C.a + P.cell_cap;
+  float *stash = reinterpret_cast<float *>(mine + PairSmem<N>::area_bytes(P.cell_cap));
+  uint64_t *recw = reinterpret_cast<uint64_t *>(stash + N);
+  const mk_skewer *rec = reinterpret_cast<const mk_skewer *>(recw);
+  C.line = reinterpret_cast<LineAxis *>(recw + PairSmem<N>::REC);
+  C.mask = reinterpret_cast<uint2 *>(C.line + 3);
+  C.first = reinterpret_cast<float *>(C.mask + N / 16);
   const WarpAcc W = WarpAcc::at(smem + warp * wbytes, P.n_z, P.n_k);
-  if (P.do_stats) zero_warp_acc(smem + warp * wbytes, wbytes);
-  fill_twiddles<N>(tws, P.tw);
+  if (P.do_stats) {
+    zero_warp_acc(smem + warp * wbytes, wbytes);
+    for (int k = threadIdx.x; k < P.n_z + 2; k += blockDim.x) bin_end[k] = P.bin_end[k];
+  }
+  fill_pair_twiddles<N>(tws, P.tw);  // (ends with a CTA barrier)
 
-  // segments segoff[0] .. segoff[n_sk] (a slice of a larger catalogue may
-  // start at segoff[0] > 0)
+  // pairs segoff[0] .. segoff[n_sk] (a slice of a larger catalogue may start
+  // at segoff[0] > 0)
   const int64_t u0 = P.segoff[0], nunits = P.segoff[P.n_sk] - u0;
   const int64_t g = static_cast<int64_t>(blockIdx.x) * teams + team;
   const int64_t G = static_cast<int64_t>(gridDim.x) * teams;
@@ -100,158 +152,263 @@ __global__ void __launch_bounds__(256, MINB) k_skewer(SkewerParams P) {
   const int64_t uend = u0 + (g + 1) * nunits / G;
   int64_t i = u < uend ? upper_index(P.segoff, P.n_sk, u) : 0;
 
+  // The skewer's record waits in shared memory, and the next skewer's in a
+  // register of each of ten threads (thread t: word t; t = 9: the end of its
+  // pairs), so that a new skewer costs no round trip to memory.
+  static_assert(sizeof(mk_skewer) == 72, "nine words");
+  auto fetch = [&](int64_t q) -> uint64_t {
+    if (q >= P.n_sk) return 0;
+    if (t < 9) return reinterpret_cast<const uint64_t *>(P.sk + q)[t];
+    return t == 9 ? static_cast<uint64_t>(P.segoff[q + 1]) : 0;
+  };
+  uint64_t next = fetch(i);
+  int64_t base = P.segoff[i], end = base;  // pairs of skewer i - 1 end where i's begin
+  --i;
+
   PixelSums acc;
   acc.zero();
   int zc = -2;  // z bin of acc (warp-uniform), -2 before the first segment
+  const uint32_t lanes_le = 0xffffffffu >> (31 - lane);
+  const P1dBins bins(N / 2, P.n_k, t);
+  const bool put_fields = P.delta_out != nullptr, put_flux = P.flux_out != nullptr;
 
   for (; u < uend; ++u) {
-    while (P.segoff[i + 1] <= u) ++i;
-    const int s = static_cast<int>(u - P.segoff[i]);
-    const mk_skewer sk = P.sk[i];
-    const int64_t j0 = static_cast<int64_t>(s) * N;
-    const int npx = static_cast<int>(min(static_cast<int64_t>(N), sk.n - j0));
-    if ((P.delta_out || P.flux_out) && sk.offset + sk.n > P.capacity) {
+    while (u >= end) {  // (the last pair ended with a barrier)
+      base = end;
+      ++i;
+      if (t < PairSmem<N>::REC) recw[t] = next;
+      next = fetch(i + 1);
+      team_sync<T>(team);
+      end = static_cast<int64_t>(recw[9]);
+      if (u >= end) team_sync<T>(team);  // an empty skewer
+    }
+    const int s = 2 * static_cast<int>(u - base);
+    const int64_t offset = rec->offset;
+    const int n = rec->n;
+    const int j0 = s * N;              // first pixel of the pair
+    const int npair = min(2 * N, n - j0);
+    if ((put_fields || put_flux) && offset + n > P.capacity) {
       if (t == 0) raise_error(P.err, ERR_CAPACITY);
+      team_sync<T>(team);
       continue;
     }
-    // ---- start the box rows of this segment's stencils on their way to L2:
-    // lane t samples pixel 8t + 4 (the modes and the inverse FFT below hide
-    // the latency)
-    {
-      const int64_t ps = j0 + min(npx - 1, 8 * t + 4);
-      prefetch_stencil<LAYOUT, BIG>(P.box_d, P.lgn, sk.p0[0] + kRoundQ + ps * sk.step[0],
-                                    sk.p0[1] + kRoundQ + ps * sk.step[1], sk.p0[2] + kRoundQ + ps * sk.step[2]);
-    }
-    // ---- small-scale field of this segment
-    if constexpr (PSZ) {  // P_s at the mean z of the segment's window, linear between nodes
-      const float zw = __ldg(P.zwin + sk.j_lo + static_cast<int>(j0));
-      const int k = P.ps_nodes;
-      int n0 = 0;
-      while (n0 + 2 < k && zw >= P.ps_z[n0 + 1]) ++n0;
-      const float w_hi = fminf(fmaxf((zw - P.ps_z[n0]) / (P.ps_z[n0 + 1] - P.ps_z[n0]), 0.f), 1.f);
-      const float *amp = P.amp + n0 * (N / 2 + 1);
-      small_scale_modes<N, true>(buf, amp, amp + (N / 2 + 1), w_hi, static_cast<uint32_t>(s), sk.id, P.seed, t);
-    } else {
-      small_scale_modes<N, false>(buf, P.amp, nullptr, 0.f, static_cast<uint32_t>(s), sk.id, P.seed, t);
-    }
-    team_sync<T>(team);
-    inverse_real_fft<N>(buf, tws, t, team);
-
-    // ---- per pixel: gather, growth, FGPA, stores, pixel sums
-    const int jb = sk.j_lo + static_cast<int>(j0);
-    int pend = 0;  // segment pixel where bin zc ends
+    const int jb0 = rec->j_lo + j0;
+    const bool two = npair > N;
+    // z bins of the two segments' first pixels and of the full segments
+    int z0[2] = {0, 0}, zs[2] = {-1, -1};
     if (P.do_stats) {
-      const int zs = __ldg(P.zbin + jb);
-      if (zs != zc) {
-        if (zc != -2) flush_bin_sums(W, P.n_z, zc, acc, lane);
-        acc.zero();
-        zc = zs;
-      }
-      pend = __ldg(P.bin_end + zc + 1) - jb;
+      z0[0] = __ldg(P.zbin + jb0);
+      if (two) z0[1] = __ldg(P.zbin + jb0 + N);
+      if (npair >= N) zs[0] = __ldg(P.segzbin + jb0);
+      if (npair == 2 * N) zs[1] = __ldg(P.segzbin + jb0 + N);
     }
-    // sight-line weights of the velocity-gradient tensor (Eq. eta)
-    float uu[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-    if constexpr (LAYOUT == MK_BOX_TENSOR) {
-      const float ux = static_cast<float>(sk.step[0]), uy = static_cast<float>(sk.step[1]),
-                  uz = static_cast<float>(sk.step[2]);
-      const float inv = rsqrtf(ux * ux + uy * uy + uz * uz);
-      const float vx = ux * inv, vy = uy * inv, vz = uz * inv;
-      uu[0] = vx * vx;
-      uu[1] = vy * vy;
-      uu[2] = vz * vz;
-      uu[3] = 2.f * vx * vy;
-      uu[4] = 2.f * vx * vz;
-      uu[5] = 2.f * vy * vz;
+    // ---- start the box rows of the pair's stencils on their way to L2, where
+    // the loads are many (the tensor's 64 bytes a corner row, 1.57 -> 1.48 ms
+    // per 1.4e8 pixels; gathers per pixel): lane t samples pixel 16t + 8.  The
+    // 8-byte layouts read each cell once and gain nothing from it.
+    if constexpr (!CELLS || LAYOUT == MK_BOX_TENSOR) {
+      const int64_t q = j0 + min(npair - 1, 16 * t + 8);
+      prefetch_stencil<LAYOUT>(P.box_d, P.lgn, rec->p0[0] + kRoundQ + q * rec->step[0],
+                               rec->p0[1] + kRoundQ + q * rec->step[1], rec->p0[2] + kRoundQ + q * rec->step[2]);
     }
-    int64_t px = sk.p0[0] + kRoundQ + (j0 + t) * sk.step[0];
-    int64_t py = sk.p0[1] + kRoundQ + (j0 + t) * sk.step[1];
-    int64_t pz = sk.p0[2] + kRoundQ + (j0 + t) * sk.step[2];
-    const int64_t sx = T * sk.step[0], sy = T * sk.step[1], sz = T * sk.step[2];
-    const int64_t out0 = sk.offset + j0;
-    // warp-uniform: this warp's pixels of the segment all lie before pend
-    const bool one_bin = min(T * 7 + wlo0 + 32, npx) <= pend;
-    // pixel p: gather, growth, small-scale field, FGPA, stores; returns F
-    auto synth = [&](int p, float2 &x) -> float {
-      float2 de;
-      if constexpr (INTERP == MK_INTERP_GAUSS7) {
-        static_assert(LAYOUT == MK_BOX_HALO, "the Gaussian kernel reads a halo box");
-        de = gather_gauss7<BIG>(P.box_d, P.lgn, px, py, pz);
-      } else if constexpr (LAYOUT == MK_BOX_TENSOR) {
-        de = gather_tensor<BIG>(P.box_d, P.lgn, px, py, pz, uu);
-      } else {
-        de = gather<LAYOUT, BIG, FIXLGN>(P.box_d, P.box_e, P.lgn, px, py, pz);
-      }
-      const float4 tb = __ldg(P.pixtab + jb + p);
-      x = make_float2(fmaf(tb.x, de.x, fb[p]), tb.x * de.y);
-      const float f = fgpa(tb, x.x, x.y);
-      if (P.delta_out) {
-        P.delta_out[out0 + p] = x.x;
-        P.eta_out[out0 + p] = x.y;
-      }
-      if (P.flux_out) P.flux_out[out0 + p] = f;
-      return f;
-    };
-    // (the tensor and Gaussian-kernel gathers keep one loop: their registers
-    // do not leave room for a second copy)
-    constexpr bool kLean = LAYOUT != MK_BOX_TENSOR && INTERP == MK_INTERP_TRILINEAR;
-    if (kLean && npx == N && (!P.do_stats || one_bin)) {
-      // a full segment inside one z bin (most segments): no per-pixel bounds or bin checks
-#pragma unroll 2
-      for (int k = 0; k < 8; ++k) {
-        const int p = t + T * k;
-        float2 x;
-        const float f = synth(p, x);
-        if (P.do_stats) acc.add_sums(f, x);
-        fb[p] = f;
-        px += sx;
-        py += sy;
-        pz += sz;
-      }
-      acc.n += 8.f;  // this thread's pixels of the segment
-    } else {
-#pragma unroll 2
-    for (int k = 0; k < 8; ++k) {
-      const int p = t + T * k;
-      float f = 0.f;
-      float2 x = make_float2(0.f, 0.f);
-      if (p < npx) f = synth(p, x);
-      if (P.do_stats && one_bin) {
-        if (p < npx) acc.add(f, x);
-      } else if (P.do_stats) {
-        // this warp's pixels at k: T k + wlo0 + lane; flush while they pass pend
-        const int hi = min(T * k + wlo0 + 32, npx);
-        bool todo = p < npx;
-        while (hi > pend) {
-          if (todo && p < pend) {
-            acc.add(f, x);
-            todo = false;
-          }
-          flush_bin_sums(W, P.n_z, zc, acc, lane);
-          acc.zero();
-          ++zc;
-          pend = __ldg(P.bin_end + zc + 1) - jb;
-        }
-        if (todo) acc.add(f, x);
-      }
-      fb[p] = f;
-      px += sx;
-      py += sy;
-      pz += sz;
-    }
-    }
+    int cells = 0;
+    if constexpr (CELLS) cells = plan_cells<N>(C, rec, j0, npair, t, team);
 
-    // ---- P1D of the segment
-    if (P.do_stats && npx == N) {
-      const int zs = __ldg(P.segzbin + jb);
-      if (zs >= 0 && zs < P.n_z) {
-        forward_packed_fft<N>(buf, tws, t, team);
-        float pk[4];
-        power_of_modes<N>(buf, P.tw, t, pk);
-        accumulate_p1d<N>(W, P.n_k, pk, P.p1d_scale, zs, t);
-        if (t == 0) W.nseg[zs] += 1u;
+    float2 v[8];
+    int za = zs[0], zb = zs[1];
+    // Two rounds of one transform: modes to delta_S, then flux to its modes
+    // (one copy of the code: the loop over pairs has to stay within what the
+    // instruction cache holds; unrolled it stalled on fetches for a third of
+    // its time)
+#pragma unroll 1
+    for (int round = 0; round < 2; ++round) {
+      if (round == 0) {
+        // ---- small-scale field of both segments: iteration (q, h) draws the
+        // modes 2c, 2c + 1 (< N/2), c = t + q T, of segment h
+        const uint64_t id = rec->id;
+        float2 a0 = make_float2(0.f, 0.f), a1 = a0;
+#pragma unroll
+        for (int it = 0; it < 4; ++it) {
+          const int h = it & 1;
+          const uint32_t c = t + (it >> 1) * T;
+          float2 y0 = make_float2(0.f, 0.f), y1 = y0;
+          if (h == 0 || two) {
+            const float *amp = P.amp;
+            float w_hi = 0.f;
+            if constexpr (PSZ) {  // P_s at the mean z of the segment's window, linear between nodes
+              const float zw = __ldg(P.zwin + jb0 + h * N);
+              const int k = P.ps_nodes;
+              int n0 = 0;
+              while (n0 + 2 < k && zw >= P.ps_z[n0 + 1]) ++n0;
+              w_hi = fminf(fmaxf((zw - P.ps_z[n0]) / (P.ps_z[n0 + 1] - P.ps_z[n0]), 0.f), 1.f);
+              amp += n0 * (N / 2 + 1);
+            }
+            small_scale_modes<N, PSZ>(c, amp, amp + (N / 2 + 1), w_hi, static_cast<uint32_t>(s + h), id, P.seed, y0,
+                                      y1);
+          }
+          if (h == 0) {
+            a0 = y0;
+            a1 = y1;
+          } else {
+            store_mode_pair<N>(buf, c, a0, a1, y0, y1);
+          }
+        }
+        team_sync<T>(team);
+        load_modes<N>(buf, v, t);
+      }
+      team_sync<T>(team);  // the modes are read; the cells are read
+      pair_fft<N>(buf, v, tws, t, team);
+      if (round == 1) break;
+
+      // v[r].x, v[r].y: delta_S of pixel t + T r of the two segments
+      // ---- the cells' cubics, over the exchange buffer
+      if constexpr (CELLS) {
+        team_sync<T>(team);
+        for (int c = t; c < cells; c += T) expand_cell<LAYOUT>(C, c, P.box_d, P.box_e, P.lgn);
+        team_sync<T>(team);
+      }
+
+      // ---- per pixel: interpolation, growth, FGPA, stores, pixel sums.  One pass
+      // of the loop per segment, with the transform's parts swapped after each
+      // (one copy of the code)
+#pragma unroll 1
+      for (int h = 0; h < 2; ++h) {
+        const int npx = min(N, npair - h * N);
+        float f8[8];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) f8[k] = 0.f;
+        if (npx > 0) {
+          const int jb = jb0 + h * N;
+          int pend = N;  // segment pixel where bin zc ends
+          if (P.do_stats) {
+            const int z = h ? z0[1] : z0[0];
+            if (z != zc) {
+              if (zc != -2) flush_bin_sums(W, P.n_z, zc, acc, lane);
+              acc.zero();
+              zc = z;
+            }
+            pend = bin_end[zc + 1] - jb;
+          }
+          // Rows of T pixels go through the stash (a thread's own pixels: no
+          // barrier), so that the loop stays rolled; everything points at the
+          // thread's pixel of row d / T.
+          const int64_t o = offset + j0 + h * N + t;
+          const float4 *tp = P.pixtab + jb + t;
+          const uint2 *mp = C.mask + ((h * N + wlo0) >> 5);
+          float *sp = stash + t, *fp = P.flux_out + o;
+          float qf = static_cast<float>(h * N + t);
+          const int rem = npx - t, rem_flux = put_flux ? rem : 0;
+#pragma unroll
+          for (int k = 0; k < 8; ++k) sp[T * k] = v[k].x;
+          // (delta, eta) at the thread's pixel of row d / T + k
+          auto interpolate = [&](int d, int k) -> float2 {
+            if constexpr (CELLS) {
+              return eval_cell(C, mp[k * (T / 32)], qf + static_cast<float>(T * k), lanes_le);
+            } else {
+              const int q = j0 + h * N + t + d + T * k;
+              const int64_t st[3] = {rec->step[0], rec->step[1], rec->step[2]};
+              const int64_t px = rec->p0[0] + kRoundQ + q * st[0], py = rec->p0[1] + kRoundQ + q * st[1],
+                            pz = rec->p0[2] + kRoundQ + q * st[2];
+              if constexpr (INTERP == MK_INTERP_GAUSS7) {
+                static_assert(LAYOUT == MK_BOX_HALO, "the Gaussian kernel reads a halo box");
+                return gather_gauss7(P.box_d, P.lgn, px, py, pz);
+              } else {
+                return gather<LAYOUT>(P.box_d, P.box_e, P.lgn, px, py, pz, st);
+              }
+            }
+          };
+          auto flux_of = [&](float2 de, float4 tb, float ds, float2 &x) -> float {
+            x = make_float2(fmaf(tb.x, de.x, ds), tb.x * de.y);
+            return fgpa(tb, x.x, x.y);
+          };
+#pragma unroll 1
+          for (int d = 0; d + wlo0 < npx; d += kRows * T) {
+            if (INTERP == MK_INTERP_TRILINEAR && (d + (kRows - 1) * T + wlo0 + 32 <= pend || pend >= npx)) {
+              // rows inside one z bin: no branches, pixels past the segment's end
+              // are computed and masked (their cells and table entries exist);
+              // the 7^3 average is too long for a second copy
+#pragma unroll
+              for (int k = 0; k < kRows; ++k) {
+                const bool on = d + T * k < rem;
+                const float2 de = interpolate(d, k);
+                float2 x;
+                float f = flux_of(de, __ldg(tp + T * k), sp[T * k], x);
+                if (d + T * k < rem_flux) fp[T * k] = f;
+                if (put_fields && on) {
+                  P.delta_out[o + d + T * k] = x.x;
+                  P.eta_out[o + d + T * k] = x.y;
+                }
+                f = on ? f : 0.f;
+                acc.n += on ? 1.f : 0.f;
+                acc.add_sums(f, make_float2(on ? x.x : 0.f, on ? x.y : 0.f));
+                sp[T * k] = f;
+              }
+            } else {
+#pragma unroll 1
+              for (int k = 0; k < kRows; ++k) {
+                const int p = t + d + T * k;
+                float f = 0.f;
+                float2 x = make_float2(0.f, 0.f);
+                bool todo = p < npx;
+                if (todo) {
+                  const float2 de = interpolate(d, k);
+                  f = flux_of(de, __ldg(tp + T * k), sp[T * k], x);
+                  if (put_fields) {
+                    P.delta_out[o + d + T * k] = x.x;
+                    P.eta_out[o + d + T * k] = x.y;
+                  }
+                  if (put_flux) fp[T * k] = f;
+                }
+                // this warp's pixels: d + T k + wlo0 + lane; flush while they pass pend
+                const int hi = min(d + T * k + wlo0 + 32, npx);
+                while (P.do_stats && hi > pend) {
+                  if (todo && p < pend) {
+                    acc.add(f, x);
+                    todo = false;
+                  }
+                  flush_bin_sums(W, P.n_z, zc, acc, lane);
+                  acc.zero();
+                  ++zc;
+                  pend = bin_end[zc + 1] - jb;
+                }
+                if (todo) acc.add(f, x);
+                sp[T * k] = f;
+              }
+            }
+            tp += kRows * T;
+            mp += kRows * (T / 32);
+            sp += kRows * T;
+            fp += kRows * T;
+            qf += static_cast<float>(kRows * T);
+          }
+#pragma unroll
+          for (int k = 0; k < 8; ++k) f8[k] = T * k < rem ? stash[T * k + t] : 0.f;
+        }
+#pragma unroll
+        for (int k = 0; k < 8; ++k) v[k] = make_float2(v[k].y, f8[k]);
+      }
+      // ---- P1D of the full segments
+      if (!((za >= 0 && za < P.n_z) || (zb >= 0 && zb < P.n_z))) {  // (always without statistics)
+        za = -2;
+        break;
       }
     }
-    team_sync<T>(team);
+    if (za != -2) {
+      float ka[4], kb[4];
+      pair_powers<N>(buf, v, t, team, ka, kb);
+#pragma unroll 1
+      for (int h = 0; h < 2; ++h) {
+        if (za >= 0 && za < P.n_z) {
+          accumulate_p1d(W, P.n_k, bins, ka, 0.25f * P.p1d_scale, za);
+          if (t == 0) W.nseg[za] += 1u;
+        }
+        za = zb;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) ka[j] = kb[j];
+      }
+    } else {
+      team_sync<T>(team);  // the cells are read
+    }
   }
   if (P.do_stats) {
     if (zc != -2) flush_bin_sums(W, P.n_z, zc, acc, lane);
@@ -295,6 +452,7 @@ __global__ void __launch_bounds__(256, 2) k_stats(StatParams P) {
   PixelSums acc;
   acc.zero();
   int zc = -2;
+  const P1dBins bins(N / 2, P.n_k, t);
   team_sync<T>(team);
 
   for (; u < uend; ++u) {
@@ -409,7 +567,7 @@ __global__ void __launch_bounds__(256, 2) k_stats(StatParams P) {
         forward_packed_fft<N>(buf, tws, t, team);
         float pk[4];
         power_of_modes<N>(buf, P.tw, t, pk);
-        accumulate_p1d<N>(W, P.n_k, pk, P.p1d_scale, zs, t);
+        accumulate_p1d(W, P.n_k, bins, pk, P.p1d_scale, zs);
         if (t == 0) W.nseg[zs] += 1u;
       }
     }

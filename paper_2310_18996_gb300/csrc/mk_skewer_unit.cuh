@@ -14,39 +14,32 @@ namespace skewer_unit_detail {
 
 // minb: register budget of the instance, that of minb 256-thread CTAs per SM;
 // psz: P_s tables at several redshifts (one instance per layout, budget 3)
-template <int NN, int L, int INTERP, typename F>
-cudaError_t with_layout(bool big, bool psz, int minb, F &&fn) {
-  if (psz) return big ? fn(k_skewer<NN, L, true, 3, INTERP, true>) : fn(k_skewer<NN, L, false, 3, INTERP, true>);
-  if (minb >= 4) return big ? fn(k_skewer<NN, L, true, 4, INTERP>) : fn(k_skewer<NN, L, false, 4, INTERP>);
-  if (minb == 3) return big ? fn(k_skewer<NN, L, true, 3, INTERP>) : fn(k_skewer<NN, L, false, 3, INTERP>);
-  return big ? fn(k_skewer<NN, L, true, 2, INTERP>) : fn(k_skewer<NN, L, false, 2, INTERP>);
+template <int NN, int L, int INTERP, bool CELLS, typename F>
+cudaError_t with_budget(bool psz, int minb, F &&fn) {
+  if (psz) return fn(k_skewer<NN, L, 3, INTERP, true, CELLS>);
+  if (minb >= 4) return fn(k_skewer<NN, L, 4, INTERP, false, CELLS>);
+  if (minb == 3) return fn(k_skewer<NN, L, 3, INTERP, false, CELLS>);
+  return fn(k_skewer<NN, L, 2, INTERP, false, CELLS>);
 }
 
-// Side 2^kFixLgn of the box whose padded-layout strides are compile-time
-// constants in the N = 256 instances (the 1024^3 box of the batched workload);
-// other sides take the strides at run time.
-constexpr int kFixLgn = 10;
+template <int NN, int L, typename F>
+cudaError_t with_layout(bool psz, bool cells, int minb, F &&fn) {
+  if (cells) return with_budget<NN, L, MK_INTERP_TRILINEAR, true>(psz, minb, fn);
+  return psz ? fn(k_skewer<NN, L, 3, MK_INTERP_TRILINEAR, true, false>)
+             : fn(k_skewer<NN, L, 3, MK_INTERP_TRILINEAR, false, false>);
+}
 
-// Calls fn with the kernel instance for (kernel variant, box size, register budget).
+// Calls fn with the kernel instance for (kernel variant, register budget).
 template <int NN, typename F>
-cudaError_t with_skewer_kernel(int variant, int lgn, int minb, F &&fn) {
-  const bool big = lgn > 10;
-  const bool psz = (variant & kPsNodesVariant) != 0;
+cudaError_t with_skewer_kernel(int variant, int minb, F &&fn) {
+  const bool psz = (variant & kPsNodesVariant) != 0, cells = (variant & kPixelGatherVariant) == 0;
   const int layout = variant & (kGauss7Variant - 1);
-  if constexpr (NN == 256) {
-    if (variant == MK_BOX_PADDED && lgn == kFixLgn) {
-      constexpr int L = MK_BOX_PADDED, I = MK_INTERP_TRILINEAR;
-      if (minb >= 4) return fn(k_skewer<NN, L, false, 4, I, false, kFixLgn>);
-      if (minb == 3) return fn(k_skewer<NN, L, false, 3, I, false, kFixLgn>);
-      return fn(k_skewer<NN, L, false, 2, I, false, kFixLgn>);
-    }
-  }
-  if (variant & kGauss7Variant) return with_layout<NN, MK_BOX_HALO, MK_INTERP_GAUSS7>(big, psz, minb, fn);
-  if (layout == MK_BOX_HALO) return with_layout<NN, MK_BOX_HALO, MK_INTERP_TRILINEAR>(big, psz, minb, fn);
-  if (layout == MK_BOX_TENSOR) return with_layout<NN, MK_BOX_TENSOR, MK_INTERP_TRILINEAR>(big, psz, minb, fn);
-  if (layout == MK_BOX_PADDED) return with_layout<NN, MK_BOX_PADDED, MK_INTERP_TRILINEAR>(big, psz, minb, fn);
-  if (layout == MK_BOX_INTERLEAVED) return with_layout<NN, MK_BOX_INTERLEAVED, MK_INTERP_TRILINEAR>(big, psz, minb, fn);
-  return with_layout<NN, MK_BOX_PLANAR, MK_INTERP_TRILINEAR>(big, psz, minb, fn);
+  if (variant & kGauss7Variant) return with_budget<NN, MK_BOX_HALO, MK_INTERP_GAUSS7, false>(psz, minb, fn);
+  if (layout == MK_BOX_HALO) return with_layout<NN, MK_BOX_HALO>(psz, cells, minb, fn);
+  if (layout == MK_BOX_TENSOR) return with_layout<NN, MK_BOX_TENSOR>(psz, cells, minb, fn);
+  if (layout == MK_BOX_PADDED) return with_layout<NN, MK_BOX_PADDED>(psz, cells, minb, fn);
+  if (layout == MK_BOX_INTERLEAVED) return with_layout<NN, MK_BOX_INTERLEAVED>(psz, cells, minb, fn);
+  return with_layout<NN, MK_BOX_PLANAR>(psz, cells, minb, fn);
 }
 
 template <typename K>
@@ -59,15 +52,10 @@ int occupancy(K kern, int threads, size_t smem) {
 }  // namespace skewer_unit_detail
 
 template <int NN>
-size_t SkewerUnit<NN>::smem_bytes(int threads, int n_z, int n_k, bool stats) {
-  return TeamSmem<NN>::bytes(threads, n_z, n_k, stats);
-}
-
-template <int NN>
-int SkewerUnit<NN>::blocks_per_sm(int variant, int lgn, int minb, int threads, int n_z, int n_k, bool stats) {
-  const size_t smem = TeamSmem<NN>::bytes(threads, n_z, n_k, stats);
+int SkewerUnit<NN>::blocks_per_sm(int variant, int cap, int minb, int threads, int n_z, int n_k, bool stats) {
+  const size_t smem = PairSmem<NN>::bytes(threads, n_z, n_k, stats, cap);
   int b = 1;
-  skewer_unit_detail::with_skewer_kernel<NN>(variant, lgn, minb, [&](auto kern) {
+  skewer_unit_detail::with_skewer_kernel<NN>(variant, minb, [&](auto kern) {
     b = skewer_unit_detail::occupancy(kern, threads, smem);
     return cudaSuccess;
   });
@@ -77,8 +65,8 @@ int SkewerUnit<NN>::blocks_per_sm(int variant, int lgn, int minb, int threads, i
 template <int NN>
 cudaError_t SkewerUnit<NN>::launch(const SkewerParams &P, int variant, int minb, int grid, int threads,
                                    cudaStream_t st) {
-  const size_t smem = TeamSmem<NN>::bytes(threads, P.n_z, P.n_k, P.do_stats != 0);
-  return skewer_unit_detail::with_skewer_kernel<NN>(variant, P.lgn, minb, [&](auto kern) {
+  const size_t smem = PairSmem<NN>::bytes(threads, P.n_z, P.n_k, P.do_stats != 0, P.cell_cap);
+  return skewer_unit_detail::with_skewer_kernel<NN>(variant, minb, [&](auto kern) {
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
     if (e != cudaSuccess) return e;
     kern<<<grid, threads, smem, st>>>(P);

@@ -134,6 +134,7 @@ __global__ void __launch_bounds__(256, 2) k_tune_stats(StatParams P) {
   PixelSums acc;
   acc.zero();
   int zc = -2;
+  const P1dBins bins(N / 2, P.n_k, t);
 
   // describe segment uu (of skewer inext, advanced as needed); team-uniform
   auto describe = [&](int64_t uu) -> TuneSeg {
@@ -280,7 +281,7 @@ __global__ void __launch_bounds__(256, 2) k_tune_stats(StatParams P) {
         forward_packed_fft<N>(buf, tws, t, team);
         float pk[4];
         power_of_modes<N>(buf, P.tw, t, pk);
-        accumulate_p1d<N>(W, P.n_k, pk, P.p1d_scale, zs, t);
+        accumulate_p1d(W, P.n_k, bins, pk, P.p1d_scale, zs);
         if (t == 0) W.nseg[zs] += 1u;
       }
     }

@@ -1,0 +1,71 @@
+"""The fused kernel's pairs of segments and cells of a sight line against the
+oracle: skewer lengths around the ends of segments and pairs, pixel lengths on
+both sides of the rule that chooses cells or gathers per pixel, every layout."""
+import numpy as np
+import pytest
+
+import oracle
+import skewer_inputs as si
+from tests.parity_util import NTHREADS, assert_field_close, assert_flux_close, assert_stats_close, box_numpy
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+import paper_2310_18996_gb300 as mk  # noqa: E402
+
+FLAGS = mk.STATS | mk.STORE_FIELDS | mk.STORE_FLUX
+
+
+@pytest.fixture(scope="module")
+def ctx():
+    c = mk.Context(0)
+    yield c
+    c.close()
+
+
+def recipe(cell, **kw):
+    w = si.shrink(si.workload("tiny"), n_q=60, **kw)
+    half = 0.5 * w["n"] * cell
+    w.update(cell=cell, origin=(si.OBSERVER_TO_BOX_CENTRE - half, -half, -half))
+    return w
+
+
+def check(ctx, w, layout):
+    d, e = box_numpy(w)
+    pos, ids = si.catalogue(w)
+    pos[: len(pos) // 2, 1:] *= -7.0  # steep sight lines, both directions along y and z
+    o = oracle.run_skewers(w, d, e, pos, ids, n_threads=NTHREADS)
+    so = oracle.stats(w, o["j_lo"], o["offsets"], o["offsets_out"], o["flux"], o["delta"], o["eta"])
+    gd, ge = torch.from_numpy(d).cuda(), torch.from_numpy(e).cuda()
+    if layout == mk.BOX_PLANAR:
+        box = ctx.load_box(w, gd, ge)
+    else:
+        packed = ctx.pack_box(gd, ge, padded=layout == mk.BOX_PADDED, halo=layout == mk.BOX_HALO)
+        box = ctx.load_box(w, packed, None, layout=layout)
+    st, g = ctx.run(box, mk.catalogue_tensor(pos, ids), len(ids), w, flags=FLAGS)
+    tot = int(o["offsets"][-1])
+    np.testing.assert_array_equal(g["offsets"].cpu().numpy(), o["offsets"])
+    assert_field_close(g["delta"][:tot].cpu().numpy(), o["delta"], "delta_tot")
+    assert_field_close(g["eta"][:tot].cpu().numpy(), o["eta"], "eta")
+    assert_flux_close(g["flux"][:tot].cpu().numpy(), o["flux"])
+    one = so["sums"][:, 0] == 1  # one pixel has no dispersion: 0, or the root of a rounding error
+    st["sigma_f"][one] = so["sigma_f"][one]
+    assert_stats_close(st, so)
+
+
+@pytest.mark.parametrize("n_fft,n_max", [(256, n) for n in (1, 31, 255, 256, 257, 511, 512, 513, 769)] +
+                         [(512, 513), (1024, 1025), (2048, 1900)])
+def test_segment_and_pair_ends(ctx, n_fft, n_max):
+    check(ctx, recipe(si.CELL, n_fft=n_fft, n_max=n_max), mk.BOX_PADDED)
+
+
+@pytest.mark.parametrize("cell", [0.3, 1.0, 1.99, 2.0, 9.0])  # dr/cell 0.67 ... 0.1005, 0.1, 0.022
+@pytest.mark.parametrize("n_fft", [256, 2048])
+def test_pixel_lengths_on_both_sides_of_the_cell_rule(ctx, cell, n_fft):
+    check(ctx, recipe(cell, n_fft=n_fft), mk.BOX_PADDED)
+
+
+@pytest.mark.parametrize("layout", [mk.BOX_PLANAR, mk.BOX_INTERLEAVED, mk.BOX_HALO])
+@pytest.mark.parametrize("cell", [1.5, 2.0])
+def test_layouts_with_and_without_cells(ctx, layout, cell):
+    check(ctx, recipe(cell, n_fft=512, n_max=1500), layout)
