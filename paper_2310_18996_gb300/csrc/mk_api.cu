@@ -189,7 +189,8 @@ struct mk_ctx {
   size_t partials_cap = 0;  // doubles
   mk_stats_out *h_stats = nullptr;  // pinned; k_finalize writes it
   int64_t *h_total = nullptr;  // pinned
-  int skewer_threads = 256;
+  void *d_scratch = nullptr;  // ctx_scratch
+  size_t scratch_cap = 0;
   // launch configurations chosen by the autotuner, per kernel variant
   std::map<uint64_t, LaunchCfg> tuned;
   // captured graph of the last mk_run with MK_GRAPH, and what it was made from
@@ -678,6 +679,7 @@ void mk_destroy(mk_ctx *ctx) {
   cudaFree(ctx->d_segoff);
   cudaFree(ctx->d_scan_ws);
   cudaFree(ctx->d_partials);
+  cudaFree(ctx->d_scratch);
   cudaFreeHost(ctx->h_stats);
   if (ctx->graph) cudaGraphExecDestroy(ctx->graph);
   if (ctx->ev0) cudaEventDestroy(ctx->ev0);
@@ -1418,6 +1420,11 @@ cudaStream_t ctx_stream(mk_ctx *c) { return c->stream; }
 int ctx_device(mk_ctx *c) { return c->device; }
 int ctx_fail(mk_ctx *c, int code, const char *msg) { return fail(c, code, "%s", msg); }
 int ctx_sms(mk_ctx *c) { return c->sms; }
+int ctx_scratch(mk_ctx *c, size_t bytes, unsigned char **p) {
+  const int rc = grow(c, &c->d_scratch, &c->scratch_cap, bytes);
+  *p = static_cast<unsigned char *>(c->d_scratch);
+  return rc;
+}
 double ctx_z_of(mk_ctx *c, double r) { return c->cos.z_of(r); }
 double ctx_growth(mk_ctx *c, double z) { return c->cos.growth(z); }
 double ctx_distance(mk_ctx *c, double z) { return c->cos.distance(z); }
