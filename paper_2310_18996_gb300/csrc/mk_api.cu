@@ -543,8 +543,8 @@ uint64_t tune_key(int n_fft, int variant, int lgn, uint32_t flags) {
          (static_cast<uint64_t>(lgn > 10) << 8) | (flags & (MK_STORE_FIELDS | MK_STORE_FLUX | MK_STATS));
 }
 
-int stats_grid(mk_ctx *ctx, const mk_stat_bins *bins, int threads, bool tune = false) {
-  return capped(ctx, ctx->sms * stats_blocks_per_sm(bins->n_fft, threads, bins->n_z, bins->n_k, tune));
+int stats_grid(mk_ctx *ctx, const mk_stat_bins *bins, int threads) {
+  return capped(ctx, ctx->sms * stats_blocks_per_sm(bins->n_fft, threads, bins->n_z, bins->n_k));
 }
 
 GeomParams geom_params(mk_ctx *ctx, const mk_box *box, const mk_skewer_params *p) {
@@ -888,11 +888,11 @@ int stats_pass(mk_ctx *ctx, const mk_skewer_params *params, const mk_skewer *d_s
   if (nodes && (rc = ensure_pixtab(ctx, nodes))) return rc;
   const int threads = 256;
   const StatLayout L{bins->n_z, bins->n_k};
-  const int grid = stats_grid(ctx, bins, threads, tune_kernel(nodes ? ctx->d_pixtab : nullptr, d_delta, d_eta, rebin));
+  const int grid = stats_grid(ctx, bins, threads);
   if ((rc = grow(ctx, reinterpret_cast<void **>(&ctx->d_partials), &ctx->partials_cap,
                  sizeof(double) * static_cast<size_t>(grid) * L.size())))
     return rc;
-  if (n_sk > 0) CK(launch_seg_counts(d_offsets_out, n_sk, bins->n_fft, ctx->d_cnt_seg, ctx->stream));
+  if (n_sk > 0) CK(launch_seg_counts(d_offsets_out, n_sk, 2 * bins->n_fft, ctx->d_cnt_seg, ctx->stream));
   CK(launch_scan(ctx->d_cnt_seg, nullptr, n_sk, ctx->d_segoff, nullptr, nullptr, ctx->d_scan_ws, ctx->stream));
   StatParams P{};
   P.sk = d_sk;
@@ -1384,7 +1384,7 @@ extern "C" int mk_stats_static(mk_ctx *ctx, const mk_skewer_params *params, cons
   if (grid < 1) return fail(ctx, MK_EINVAL, "binning too large for the static scratch");
 
   // every piece below is fully rewritten by this call, so nothing is cleared
-  if (n_sk > 0) CK(launch_seg_counts(d_offsets_out, n_sk, bins->n_fft, d_cnt, ctx->stream));
+  if (n_sk > 0) CK(launch_seg_counts(d_offsets_out, n_sk, 2 * bins->n_fft, d_cnt, ctx->stream));
   CK(launch_scan(d_cnt, nullptr, n_sk, d_seg, nullptr, nullptr, d_tiles, ctx->stream));
   StatParams P{};
   P.sk = d_sk;

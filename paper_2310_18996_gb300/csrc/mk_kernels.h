@@ -41,13 +41,13 @@ cudaError_t launch_bin_end(const int16_t *zbin, int32_t j_max, int n_z, int32_t 
 cudaError_t launch_out_counts(const mk_skewer *sk, int64_t n, int rebin, int64_t *cnt, cudaStream_t st);
 cudaError_t launch_seg_counts(const int64_t *off, int64_t n, int n_fft, int64_t *cnt, cudaStream_t st);
 int skewer_blocks_per_sm(int n_fft, int variant, int cap, int minb, int threads, int n_z, int n_k, bool stats);
-// The tuning pass (FGPA table set, rebin 1, 16-byte aligned fields) runs the
-// staged kernel k_tune_stats; every other statistics pass runs k_stats.
-inline bool tune_kernel(const void *pixtab, const float *delta, const float *eta, int rebin) {
+// Whether a statistics pass is a tuning pass whose fields can be staged with
+// bulk copies (FGPA table set, rebin 1, 16-byte aligned fields).
+inline bool staged_pass(const void *pixtab, const float *delta, const float *eta, int rebin) {
   return pixtab && delta && eta && rebin == 1 &&
          ((reinterpret_cast<uintptr_t>(delta) | reinterpret_cast<uintptr_t>(eta)) & 15) == 0;
 }
-int stats_blocks_per_sm(int n_fft, int threads, int n_z, int n_k, bool tune);
+int stats_blocks_per_sm(int n_fft, int threads, int n_z, int n_k);
 // variant: box layout, plus kGauss7Variant for the Gaussian-kernel interpolation,
 // plus kPsNodesVariant for z-dependent P_s (built for register budget 3 only),
 // plus kPixelGatherVariant (budget 3 only); cap: cells of a run (P.cell_cap);
@@ -62,7 +62,7 @@ template <int N>
 struct SkewerUnit {
   static int blocks_per_sm(int variant, int cap, int minb, int threads, int n_z, int n_k, bool stats);
   static cudaError_t launch(const SkewerParams &P, int variant, int minb, int grid, int threads, cudaStream_t st);
-  static int stats_blocks_per_sm(int threads, int n_z, int n_k, bool tune);
+  static int stats_blocks_per_sm(int threads, int n_z, int n_k);
   static cudaError_t launch_stats(const StatParams &P, int grid, int threads, cudaStream_t st);
 };
 extern template struct SkewerUnit<256>;

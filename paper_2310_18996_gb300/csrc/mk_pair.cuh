@@ -27,11 +27,14 @@ struct PairFft {
   static constexpr int BUF = N + N / 8;
   // twiddles (forward sign), shared by the CTA's teams: pass 1 (7 x 8 entries,
   // e^{-2 pi i r j / 64}), pass 2 (7 x 64 entries, e^{-2 pi i r j / 512}, P8 = 3),
-  // last pass (slot (i, q), i < 8 / F, q = 1..F-1: e^{-2 pi i q (t + T i) / N}, T entries each)
+  // last pass (slot (i, q), i < 8 / F, q = 1..F-1: e^{-2 pi i q (t + T i) / N}, T
+  // entries each; at N = 2048 these 12 KB would cost a CTA per SM, and the pass
+  // reads the global table)
+  static constexpr bool kGlobalLast = N == 2048;
   static constexpr int TW1 = 0;
   static constexpr int TW2 = 56;
   static constexpr int TWF = P8 == 3 ? TW2 + 7 * 64 : TW2;
-  static constexpr int TWN = TWF + (8 / F) * (F - 1) * T;
+  static constexpr int TWN = TWF + (kGlobalLast ? 0 : (8 / F) * (F - 1) * T);
   static constexpr size_t TW_BYTES = sizeof(float2) * TWN;
 };
 
@@ -79,7 +82,8 @@ __device__ __forceinline__ void dft8(float2 (&v)[8]) {
 // after pass 1, plain after pass 2: every access is a lane base plus a
 // compile-time offset and its half warps hit 16 distinct 8-byte slots.
 template <int N>
-__device__ __forceinline__ void pair_fft(float2 *buf, float2 (&v)[8], const float2 *tws, int t, int team) {
+__device__ __forceinline__ void pair_fft(float2 *buf, float2 (&v)[8], const float2 *tws,
+                                         const float2 *__restrict__ tab, int t, int team) {
   using P = PairFft<N>;
   constexpr int T = P::T;
   dft8(v);
@@ -146,7 +150,7 @@ __device__ __forceinline__ void pair_fft(float2 *buf, float2 (&v)[8], const floa
     for (int i = 0; i < 2; ++i) {
 #pragma unroll
       for (int q = 1; q < 4; ++q) {
-        const float2 w = tws[P::TWF + (3 * i + q - 1) * T + t];
+        const float2 w = P::kGlobalLast ? __ldg(tab + q * (t + T * i)) : tws[P::TWF + (3 * i + q - 1) * T + t];
         v[i + 2 * q] = cmul(v[i + 2 * q], w);
       }
       dft4<-1>(v[i], v[i + 2], v[i + 4], v[i + 6]);

@@ -128,7 +128,7 @@ inline int cell_capacity(int n, double dr_over_cell) {
 struct StatParams {
   const mk_skewer *sk;
   const int64_t *off_out;  // output offsets, n_sk + 1
-  const int64_t *segoff;   // prefix of ceil(n_out / N) per skewer
+  const int64_t *segoff;   // prefix of pairs of segments, ceil(n_out / 2N) per skewer
   int64_t n_sk;
   const float *flux;         // stored flux, or NULL with pixtab set
   const float *delta, *eta;  // fine fields or NULL

@@ -1,5 +1,6 @@
-// Templates of the fused skewer kernel and the statistics kernel; each FFT
-// length is instantiated in its own translation unit (mk_skewer_<N>.cu).
+// Template of the fused skewer kernel and what it shares with the statistics
+// kernels (mk_stats.cuh); each FFT length is instantiated in its own translation
+// unit (mk_skewer_<N>.cu).
 #pragma once
 
 #include "mk_pair.cuh"
@@ -7,20 +8,9 @@
 namespace mk {
 
 // =================================================================== shared-memory plan
-// Statistics kernels, per CTA: per-warp statistic accumulators, the twiddle
-// table, then one FFT buffer of N/2 + 2 complex values per team.
-template <int N>
-struct TeamSmem {
-  static constexpr int T = N / 8;
-  static constexpr int BUF = N == 256 ? kBuf256 : N / 2 + 2;  // complex slots per team buffer
-  __host__ __device__ static size_t acc_bytes(int threads, int n_z, int n_k, bool stats) {
-    return stats ? static_cast<size_t>(threads / 32) * WarpAcc::bytes(n_z, n_k) : 0;
-  }
-  __host__ __device__ static size_t bytes(int threads, int n_z, int n_k, bool stats) {
-    return acc_bytes(threads, n_z, n_k, stats) + TwTab<N>::BYTES +
-           static_cast<size_t>(threads / T) * BUF * sizeof(float2);
-  }
-};
+__host__ __device__ inline size_t acc_bytes(int threads, int n_z, int n_k, bool stats) {
+  return stats ? static_cast<size_t>(threads / 32) * WarpAcc::bytes(n_z, n_k) : 0;
+}
 
 // Fused kernel, per CTA: per-warp accumulators (when statistics are on), the
 // twiddles, the ends of the z bins, then per team one area that is the FFT's
@@ -42,7 +32,7 @@ struct PairSmem {
            (cap > 0 ? CellPlan::kLineBytes + sizeof(uint2) * (N / 16) + sizeof(float) * cap : 0);
   }
   __host__ __device__ static size_t bytes(int threads, int n_z, int n_k, bool stats, int cap) {
-    return TeamSmem<N>::acc_bytes(threads, n_z, n_k, stats) + HEAD + static_cast<size_t>(threads / T) * team_bytes(cap);
+    return acc_bytes(threads, n_z, n_k, stats) + HEAD + static_cast<size_t>(threads / T) * team_bytes(cap);
   }
 };
 
@@ -257,7 +247,7 @@ __global__ void __launch_bounds__(256, MINB) k_skewer(SkewerParams P) {
         load_modes<N>(buf, v, t);
       }
       team_sync<T>(team);  // the modes are read; the cells are read
-      pair_fft<N>(buf, v, tws, t, team);
+      pair_fft<N>(buf, v, tws, P.tw, t, team);
       if (round == 1) break;
 
       // v[r].x, v[r].y: delta_S of pixel t + T r of the two segments
@@ -414,167 +404,6 @@ __global__ void __launch_bounds__(256, MINB) k_skewer(SkewerParams P) {
     if (zc != -2) flush_bin_sums(W, P.n_z, zc, acc, lane);
     flush_warp_partials(smem, nwarps, wbytes, P.n_z, P.n_k, P.partials);
   }
-}
-
-// =================================================================== statistics kernel
-// Statistics of output pixels of R = P.rebin fine pixels: of stored flux, or
-// (rebin 1, pixtab set) of the FGPA of stored fields.  The pixel sums stay in
-// registers across segments while the warp's pixels stay in one z bin and are
-// flushed at the bin's end, as in k_skewer; an output pixel's z bin comes from
-// the tables of mean z over R pixels (zbin, bin_end) for every R.  (With R > 1
-// the bin once came from an FP64 division per pixel, and this GPU's FP64 pipe
-// was the bound: flux and statistics of 1.4e8 fine pixels at R = 3 took 3.28 ms
-// then and 1.19 ms with the tables.)
-template <int N>
-__global__ void __launch_bounds__(256, 2) k_stats(StatParams P) {
-  constexpr int T = N / 8;
-  constexpr int BUF = TeamSmem<N>::BUF;
-  const int teams = blockDim.x / T;
-  const int team = threadIdx.x / T, t = threadIdx.x % T, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int nwarps = blockDim.x >> 5;
-  extern __shared__ __align__(16) unsigned char smem[];
-  const size_t wbytes = WarpAcc::bytes(P.n_z, P.n_k);
-  float2 *tws = reinterpret_cast<float2 *>(smem + nwarps * wbytes);
-  float2 *buf = tws + TwTab<N>::SLOTS * T + team * BUF;
-  float *fb = reinterpret_cast<float *>(buf);
-  const WarpAcc W = WarpAcc::at(smem + warp * wbytes, P.n_z, P.n_k);
-  zero_warp_acc(smem + warp * wbytes, wbytes);
-  fill_twiddles<N>(tws, P.tw);
-
-  const int64_t nunits = P.segoff[P.n_sk];
-  const int64_t g = static_cast<int64_t>(blockIdx.x) * teams + team;
-  const int64_t G = static_cast<int64_t>(gridDim.x) * teams;
-  int64_t u = g * nunits / G;
-  const int64_t uend = (g + 1) * nunits / G;
-  int64_t i = u < uend ? upper_index(P.segoff, P.n_sk, u) : 0;
-  const int R = P.rebin;
-  const int wlo0 = t & ~31;  // first team pixel of this warp
-  PixelSums acc;
-  acc.zero();
-  int zc = -2;
-  const P1dBins bins(N / 2, P.n_k, t);
-  team_sync<T>(team);
-
-  for (; u < uend; ++u) {
-    while (P.segoff[i + 1] <= u) ++i;
-    const int s = static_cast<int>(u - P.segoff[i]);
-    const mk_skewer sk = P.sk[i];
-    const int64_t o = P.off_out[i];
-    const int64_t nout = P.off_out[i + 1] - o;
-    // records made for another pixel length may run past the pixel tables
-    // (team-uniform: the whole team skips the segment)
-    if (sk.j_lo < 0 || sk.j_lo + nout * R > P.j_max) {
-      if (t == 0) raise_error(P.err, ERR_RANGE);
-      continue;
-    }
-    const int64_t k0 = static_cast<int64_t>(s) * N;
-    const int npx = static_cast<int>(min(static_cast<int64_t>(N), nout - k0));
-    const int jb = sk.j_lo + static_cast<int>(k0 * R);
-    const int zs0 = __ldg(P.zbin + jb);
-    if (zs0 != zc) {
-      if (zc != -2) flush_bin_sums(W, P.n_z, zc, acc, lane);
-      acc.zero();
-      zc = zs0;
-    }
-    // segment pixel where bin zc ends
-    auto bin_stop = [&]() -> int {
-      const int d = __ldg(P.bin_end + zc + 1) - jb;
-      return R == 1 ? d : (d + R - 1) / R;
-    };
-    int pend = bin_stop();
-    // warp-uniform: this warp's pixels of the segment all lie before pend
-    const bool one_bin = min(T * 7 + wlo0 + 32, npx) <= pend;
-    // issue every load of the thread's 8 pixels before any use
-    float dv[8], ev[8], fv[8];
-    float4 tb[8];
-#pragma unroll
-    for (int q = 0; q < 8; ++q) {
-      const int p = t + T * q;
-      const bool ok = p < npx;
-      const int64_t kk = k0 + (ok ? p : 0);
-      dv[q] = ev[q] = 0.f;
-      if (R == 1 && ok && P.delta) {
-        dv[q] = __ldg(P.delta + sk.offset + kk);
-        ev[q] = __ldg(P.eta + sk.offset + kk);
-      }
-      if (P.pixtab) {
-        tb[q] = __ldg(P.pixtab + sk.j_lo + kk);
-        fv[q] = 0.f;
-      } else {
-        fv[q] = ok ? __ldg(P.flux + o + kk) : 0.f;
-      }
-    }
-    if (R > 1 && P.delta) {  // the mean of R fine pixels; fine pixel r of all 8 at a time
-      const float *dp = P.delta + sk.offset + k0 * R, *ep = P.eta + sk.offset + k0 * R;
-#pragma unroll 2
-      for (int r = 0; r < R; ++r) {
-#pragma unroll
-        for (int q = 0; q < 8; ++q) {
-          const int p = t + T * q;
-          if (p < npx) {
-            dv[q] += __ldg(dp + p * R + r);
-            ev[q] += __ldg(ep + p * R + r);
-          }
-        }
-      }
-      const float fr = static_cast<float>(R);
-#pragma unroll
-      for (int q = 0; q < 8; ++q) {
-        dv[q] /= fr;
-        ev[q] /= fr;
-      }
-    }
-    if (npx == N && one_bin) {
-      // a full segment inside one z bin: no bounds or bin checks
-#pragma unroll
-      for (int q = 0; q < 8; ++q) {
-        const float f = P.pixtab ? fgpa(tb[q], dv[q], ev[q]) : fv[q];
-        acc.add_sums(f, make_float2(dv[q], ev[q]));
-        fb[t + T * q] = f;
-      }
-      acc.n += 8.f;
-    } else {
-#pragma unroll
-      for (int q = 0; q < 8; ++q) {
-        const int p = t + T * q;
-        float f = 0.f;
-        if (p < npx) f = P.pixtab ? fgpa(tb[q], dv[q], ev[q]) : fv[q];
-        const float2 x = make_float2(dv[q], ev[q]);
-        if (one_bin) {
-          if (p < npx) acc.add(f, x);
-        } else {
-          // this warp's pixels at q: T q + wlo0 + lane; flush while they pass pend
-          const int hi = min(T * q + wlo0 + 32, npx);
-          bool todo = p < npx;
-          while (hi > pend) {
-            if (todo && p < pend) {
-              acc.add(f, x);
-              todo = false;
-            }
-            flush_bin_sums(W, P.n_z, zc, acc, lane);
-            acc.zero();
-            ++zc;
-            pend = bin_stop();
-          }
-          if (todo) acc.add(f, x);
-        }
-        fb[p] = f;
-      }
-    }
-    if (npx == N) {
-      const int zs = __ldg(P.segzbin + jb);
-      if (zs >= 0 && zs < P.n_z) {
-        forward_packed_fft<N>(buf, tws, t, team);
-        float pk[4];
-        power_of_modes<N>(buf, P.tw, t, pk);
-        accumulate_p1d(W, P.n_k, bins, pk, P.p1d_scale, zs);
-        if (t == 0) W.nseg[zs] += 1u;
-      }
-    }
-    team_sync<T>(team);
-  }
-  if (zc != -2) flush_bin_sums(W, P.n_z, zc, acc, lane);
-  flush_warp_partials(smem, nwarps, wbytes, P.n_z, P.n_k, P.partials);
 }
 
 }  // namespace mk

@@ -6,7 +6,7 @@
 
 #include "mk_kernels.h"
 #include "mk_skewer.cuh"
-#include "mk_tune_stats.cuh"
+#include "mk_stats.cuh"
 
 namespace mk {
 
@@ -74,27 +74,25 @@ cudaError_t SkewerUnit<NN>::launch(const SkewerParams &P, int variant, int minb,
   });
 }
 
+// The same for both variants, which then agree bit for bit.
 template <int NN>
-int SkewerUnit<NN>::stats_blocks_per_sm(int threads, int n_z, int n_k, bool tune) {
-  if (tune) return skewer_unit_detail::occupancy(k_tune_stats<NN>, threads, TuneSmem<NN>::bytes(threads, n_z, n_k));
-  return skewer_unit_detail::occupancy(k_stats<NN>, threads, TeamSmem<NN>::bytes(threads, n_z, n_k, true));
+int SkewerUnit<NN>::stats_blocks_per_sm(int threads, int n_z, int n_k) {
+  const int a = skewer_unit_detail::occupancy(k_stats<NN, true>, threads, StatSmem<NN, true>::bytes(threads, n_z, n_k));
+  const int b = skewer_unit_detail::occupancy(k_stats<NN, false>, threads, StatSmem<NN, false>::bytes(threads, n_z, n_k));
+  return a < b ? a : b;
 }
 
 template <int NN>
 cudaError_t SkewerUnit<NN>::launch_stats(const StatParams &P, int grid, int threads, cudaStream_t st) {
-  if (tune_kernel(P.pixtab, P.delta, P.eta, P.rebin)) {
-    const size_t smem = TuneSmem<NN>::bytes(threads, P.n_z, P.n_k);
-    cudaError_t e =
-        cudaFuncSetAttribute(k_tune_stats<NN>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+  auto run = [&](auto kern, size_t smem) {
+    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
     if (e != cudaSuccess) return e;
-    k_tune_stats<NN><<<grid, threads, smem, st>>>(P);
+    kern<<<grid, threads, smem, st>>>(P);
     return cudaGetLastError();
-  }
-  const size_t smem = TeamSmem<NN>::bytes(threads, P.n_z, P.n_k, true);
-  cudaError_t e = cudaFuncSetAttribute(k_stats<NN>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
-  if (e != cudaSuccess) return e;
-  k_stats<NN><<<grid, threads, smem, st>>>(P);
-  return cudaGetLastError();
+  };
+  if (staged_pass(P.pixtab, P.delta, P.eta, P.rebin))
+    return run(k_stats<NN, true>, StatSmem<NN, true>::bytes(threads, P.n_z, P.n_k));
+  return run(k_stats<NN, false>, StatSmem<NN, false>::bytes(threads, P.n_z, P.n_k));
 }
 
 }  // namespace mk

@@ -69,3 +69,27 @@ def test_pixel_lengths_on_both_sides_of_the_cell_rule(ctx, cell, n_fft):
 @pytest.mark.parametrize("cell", [1.5, 2.0])
 def test_layouts_with_and_without_cells(ctx, layout, cell):
     check(ctx, recipe(cell, n_fft=512, n_max=1500), layout)
+
+
+@pytest.mark.parametrize("n_fft,n_max,rebin", [(256, n, 1) for n in (255, 256, 257, 512, 513, 769)] +
+                         [(512, 1025, 1), (2048, 1900, 1), (256, 514, 2), (256, 1500, 5), (512, 1537, 3)])
+def test_statistics_at_pair_ends(ctx, n_fft, n_max, rebin):
+    """Statistics of stored flux at any rebin, and the tuning pass with its
+    fields staged and not, at lengths around the ends of segments and pairs."""
+    w = recipe(si.CELL, n_fft=n_fft, n_max=n_max)
+    d, e = box_numpy(w)
+    pos, ids = si.catalogue(w)
+    n = len(ids)
+    o = oracle.run_skewers(w, d, e, pos, ids, rebin=rebin, n_threads=NTHREADS)
+    so = oracle.stats(w, o["j_lo"], o["offsets"], o["offsets_out"], o["flux"], o["delta"], o["eta"], rebin=rebin)
+    box = ctx.load_box(w, torch.from_numpy(d).cuda(), torch.from_numpy(e).cuda())
+    r = ctx.make_skewers(box, mk.catalogue_tensor(pos, ids), n, w)
+    f, off = ctx.flux(w, r["sk"], n, r["delta"], r["eta"], rebin=rebin)
+    st = ctx.stats(w, r["sk"], n, off, f, rebin=rebin, delta=r["delta"], eta=r["eta"])
+    assert_stats_close(st, so)
+    if rebin == 1:
+        odd = [torch.cat([torch.zeros(1, device="cuda"), x])[1:] for x in (r["delta"], r["eta"])]
+        for x in ((r["delta"], r["eta"]), odd):
+            tp = ctx.flux_stats(w, r["sk"], n, r["offsets"], *x)
+            for k in ("sums", "p1d_sum", "n_seg"):
+                np.testing.assert_array_equal(tp[k], st[k])
