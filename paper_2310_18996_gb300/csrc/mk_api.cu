@@ -1530,6 +1530,15 @@ extern "C" int mk_synth_box(mk_ctx *ctx, int32_t n, double cell, uint64_t seed, 
   P.lgn = lgn;
   const bool in_place = layout == MK_BOX_INTERLEAVED && d_out == d_work;
   P.out = in_place ? nullptr : d_out;
+  // The work box is kept in bricks of 64^3 values, one per 2 MB page: a line
+  // then touches n/64 pages along every axis, where rows of a plain box put each
+  // element of a z line on a page of its own and the z pass waited for the
+  // TLBs.  (In place of the output the box has to be plain.)
+  const int64_t m = n / 64, brick = 64 * 64 * 64;
+  P.ax = BoxAxis{1, in_place ? 64 : brick};
+  P.ay = BoxAxis{in_place ? n : 64, in_place ? 64 * static_cast<int64_t>(n) : m * brick};
+  P.az = BoxAxis{in_place ? static_cast<int64_t>(n) * n : 64 * 64,
+                 in_place ? 64 * static_cast<int64_t>(n) * n : m * m * brick};
   P.out_side = side;
   P.out_margin = margin;
   P.out_stride = stride;
@@ -1537,19 +1546,11 @@ extern "C" int mk_synth_box(mk_ctx *ctx, int32_t n, double cell, uint64_t seed, 
     P.pair = p;
     P.out_slot = 2 * p;
     if (p == 0) {
-      P.axis = 0;
-      CK(launch_box_pass(P, kBoxNoiseX, ctx->sms, ctx->stream));
-      P.axis = 1;
-      CK(launch_box_pass(P, kBoxFwd, ctx->sms, ctx->stream));
-      P.axis = 2;
-      CK(launch_box_pass(P, kBoxShapeZ, ctx->sms, ctx->stream));
+      for (const int mode : {kBoxNoiseX, kBoxFwd, kBoxShapeZ}) CK(launch_box_pass(P, mode, ctx->sms, ctx->stream));
     } else {
-      P.axis = 2;
       CK(launch_box_pass(P, kBoxSpecZ, ctx->sms, ctx->stream));
     }
-    P.axis = 1;
     CK(launch_box_pass(P, kBoxInv, ctx->sms, ctx->stream));
-    P.axis = 0;
     CK(launch_box_pass(P, kBoxInvXOut, ctx->sms, ctx->stream));
   }
   return MK_OK;

@@ -71,12 +71,16 @@ extern template struct SkewerUnit<1024>;
 extern template struct SkewerUnit<2048>;
 cudaError_t launch_flux(const FluxParams &P, int sms, cudaStream_t st);
 cudaError_t launch_stats(const StatParams &P, int n_fft, int grid, int threads, cudaStream_t st);
-// One pass of the box synthesis: batched line FFTs of an n^3 complex box
-// ([z][y][x], x fastest) along one axis, with the pass's extra step (noise,
-// mode filter or output layout).
+// One pass of the box synthesis: batched line FFTs along one axis, with the
+// pass's extra step (noise, mode filter or output layout).
+// Coordinate c of an axis of the work box sits at (c mod 64) lo + (c / 64) hi.
+struct BoxAxis {
+  int64_t lo, hi;
+};
 struct BoxPassParams {
-  float2 *work;          // n^3, transformed in place
-  float2 *spec;          // n^3 delta modes (kept for further filter pairs) or NULL
+  float2 *work;          // n^3: along x the modes kx < n/2 of one field, then those of the other
+  float2 *spec;          // the filtered noise modes, in the places of the first field's (kept for further pairs) or NULL
+  BoxAxis ax, ay, az;    // of work and spec
   const float2 *tw;      // e^{-2 pi i k / 2n}, k < 2n
   const float *pk;       // P(k) at k = i dk, i < n_pk
   int32_t n_pk;
@@ -85,7 +89,6 @@ struct BoxPassParams {
   float amp;             // 1 / (cell^{3/2} n^3): sqrt(P / cell^3) and the inverse 1/n^3
   uint32_t key0, key1;   // Philox key of the white noise
   int32_t pair;          // filter pair 0..3: (1, eta_xx), (eta_yy, eta_zz), (eta_xy, eta_xz), (eta_yz, 0)
-  int32_t axis;          // 0 x, 1 y, 2 z
   int32_t lgn;
   float *out;            // output layout (last pass) or NULL
   int32_t out_side, out_margin, out_stride, out_slot;
@@ -94,10 +97,10 @@ struct BoxPassParams {
 // Box synthesis passes (mk_box.cu), modes in the order they run:
 enum BoxPass : int {
   kBoxNoiseX = 0,  // white noise, forward FFT along x
-  kBoxFwd = 1,     // forward FFT along P.axis
-  kBoxShapeZ = 2,  // forward FFT along z, filter (delta modes to spec if set), inverse along z
-  kBoxSpecZ = 3,   // delta modes from spec, filter, inverse FFT along z
-  kBoxInv = 4,     // inverse FFT along P.axis
+  kBoxFwd = 1,     // forward FFT along y
+  kBoxShapeZ = 2,  // forward FFT along z, filter (delta modes to spec if set), inverse along z of both fields
+  kBoxSpecZ = 3,   // delta modes from spec, filter, inverse FFT along z of both fields
+  kBoxInv = 4,     // inverse FFT along y of both fields
   kBoxInvXOut = 5  // inverse FFT along x, lines written into the output layout (or in place)
 };
 cudaError_t launch_box_pass(const BoxPassParams &P, int mode, int sms, cudaStream_t st);
