@@ -99,9 +99,10 @@ __device__ __forceinline__ void flush_warp_partials(unsigned char *smem, int nwa
 // ran 10 to 50 % slower, stalled on fetches.
 //
 // CELLS: the trilinear interpolant from the cubics of the line's cells (needs
-// P.cell_cap); otherwise each pixel gathers for itself: INTERP ==
-// MK_INTERP_GAUSS7 (LAYOUT must be MK_BOX_HALO), or trilinear with pixels too
-// long for the cells to pay (see use_cells).
+// P.cell_cap).  Otherwise INTERP == MK_INTERP_GAUSS7 (LAYOUT must be
+// MK_BOX_HALO): the averages of a segment are computed ahead of its pixel loop
+// into the exchange buffer (gauss7_run); or trilinear with pixels too long for
+// the cells to pay (see use_cells), each pixel gathering for itself.
 // PSZ: P_s given at several redshifts (P.ps_nodes >= 2), interpolated per segment
 template <int N, int LAYOUT, int MINB, int INTERP, bool PSZ, bool CELLS>
 __global__ void __launch_bounds__(256, MINB) k_skewer(SkewerParams P) {
@@ -264,6 +265,14 @@ __global__ void __launch_bounds__(256, MINB) k_skewer(SkewerParams P) {
 #pragma unroll 1
       for (int h = 0; h < 2; ++h) {
         const int npx = min(N, npair - h * N);
+        if constexpr (INTERP == MK_INTERP_GAUSS7) {  // (delta, eta) of the segment, over the exchange buffer
+          static_assert(LAYOUT == MK_BOX_HALO, "the Gaussian kernel reads a halo box");
+          team_sync<T>(team);
+          if (npx > 0)
+            gauss7_run(buf, reinterpret_cast<uint16_t *>(stash + 8 * wlo0), P.box_d, P.lgn, rec, j0 + h * N, npx, t >> 5,
+                       T / 32, lane);
+          team_sync<T>(team);
+        }
         float f8[8];
 #pragma unroll
         for (int k = 0; k < 8; ++k) f8[k] = 0.f;
@@ -294,17 +303,14 @@ __global__ void __launch_bounds__(256, MINB) k_skewer(SkewerParams P) {
           auto interpolate = [&](int d, int k) -> float2 {
             if constexpr (CELLS) {
               return eval_cell(C, mp[k * (T / 32)], qf + static_cast<float>(T * k), lanes_le);
+            } else if constexpr (INTERP == MK_INTERP_GAUSS7) {
+              return buf[t + d + T * k];
             } else {
               const int q = j0 + h * N + t + d + T * k;
               const int64_t st[3] = {rec->step[0], rec->step[1], rec->step[2]};
               const int64_t px = rec->p0[0] + kRoundQ + q * st[0], py = rec->p0[1] + kRoundQ + q * st[1],
                             pz = rec->p0[2] + kRoundQ + q * st[2];
-              if constexpr (INTERP == MK_INTERP_GAUSS7) {
-                static_assert(LAYOUT == MK_BOX_HALO, "the Gaussian kernel reads a halo box");
-                return gather_gauss7(P.box_d, P.lgn, px, py, pz);
-              } else {
-                return gather<LAYOUT>(P.box_d, P.box_e, P.lgn, px, py, pz, st);
-              }
+              return gather<LAYOUT>(P.box_d, P.box_e, P.lgn, px, py, pz, st);
             }
           };
           auto flux_of = [&](float2 de, float4 tb, float ds, float2 &x) -> float {
@@ -313,10 +319,9 @@ __global__ void __launch_bounds__(256, MINB) k_skewer(SkewerParams P) {
           };
 #pragma unroll 1
           for (int d = 0; d + wlo0 < npx; d += kRows * T) {
-            if (INTERP == MK_INTERP_TRILINEAR && (d + (kRows - 1) * T + wlo0 + 32 <= pend || pend >= npx)) {
+            if (d + (kRows - 1) * T + wlo0 + 32 <= pend || pend >= npx) {
               // rows inside one z bin: no branches, pixels past the segment's end
-              // are computed and masked (their cells and table entries exist);
-              // the 7^3 average is too long for a second copy
+              // are computed and masked (their cells and table entries exist)
 #pragma unroll
               for (int k = 0; k < kRows; ++k) {
                 const bool on = d + T * k < rem;

@@ -93,3 +93,11 @@ def test_statistics_at_pair_ends(ctx, n_fft, n_max, rebin):
             tp = ctx.flux_stats(w, r["sk"], n, r["offsets"], *x)
             for k in ("sums", "p1d_sum", "n_seg"):
                 np.testing.assert_array_equal(tp[k], st[k])
+
+
+@pytest.mark.parametrize("n_fft,n_max,cell", [(256, n, 9.0) for n in (1, 3, 5, 255, 257, 769)] +
+                         [(256, 1500, c) for c in (0.3, 2.0)] + [(1024, 742, 2.0), (2048, 1900, 0.3), (2048, 7, 2.0)])
+def test_gaussian_kernel_runs(ctx, n_fft, n_max, cell):
+    """Runs of pixels in one voxel: of one pixel (a voxel a pixel) to many, cut
+    by the ends of segments, with fewer runs than warps and more than lanes."""
+    check(ctx, recipe(cell, n_fft=n_fft, n_max=n_max, interp=mk.INTERP_GAUSS7), mk.BOX_HALO)
