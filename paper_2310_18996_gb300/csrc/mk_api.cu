@@ -550,16 +550,16 @@ int stats_grid(mk_ctx *ctx, const mk_stat_bins *bins, int threads) {
 GeomParams geom_params(mk_ctx *ctx, const mk_box *box, const mk_skewer_params *p) {
   GeomParams G;
   std::memset(&G, 0, sizeof(G));
-  G.tab = DcTable{ctx->d_dc, ctx->n_dc, kDcStep, ctx->cosmo.omega_m, ctx->d_zr, ctx->n_zr, 1.0 / kZrStep};
+  G.tab = DcTable{ctx->d_dc, ctx->n_dc, kDcStep, 1.0 / kDcStep, ctx->cosmo.omega_m, ctx->d_zr, ctx->n_zr, 1.0 / kZrStep};
   G.lambda_lya = ctx->cosmo.lambda_lya;
   G.dr = p->dr;
   G.lrf_min = p->lrf_min;
   G.lrf_max = p->lrf_max;
-  G.lobs_min = p->lobs_min;
+  G.z_obs_min = p->lobs_min > 0.0 ? std::max(p->lobs_min / ctx->cosmo.lambda_lya - 1.0, 0.0) : 0.0;
   G.n_min = p->n_min;
   G.n_max = p->n_max;
   for (int d = 0; d < 3; ++d) G.origin[d] = box->desc.origin[d];
-  G.cell = box->desc.cell;
+  G.inv_cell = 1.0 / box->desc.cell;
   G.j_max = ctx->j_max;
   G.unit_px = 2 * p->n_fft;
   return G;

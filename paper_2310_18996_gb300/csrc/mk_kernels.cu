@@ -1,4 +1,5 @@
 // Kernels of the skewer-synthesis path (sm_103a) and their host launchers.
+#include <cooperative_groups.h>
 #include <cuda_runtime.h>
 
 #include <cmath>
@@ -8,11 +9,12 @@
 #include "mk_kernels.h"
 
 namespace mk {
+namespace cg = cooperative_groups;
 
 // =================================================================== geometry
 // D_C(z) by cubic Hermite interpolation of the FP64 table (values + slopes).
 __device__ __forceinline__ double dc_eval(const DcTable &T, double z) {
-  double s = z / T.h;
+  const double s = z * T.inv_h;  // (h is a power of two: exact)
   int i = static_cast<int>(floor(s));
   i = max(0, min(i, T.n - 2));
   const double t = s - i;
@@ -23,21 +25,29 @@ __device__ __forceinline__ double dc_eval(const DcTable &T, double z) {
 }
 
 // z(r): linear interpolation in the z(r) table (error ~1e-7), then two
-// Newton steps on the Hermite D_C, dz = (D_C(z) - r) E(z) H0/c.
+// Newton steps on the Hermite D_C, dz = (D_C(z) - r) E(z) H0/c.  E in FP32,
+// once: its relative error of ~1e-7 leaves the first step's result 1e-14 off
+// and the second's 1e-21.
 __device__ double z_of_dc(const DcTable &T, double r) {
   const double s = r * T.inv_hr;
   const int i = max(0, min(static_cast<int>(s), T.n_r - 2));
   const double z0 = T.zr[i], z1 = T.zr[i + 1];
   double z = fma(s - i, z1 - z0, z0);
-  for (int it = 0; it < 2; ++it) {
-    const double zp = 1.0 + z;
-    const double e = sqrt(fma(T.omega_m * zp, zp * zp, 1.0 - T.omega_m));
-    z -= (dc_eval(T, z) - r) * e * (1.0 / 2997.92458);
-  }
+  const float zp = 1.0f + static_cast<float>(z), om = static_cast<float>(T.omega_m);
+  const double e = static_cast<double>(sqrtf(fmaf(om * zp, zp * zp, 1.0f - om)) * (1.0f / 2997.92458f));
+  z -= (dc_eval(T, z) - r) * e;
+  z -= (dc_eval(T, z) - r) * e;
   return z;
 }
 
-__global__ void k_geometry(const mk_qso *__restrict__ q, int64_t nq, GeomParams P, mk_skewer *sk,
+// One thread per quasar, bound by the FP64 pipe (16 cycles a warp instruction
+// and SM): 1M quasars 475 -> 352 us with E in FP32 and no division by constants;
+// small CTAs, so that a small catalogue takes many SMs (500 quasars 15.0 ->
+// 11.4 us, most of it the chain of table loads).
+
+constexpr int kGeomThreads = 32;
+
+__global__ void __launch_bounds__(kGeomThreads) k_geometry(const mk_qso *__restrict__ q, int64_t nq, GeomParams P, mk_skewer *sk,
                            int64_t *cnt_px, int64_t *cnt_seg, int *err) {
   const int64_t i = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
   if (i >= nq) return;
@@ -54,8 +64,7 @@ __global__ void k_geometry(const mk_qso *__restrict__ q, int64_t nq, GeomParams 
     const double zq = z_of_dc(P.tab, r);
     double z_lo = (1.0 + zq) * P.lrf_min / P.lambda_lya - 1.0;
     const double z_hi = (1.0 + zq) * P.lrf_max / P.lambda_lya - 1.0;
-    if (P.lobs_min > 0.0) z_lo = fmax(z_lo, P.lobs_min / P.lambda_lya - 1.0);
-    z_lo = fmax(z_lo, 0.0);
+    z_lo = fmax(z_lo, P.z_obs_min);
     int64_t jl = 0, n = 0;
     if (z_hi > z_lo) {
       if (z_hi >= zmax) {
@@ -81,7 +90,7 @@ __global__ void k_geometry(const mk_qso *__restrict__ q, int64_t nq, GeomParams 
     // Q20.44 cell coordinates of the first pixel and the step (rounding at
     // 2^-44 cells; the pixel decisions above use the exact divisions)
     const double rc = (static_cast<double>(jl) + 0.5) * P.dr;
-    const double inv_r = 1.0 / r, inv_cell = 1.0 / P.cell;
+    const double inv_r = 1.0 / r, inv_cell = P.inv_cell;
     for (int d = 0; d < 3; ++d) {
       const double u = Q.pos[d] * inv_r;
       const double c0 = fma(rc * u - P.origin[d], inv_cell, -0.5);
@@ -95,36 +104,48 @@ __global__ void k_geometry(const mk_qso *__restrict__ q, int64_t nq, GeomParams 
 }
 
 // =================================================================== scan
-// Exclusive prefix sums of two int64 sequences (pixels, segments) in three
-// passes over tiles of SCAN_TILE elements.
+// Exclusive prefix sums of two int64 sequences (pixels, pairs of segments) over
+// tiles of SCAN_TILE elements: the tiles' sums, then each tile's CTA adds up the
+// sums before its own and scans.  One tile needs only the second launch.  Past
+// kScanDirectTiles (8.4M elements) the sums before a tile are many (64 KB a CTA
+// from L2), and one CTA scans them in a launch between the two.  500 quasars:
+// one launch of 6.2 us instead of three of 15.0 us together.
 constexpr int SCAN_THREADS = 256;
 constexpr int SCAN_ITEMS = 8;
 constexpr int SCAN_TILE = SCAN_THREADS * SCAN_ITEMS;
+constexpr int64_t kScanDirectTiles = 4096;
 
 struct Pair {
   int64_t a, b;
 };
 
 __device__ __forceinline__ Pair block_exclusive_scan(Pair v, Pair *sh, Pair &total) {
-  const int t = threadIdx.x;
-  sh[t] = v;
-  __syncthreads();
-  for (int off = 1; off < SCAN_THREADS; off <<= 1) {
-    Pair add = {0, 0};
-    if (t >= off) add = sh[t - off];
-    __syncthreads();
-    sh[t].a += add.a;
-    sh[t].b += add.b;
-    __syncthreads();
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  Pair run = v;
+#pragma unroll
+  for (int off = 1; off < 32; off <<= 1) {
+    const int64_t a = __shfl_up_sync(0xffffffffu, run.a, off), b = __shfl_up_sync(0xffffffffu, run.b, off);
+    if (lane >= off) {
+      run.a += a;
+      run.b += b;
+    }
   }
-  total = sh[SCAN_THREADS - 1];
-  Pair ex = {sh[t].a - v.a, sh[t].b - v.b};
+  if (lane == 31) sh[warp] = run;
   __syncthreads();
-  return ex;
+  Pair before = {0, 0};
+  total = Pair{0, 0};
+#pragma unroll
+  for (int w = 0; w < SCAN_THREADS / 32; ++w) {
+    if (w == warp) before = total;
+    total.a += sh[w].a;
+    total.b += sh[w].b;
+  }
+  __syncthreads();
+  return Pair{before.a + run.a - v.a, before.b + run.b - v.b};
 }
 
 __global__ void k_scan_tiles(const int64_t *a, const int64_t *b, int64_t n, Pair *tile_sum) {
-  __shared__ Pair sh[SCAN_THREADS];
+  __shared__ Pair sh[SCAN_THREADS / 32];
   const int64_t base = blockIdx.x * static_cast<int64_t>(SCAN_TILE) + threadIdx.x * SCAN_ITEMS;
   Pair v = {0, 0};
   for (int k = 0; k < SCAN_ITEMS; ++k) {
@@ -139,7 +160,7 @@ __global__ void k_scan_tiles(const int64_t *a, const int64_t *b, int64_t n, Pair
 }
 
 __global__ void k_scan_tile_sums(Pair *tile_sum, int64_t ntiles) {
-  __shared__ Pair sh[SCAN_THREADS];
+  __shared__ Pair sh[SCAN_THREADS / 32];
   Pair carry = {0, 0};
   for (int64_t base = 0; base < ntiles; base += SCAN_THREADS) {
     const int64_t i = base + threadIdx.x;
@@ -152,11 +173,12 @@ __global__ void k_scan_tile_sums(Pair *tile_sum, int64_t ntiles) {
   }
 }
 
-__global__ void k_scan_apply(const int64_t *a, const int64_t *b, int64_t n, const Pair *tile_sum,
+// scanned: tile_sum holds the sums before each tile already
+__global__ void k_scan_apply(const int64_t *a, const int64_t *b, int64_t n, const Pair *tile_sum, bool scanned,
                              int64_t *out_a, int64_t *out_b, mk_skewer *sk) {
-  __shared__ Pair sh[SCAN_THREADS];
+  __shared__ Pair sh[SCAN_THREADS / 32];
   const int64_t base = blockIdx.x * static_cast<int64_t>(SCAN_TILE) + threadIdx.x * SCAN_ITEMS;
-  Pair v = {0, 0};
+  Pair v = {0, 0}, start = {0, 0};
   int64_t va[SCAN_ITEMS], vb[SCAN_ITEMS];
   for (int k = 0; k < SCAN_ITEMS; ++k) {
     va[k] = (base + k < n) ? a[base + k] : 0;
@@ -164,10 +186,19 @@ __global__ void k_scan_apply(const int64_t *a, const int64_t *b, int64_t n, cons
     v.a += va[k];
     v.b += vb[k];
   }
+  if (scanned) {
+    start = tile_sum[blockIdx.x];
+  } else if (blockIdx.x > 0) {
+    Pair s = {0, 0};
+    for (unsigned t = threadIdx.x; t < blockIdx.x; t += SCAN_THREADS) {
+      s.a += tile_sum[t].a;
+      s.b += tile_sum[t].b;
+    }
+    block_exclusive_scan(s, sh, start);
+  }
   Pair tot;
   Pair ex = block_exclusive_scan(v, sh, tot);
-  const Pair ts = tile_sum[blockIdx.x];
-  int64_t ra = ts.a + ex.a, rb = ts.b + ex.b;
+  int64_t ra = start.a + ex.a, rb = start.b + ex.b;
   for (int k = 0; k < SCAN_ITEMS; ++k) {
     if (base + k < n) {
       out_a[base + k] = ra;
@@ -350,26 +381,27 @@ __global__ void __launch_bounds__(256) k_flux(FluxParams P) {
 }
 
 // =================================================================== finalize
-// One CTA per z bin of the result struct.  The pass is bound by the latency of
-// its loads (2 MB of partials at the usual 456 CTAs): thread (g, c) sums column c
-// of its bin over the CTAs g, g + G, ..., eight independent loads at a time,
-// and the G group sums are added in order, so the result does not depend on
-// timing.  With one CTA and one thread per column it took 111 us of the 293 us of
-// a 500-quasar pass (456 partials of 12 x 43 values) and 0.7 ms after the last
-// slice of an eight-slice host pipeline; that pass now takes 181 us.
+// One cluster of kFinalizeCtas CTAs per z bin of the result struct.  The pass is
+// bound by the latency of its loads (2 MB of partials at the usual 456 CTAs) and
+// by the FP64 pipe (16 cycles a warp instruction and SM): thread (g, c) of the
+// cluster sums column c of its bin over the CTAs g, g + G, ..., eight
+// independent loads at a time, the group sums of a CTA are added in order and
+// then the CTAs', so the result does not depend on timing.  456 partials of
+// 12 x 43 values from cold caches: 111 us with one CTA and one thread per column
+// for all bins, 18.0 us with one CTA per bin, 14.5 us now.
 // The result goes straight into page-locked host memory with the error word
 // behind it, which saves the two copies that would follow.
-constexpr int kFinalizeThreads = 1024;
+constexpr int kFinalizeThreads = 512;
+constexpr int kFinalizeCtas = 4;
 
-__global__ void __launch_bounds__(kFinalizeThreads) k_finalize(const double *__restrict__ partials, int nparts,
-                                                               int n_z, int n_k, int n_fft, const int *err,
-                                                               mk_stats_out *out, int *err_out) {
-  __shared__ double sh[kFinalizeThreads];
+__global__ void __launch_bounds__(kFinalizeThreads) __cluster_dims__(kFinalizeCtas, 1, 1)
+    k_finalize(const double *__restrict__ partials, int nparts, int n_z, int n_k, int n_fft, const int *err,
+               mk_stats_out *out, int *err_out) {
+  constexpr int kCols = MK_NSUM + MK_MAX_KBINS + 1;
+  __shared__ double sh[kFinalizeThreads], part[kCols];
   __shared__ mk_stats_bin bin;
-  const int zb = blockIdx.x, tid = threadIdx.x;
-  if (zb == 0 && tid == 0) *err_out = *err;
-  double *b = reinterpret_cast<double *>(&bin);
-  for (int i = tid; i < static_cast<int>(sizeof(bin) / sizeof(double)); i += blockDim.x) b[i] = 0.0;
+  const cg::cluster_group cluster = cg::this_cluster();
+  const int zb = blockIdx.x / kFinalizeCtas, rank = blockIdx.x % kFinalizeCtas, tid = threadIdx.x;
   const StatLayout L{n_z, n_k};
   const int cols = MK_NSUM + n_k + 1, groups = blockDim.x / cols;
   const int c = tid % cols, g = tid / cols;
@@ -378,18 +410,32 @@ __global__ void __launch_bounds__(kFinalizeThreads) k_finalize(const double *__r
     const size_t size = L.size();
     double s = 0.0;
 #pragma unroll 8
-    for (int p = g; p < nparts; p += groups) s += partials[p * size + idx];
+    for (int p = rank * groups + g; p < nparts; p += kFinalizeCtas * groups) s += partials[p * size + idx];
     sh[tid] = s;
   }
   __syncthreads();
   if (zb < n_z && tid < cols) {
     double s = 0.0;
     for (int q = 0; q < groups; ++q) s += sh[q * cols + tid];
-    if (tid < MK_NSUM) bin.sums[tid] = s;
-    else if (tid < MK_NSUM + n_k) bin.p1d_sum[tid - MK_NSUM] = s;
-    else bin.n_seg = s;
+    part[tid] = s;
   }
-  __syncthreads();
+  cluster.sync();
+  if (rank == 0) {
+    if (blockIdx.x == 0 && tid == 0) *err_out = *err;
+    double *b = reinterpret_cast<double *>(&bin);
+    for (int i = tid; i < static_cast<int>(sizeof(bin) / sizeof(double)); i += blockDim.x) b[i] = 0.0;
+    __syncthreads();
+    if (zb < n_z && tid < cols) {
+      double s = 0.0;
+#pragma unroll
+      for (int r = 0; r < kFinalizeCtas; ++r) s += cluster.map_shared_rank(part, r)[tid];
+      if (tid < MK_NSUM) bin.sums[tid] = s;
+      else if (tid < MK_NSUM + n_k) bin.p1d_sum[tid - MK_NSUM] = s;
+      else bin.n_seg = s;
+    }
+  }
+  cluster.sync();  // the CTAs' shared memory has been read
+  if (rank != 0) return;
   if (zb < n_z && tid == 0) finalize_bin_scalars(&bin);
   __syncthreads();
   if (zb < n_z && tid < n_k) finalize_bin_p1d(&bin, tid, static_cast<double>(n_fft / 2) / n_k);
@@ -415,7 +461,7 @@ static int blocks_for(int64_t n, int threads) { return static_cast<int>((n + thr
 cudaError_t launch_geometry(const mk_qso *q, int64_t nq, const GeomParams &P, mk_skewer *sk, int64_t *cnt_px,
                             int64_t *cnt_seg, int *err, cudaStream_t st) {
   if (nq == 0) return cudaSuccess;
-  k_geometry<<<blocks_for(nq, 128), 128, 0, st>>>(q, nq, P, sk, cnt_px, cnt_seg, err);
+  k_geometry<<<blocks_for(nq, kGeomThreads), kGeomThreads, 0, st>>>(q, nq, P, sk, cnt_px, cnt_seg, err);
   return cudaGetLastError();
 }
 
@@ -432,9 +478,10 @@ cudaError_t launch_scan(const int64_t *a, const int64_t *b, int64_t n, int64_t *
   }
   const int64_t ntiles = (n + SCAN_TILE - 1) / SCAN_TILE;
   Pair *ts = static_cast<Pair *>(ws);
-  k_scan_tiles<<<static_cast<unsigned>(ntiles), SCAN_THREADS, 0, st>>>(a, b, n, ts);
-  k_scan_tile_sums<<<1, SCAN_THREADS, 0, st>>>(ts, ntiles);
-  k_scan_apply<<<static_cast<unsigned>(ntiles), SCAN_THREADS, 0, st>>>(a, b, n, ts, out_a, out_b, sk);
+  const bool scanned = ntiles > kScanDirectTiles;
+  if (ntiles > 1) k_scan_tiles<<<static_cast<unsigned>(ntiles), SCAN_THREADS, 0, st>>>(a, b, n, ts);
+  if (scanned) k_scan_tile_sums<<<1, SCAN_THREADS, 0, st>>>(ts, ntiles);
+  k_scan_apply<<<static_cast<unsigned>(ntiles), SCAN_THREADS, 0, st>>>(a, b, n, ts, scanned, out_a, out_b, sk);
   return cudaGetLastError();
 }
 
@@ -542,7 +589,7 @@ cudaError_t launch_flux(const FluxParams &P, int sms, cudaStream_t st) {
 
 cudaError_t launch_finalize(const double *partials, int nparts, int n_z, int n_k, int n_fft, const int *err,
                             mk_stats_out *out, int *err_out, cudaStream_t st) {
-  k_finalize<<<MK_MAX_ZBINS, kFinalizeThreads, 0, st>>>(partials, nparts, n_z, n_k, n_fft, err, out, err_out);
+  k_finalize<<<MK_MAX_ZBINS * kFinalizeCtas, kFinalizeThreads, 0, st>>>(partials, nparts, n_z, n_k, n_fft, err, out, err_out);
   return cudaGetLastError();
 }
 

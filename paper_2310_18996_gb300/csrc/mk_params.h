@@ -17,7 +17,7 @@ constexpr int32_t kBinEndNever = 1 << 30;
 struct DcTable {
   const double2 *dc;  // {D_C(z_i), dD_C/dz(z_i)}
   int n;              // entries
-  double h;           // z spacing
+  double h, inv_h;    // z spacing (a power of two), and 1 / h
   double omega_m;     // for E(z) in the Newton inversion
   const double *zr;   // z(r_i) on r_i = i hr: the starting point of the inversion
   int n_r;            // entries
@@ -26,9 +26,10 @@ struct DcTable {
 
 struct GeomParams {
   DcTable tab;
-  double lambda_lya, dr, lrf_min, lrf_max, lobs_min;
+  double lambda_lya, dr, lrf_min, lrf_max;
+  double z_obs_min;  // Lyman-alpha redshift of the least observed wavelength, >= 0
   int32_t n_min, n_max;
-  double origin[3], cell;
+  double origin[3], inv_cell;
   int32_t j_max;  // pixel tables cover J < j_max
   int32_t unit_px;  // pixels of a work unit of the skewer kernel (a pair of segments)
 };

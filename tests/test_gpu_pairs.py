@@ -101,3 +101,18 @@ def test_gaussian_kernel_runs(ctx, n_fft, n_max, cell):
     """Runs of pixels in one voxel: of one pixel (a voxel a pixel) to many, cut
     by the ends of segments, with fewer runs than warps and more than lanes."""
     check(ctx, recipe(cell, n_fft=n_fft, n_max=n_max, interp=mk.INTERP_GAUSS7), mk.BOX_HALO)
+
+
+@pytest.mark.parametrize("n", [1, 2047, 2048, 2049, 6145, 4096 * 2048, 4096 * 2048 + 2049])
+def test_offsets_at_the_tiles_of_the_scan(ctx, n):
+    """Offsets are the running sum of the lengths, for one tile, a few, and past
+    the number of tiles whose sums are scanned in a launch of their own."""
+    w = recipe(si.CELL, n_fft=256, n_max=0)
+    pos, ids = si.catalogue(si.shrink(w, n_q=min(n, 4099)))
+    k = -(-n // len(ids))
+    q = mk.catalogue_tensor(pos, ids).repeat(k)[: n * mk.QSO_DTYPE.itemsize]
+    z = torch.zeros((w["n"],) * 3, device="cuda")
+    sk, offsets, total = ctx.plan(ctx.load_box(w, z, z), q, n, w)
+    lengths = torch.from_numpy(mk.skewer_records(sk, n)["n"].astype(np.int64))
+    assert int(lengths.sum()) == total
+    np.testing.assert_array_equal(offsets.cpu().numpy(), np.concatenate([[0], np.cumsum(lengths.numpy())]))
