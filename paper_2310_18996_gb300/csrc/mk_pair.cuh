@@ -201,15 +201,19 @@ __device__ __forceinline__ void small_scale_modes(uint32_t c, const float *__res
   const u32x4 w = philox4x32_10(u32x4{c, seg, static_cast<uint32_t>(id >> 32), 0u}, seed, static_cast<uint32_t>(id));
   const bool nyq = (c == 0);
   const int m0 = nyq ? N / 2 : 2 * c, m1 = 2 * c + 1;
-  float s0 = __ldg(amp + m0), s1 = __ldg(amp + m1);
-  if (ZNODES) {  // interpolate P_s between the nodes, then the root
-    s0 = sqrtf(fmaf(w_hi, __ldg(amp_hi + m0) - s0, s0));
-    s1 = sqrtf(fmaf(w_hi, __ldg(amp_hi + m1) - s1, s1));
-  }
+  const float s0 = __ldg(amp + m0), s1 = __ldg(amp + m1);
   const float2 p0 = unit_phase(w.y), p1 = unit_phase(w.w);
   const float2 nl = neg_log_uniform2(w.x, w.z);
-  const float a0 = s0 * sqrt_pos((nyq ? 2.0f : 1.0f) * nl.x);
-  const float a1 = s1 * sqrt_pos(nl.y);
+  const float e0 = (nyq ? 2.0f : 1.0f) * nl.x, e1 = nl.y;
+  float a0, a1;
+  if (ZNODES) {  // interpolate P_s between the nodes; one root for amplitude and modulus
+    const float x0 = fmaf(w_hi, __ldg(amp_hi + m0) - s0, s0) * e0, x1 = fmaf(w_hi, __ldg(amp_hi + m1) - s1, s1) * e1;
+    a0 = x0 > 0.f ? sqrt_pos(x0) : 0.f;
+    a1 = x1 > 0.f ? sqrt_pos(x1) : 0.f;
+  } else {
+    a0 = s0 * sqrt_pos(e0);
+    a1 = s1 * sqrt_pos(e1);
+  }
   y0 = make_float2(a0 * p0.x, nyq ? 0.f : a0 * p0.y);
   y1 = make_float2(a1 * p1.x, a1 * p1.y);
 }

@@ -116,3 +116,12 @@ def test_offsets_at_the_tiles_of_the_scan(ctx, n):
     lengths = torch.from_numpy(mk.skewer_records(sk, n)["n"].astype(np.int64))
     assert int(lengths.sum()) == total
     np.testing.assert_array_equal(offsets.cpu().numpy(), np.concatenate([[0], np.cumsum(lengths.numpy())]))
+
+
+@pytest.mark.parametrize("zs", [[2.2, 2.9], list(np.linspace(1.9, 3.6, 32)), [0.5, 1.0, 1.5], [5.0, 6.0, 7.0]])
+@pytest.mark.parametrize("n_max", [0, 300])
+def test_p_s_nodes_around_the_segments(ctx, zs, n_max):
+    """The fewest and the most nodes, and segments below and above all of them."""
+    w = recipe(si.CELL, n_max=n_max)
+    p_s = np.stack([(0.5 + k / len(zs)) * np.asarray(w["p_s"]) for k in range(len(zs))])
+    check(ctx, si.shrink(w, p_s=p_s, p_s_z=zs), mk.BOX_PADDED)
