@@ -416,9 +416,10 @@ def box_synth_leg(ctx, mk, w, dev, peak, reps=3):
     draw_ms = 1000.0 * (time.perf_counter() - t0)
     del boxes, wq
     torch.cuda.empty_cache()
-    # bytes of the five passes: noise+x (write), y, z (read+write each), inverse y,
-    # inverse x (read, padded write)
-    b = 8.0 * n ** 3 * (1 + 2 + 2 + 2 + 1) + 8.0 * (n + 1) ** 3
+    # bytes of the five passes over the half spectra (n^3/2 values per field): noise+x
+    # (write one), y (read, write), z (read one, write both), inverse y (read, write
+    # both), inverse x (read both, padded write)
+    b = 8.0 * n ** 3 * (0.5 + 1 + 1.5 + 2 + 1) + 8.0 * (n + 1) ** 3
     return {"box": f"{n}^3, cell {cell}, delta + eta_xx into the padded layout",
             "ms": res["library"], "fixture_ms": res["torch_cufft_fixture"],
             "pass_bytes": b, "achieved_gbs": b / (res["library"] * 1e6), "frac_of_hbm_peak": b / (res["library"] * 1e6) / peak,
@@ -428,7 +429,7 @@ def box_synth_leg(ctx, mk, w, dev, peak, reps=3):
                                   "alone (planar), then mk_draw_qso (App. A) at nbar 1e-4 (h/Mpc)^3",
                           "synth_3_boxes_ms": synth3, "draw_wall_ms": draw_ms, "quasars": cnt,
                           "draw_note": "wall time of the synchronous call: box moments, r table on the host, "
-                                       "count pass, host scan, write pass"}}
+                                       "count pass, scan of the counts, write pass"}}
 
 
 # ---------------------------------------------------------------- Sec. 2.6 P_S tuning
@@ -768,7 +769,8 @@ def run_gb300(args, rank, world, local_rank):
                     "method": f"mk_run_host: catalogue H2D from pinned memory, {args.e2e_chunks} slices, each "
                               "slice's flux copied to pinned host memory while the next is computed",
                     "sequential_ms_per_step": e2e_copy_ms},
-            "gpu_launches": 6 * args.steps,  # per step: geometry, 3 scan passes, fused kernel, finalize
+            # per step: geometry, the scan (1 to 3 launches by catalogue size), fused kernel, finalize
+            "gpu_launches": (4 + (n_q > 2048) + (n_q > 4096 * 2048)) * args.steps,
             "launch": "CUDA graph per step (mk_run MK_GRAPH), fused persistent kernel, launch shape autotuned",
             "clocks": clk,
         }

@@ -454,7 +454,9 @@ int mk_run_host(mk_ctx *ctx, const mk_box *box, const mk_qso *h_qso, int64_t n_q
    and *occupancy target, the register budget of that many 256-thread CTAs
    per SM (2, 3 or 4).  layout: the box layout, plus 16 for MK_INTERP_GAUSS7,
    plus 32 for P_S tables at several redshifts (p_s_nodes >= 2; that
-   instance has one register budget, 3).
+   instance has one register budget, 3), plus 64 for trilinear interpolation
+   with pixels longer than 0.1 cell (p_s_nodes and length as before; that
+   instance has one register budget too).
    MK_OK when the autotuner chose it, MK_ERANGE when it is the default
    (still written). */
 int mk_launch_config(mk_ctx *ctx, int32_t n_fft, int32_t layout, int32_t big_box, uint32_t flags,
@@ -468,7 +470,7 @@ int mk_launch_config(mk_ctx *ctx, int32_t n_fft, int32_t layout, int32_t big_box
    processes running under a hard device-memory cap, and latency-bound loops in
    which a cudaMalloc or cudaFree, which waits for the whole device, is not
    acceptable.  mk_stats keeps its scratch (segment counts and offsets, scan tile
-   sums, per-CTA FP64 partial sums, the device copy of the result) in a
+   sums, per-CTA FP64 partial sums) in a
    workspace that it grows with cudaMalloc when a larger catalogue arrives.
    This call keeps the same scratch in one fixed array of
    MK_STATIC_SCRATCH_BYTES bytes in the library's own device memory, which every

@@ -88,7 +88,7 @@ __device__ __forceinline__ void flush_warp_partials(unsigned char *smem, int nwa
 // accumulators when its pixels reach the end of the bin (bin_end) or a
 // segment starts in another bin.
 //
-// Bound by instruction issue: 6.4 warp instructions a pixel at 70 % of the issue
+// Bound by instruction issue: 6.6 warp instructions a pixel at 68 % of the issue
 // slots, DRAM ~10 B a pixel.  One radix-8 transform for two segments and one set
 // of corner loads per cell of the sight line take 1.07 ms per 1.37e8 pixels
 // (512^3 box, 100k quasars, N = 256) where a radix-4 transform per segment and a
