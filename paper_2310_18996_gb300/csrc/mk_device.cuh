@@ -489,21 +489,49 @@ struct PixelSums {
 };
 
 // Add the warp's PixelSums of bin zb to the warp accumulators (warp-uniform
-// call; bins outside [0, n_z) are dropped).  A rolled butterfly: it runs about
-// once a pair of segments, and its code (60 instructions; 260 for a
-// reduce-scatter of unrolled steps) shares the instruction cache with the
-// segment loop it interrupts.
+// call; bins outside [0, n_z) are dropped).  It runs about once a pair of
+// segments, and its code shares the instruction cache with the segment loop it
+// interrupts: a rolled butterfly of the ten sums (60 instructions, 50 shuffles).
+// HALVE: two steps that halve the values a lane holds (10, 5, 3), then a rolled
+// butterfly of three: 17 shuffles in more code.  Both add in the same order, bit
+// for bit.  The staged statistics kernel gains (4.57 -> 4.36 ms a pass of 1M
+// skewers); the fused kernel (11.10 -> 11.26 ms a step) and the direct statistics
+// kernel (1.07 -> 1.25 ms a call) lose more to instruction fetches.
+template <bool HALVE>
 __device__ __forceinline__ void flush_bin_sums(const WarpAcc &W, int n_z, int zb, const PixelSums &a, int lane) {
   float v[MK_NSUM] = {a.n, a.f, a.ff, a.m1.x, a.m1.y, a.m2.x, a.m2.y, a.de, a.fm.x, a.fm.y};
+  if constexpr (HALVE) {
+    static_assert(MK_NSUM == 10, "the halving steps");
+    const bool hi = lane & 16, mid = lane & 8;
+    float w[6], x[3];
+#pragma unroll
+    for (int i = 0; i < 5; ++i)
+      w[i] = (hi ? v[i + 5] : v[i]) + __shfl_xor_sync(0xffffffffu, hi ? v[i] : v[i + 5], 16);
+    w[5] = 0.f;
+#pragma unroll
+    for (int i = 0; i < 3; ++i)
+      x[i] = (mid ? w[i + 3] : w[i]) + __shfl_xor_sync(0xffffffffu, mid ? w[i] : w[i + 3], 8);
 #pragma unroll 1
-  for (int s = 16; s >= 1; s >>= 1) {
+    for (int s = 4; s >= 1; s >>= 1) {
 #pragma unroll
-    for (int i = 0; i < MK_NSUM; ++i) v[i] += __shfl_xor_sync(0xffffffffu, v[i], s);
+      for (int i = 0; i < 3; ++i) x[i] += __shfl_xor_sync(0xffffffffu, x[i], s);
+    }
+    // lane 16 h + 8 m + k holds sum 5 h + 3 m + k
+    const int k = lane & 7;
+    const float sum = k == 0 ? x[0] : (k == 1 ? x[1] : x[2]);
+    if (k < (mid ? 2 : 3) && zb >= 0 && zb < n_z)
+      kahan_add(W.sums[zb * MK_NSUM + (hi ? 5 : 0) + (mid ? 3 : 0) + k], sum);
+  } else {
+#pragma unroll 1
+    for (int s = 16; s >= 1; s >>= 1) {
+#pragma unroll
+      for (int i = 0; i < MK_NSUM; ++i) v[i] += __shfl_xor_sync(0xffffffffu, v[i], s);
+    }
+    float s = v[0];
+#pragma unroll
+    for (int i = 1; i < MK_NSUM; ++i) s = lane == i ? v[i] : s;
+    if (lane < MK_NSUM && zb >= 0 && zb < n_z) kahan_add(W.sums[zb * MK_NSUM + lane], s);
   }
-  float s = v[0];
-#pragma unroll
-  for (int i = 1; i < MK_NSUM; ++i) s = lane == i ? v[i] : s;
-  if (lane < MK_NSUM && zb >= 0 && zb < n_z) kahan_add(W.sums[zb * MK_NSUM + lane], s);
 }
 
 // P1D bins of a thread's 4 modes 4t+1 .. 4t+4 (m modes, n_k equal bins), worked

@@ -295,7 +295,7 @@ __global__ void __launch_bounds__(256, MINB) k_skewer(SkewerParams P) {
           if (P.do_stats) {
             const int z = h ? z0[1] : z0[0];
             if (z != zc) {
-              if (zc != -2) flush_bin_sums(W, P.n_z, zc, acc, lane);
+              if (zc != -2) flush_bin_sums<false>(W, P.n_z, zc, acc, lane);
               acc.zero();
               zc = z;
             }
@@ -374,7 +374,7 @@ __global__ void __launch_bounds__(256, MINB) k_skewer(SkewerParams P) {
                     acc.add(f, x);
                     todo = false;
                   }
-                  flush_bin_sums(W, P.n_z, zc, acc, lane);
+                  flush_bin_sums<false>(W, P.n_z, zc, acc, lane);
                   acc.zero();
                   ++zc;
                   pend = bin_end[zc + 1] - jb;
@@ -419,7 +419,7 @@ __global__ void __launch_bounds__(256, MINB) k_skewer(SkewerParams P) {
     }
   }
   if (P.do_stats) {
-    if (zc != -2) flush_bin_sums(W, P.n_z, zc, acc, lane);
+    if (zc != -2) flush_bin_sums<false>(W, P.n_z, zc, acc, lane);
     flush_warp_partials(smem, nwarps, wbytes, P.n_z, P.n_k, P.partials);
   }
 }

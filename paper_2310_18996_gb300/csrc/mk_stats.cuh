@@ -108,7 +108,7 @@ struct StatPair {
 // STAGED: a tuning pass (rebin 1, fields and FGPA table set; delta, eta 16-byte
 // aligned): the next pair's fields are copied into shared memory by the bulk-copy
 // (TMA) engine while the current one is processed.  It reads 8 bytes a pixel and
-// is bound by latency and issue: 2.4 warp instructions a pixel, 4.42 ms per
+// is bound by latency and issue: 2.4 warp instructions a pixel, 4.21 ms per
 // 1.45e9 pixels, where one radix-4 transform per segment took 3.1 and 5.67 ms.
 // Both variants work through the same pairs in the same order with the same
 // grid, so a tuning pass and the statistics of its stored flux agree bit for bit.
@@ -294,7 +294,7 @@ __global__ void __launch_bounds__(256, 2) k_stats(StatParams P) {
         }
         // pixel sums
         if (z0[0] != zc) {
-          if (zc != -2) flush_bin_sums(W, P.n_z, zc, acc, lane);
+          if (zc != -2) flush_bin_sums<STAGED>(W, P.n_z, zc, acc, lane);
           acc.zero();
           zc = z0[0];
         }
@@ -321,7 +321,7 @@ __global__ void __launch_bounds__(256, 2) k_stats(StatParams P) {
                 acc.add(f8[q], x8[q]);
                 todo = false;
               }
-              flush_bin_sums(W, P.n_z, zc, acc, lane);
+              flush_bin_sums<STAGED>(W, P.n_z, zc, acc, lane);
               acc.zero();
               ++zc;
               pend = bin_stop();
@@ -354,7 +354,7 @@ __global__ void __launch_bounds__(256, 2) k_stats(StatParams P) {
     }
     cur = nxt;
   }
-  if (zc != -2) flush_bin_sums(W, P.n_z, zc, acc, lane);
+  if (zc != -2) flush_bin_sums<STAGED>(W, P.n_z, zc, acc, lane);
   flush_warp_partials(smem, nwarps, wbytes, P.n_z, P.n_k, P.partials);
 }
 
