@@ -454,7 +454,8 @@ int mk_run_host(mk_ctx *ctx, const mk_box *box, const mk_qso *h_qso, int64_t n_q
    and *occupancy target, the register budget of that many 256-thread CTAs
    per SM (2, 3 or 4).  layout: the box layout, plus 16 for MK_INTERP_GAUSS7,
    plus 32 for P_S tables at several redshifts (p_s_nodes >= 2; that
-   instance has one register budget, 3), plus 64 for trilinear interpolation
+   instance has one register budget: 2 for MK_BOX_TENSOR up to N = 1024, else
+   3), plus 64 for trilinear interpolation
    with pixels longer than 0.1 cell (p_s_nodes and length as before; that
    instance has one register budget too).
    MK_OK when the autotuner chose it, MK_ERANGE when it is the default

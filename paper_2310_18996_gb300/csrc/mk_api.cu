@@ -512,9 +512,9 @@ int skewer_grid(mk_ctx *ctx, int n_fft, int variant, int cap, LaunchCfg cfg, con
                                                      bins ? bins->n_z : 0, bins ? bins->n_k : 0, bins != nullptr));
 }
 
-// default launch: 256-thread CTAs with the register budget of three per SM
-// (85 registers; measured fastest on GB300 for N = 256)
-LaunchCfg default_cfg() { return LaunchCfg{256, 3}; }
+LaunchCfg default_cfg(int n_fft, int variant) {
+  return LaunchCfg{256, default_budget(n_fft, variant & (kGauss7Variant - 1))};
+}
 
 // kernel variant: the box layout, plus kGauss7Variant for the Gaussian kernel,
 // plus kPsNodesVariant for P_s tables at several redshifts, plus
@@ -828,7 +828,7 @@ int mk_make_skewers(mk_ctx *ctx, const mk_box *box, const mk_qso *d_qso, int64_t
   S.capacity = capacity_px;
   S.do_stats = 0;
   const int variant = kernel_variant(box, params);
-  const LaunchCfg cfg = default_cfg();
+  const LaunchCfg cfg = default_cfg(params->n_fft, variant);
   const int grid = skewer_grid(ctx, params->n_fft, variant, S.cell_cap, cfg, nullptr);
   if ((rc = time_begin(ctx))) return rc;
   CK(launch_skewer(S, params->n_fft, variant, cfg.minb, grid, cfg.threads, ctx->stream));
@@ -981,7 +981,7 @@ int mk_run(mk_ctx *ctx, const mk_box *box, const mk_qso *d_qso, int64_t n_qso, c
   // the launch shape: tuned, or tune now, or the default
   const int variant = kernel_variant(box, params);
   const uint64_t key = tune_key(params->n_fft, variant, box->lgn, flags);
-  LaunchCfg cfg = default_cfg();
+  LaunchCfg cfg = default_cfg(params->n_fft, variant);
   auto it = ctx->tuned.find(key);
   if (it != ctx->tuned.end()) cfg = it->second;
 
@@ -1161,7 +1161,7 @@ int mk_run_host(mk_ctx *ctx, const mk_box *box, const mk_qso *h_qso, int64_t n_q
 
   const uint32_t kflags = MK_STORE_FLUX | (stats ? MK_STATS : 0u);
   const int variant = kernel_variant(box, params);
-  LaunchCfg cfg = default_cfg();
+  LaunchCfg cfg = default_cfg(params->n_fft, variant);
   auto it = ctx->tuned.find(tune_key(params->n_fft, variant, box->lgn, kflags));
   if (it != ctx->tuned.end()) cfg = it->second;
   const int grid = skewer_grid(ctx, params->n_fft, variant, run_cells(box, params), cfg, stats ? bins : nullptr);
@@ -1217,7 +1217,7 @@ int mk_launch_config(mk_ctx *ctx, int32_t n_fft, int32_t layout, int32_t big_box
                      int32_t *threads, int32_t *occupancy) {
   if (!ctx || !threads || !occupancy) return MK_EINVAL;
   if (!skewer_fft(n_fft)) return fail(ctx, MK_EINVAL, "bad n_fft");
-  LaunchCfg c = default_cfg();
+  LaunchCfg c = default_cfg(n_fft, layout);
   auto it = ctx->tuned.find(tune_key(n_fft, layout, big_box ? 11 : 10, flags));
   if (it != ctx->tuned.end()) c = it->second;
   *threads = c.threads;

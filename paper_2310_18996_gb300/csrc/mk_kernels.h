@@ -11,6 +11,14 @@ constexpr int kGauss7Variant = 16;   // kernel variant bit of MK_INTERP_GAUSS7
 constexpr int kPsNodesVariant = 32;  // kernel variant bit of P_s tables at several redshifts
 constexpr int kPixelGatherVariant = 64;  // kernel variant bit of trilinear gathers per pixel (see use_cells)
 
+// Default register budget of the fused kernel, in 256-thread CTAs per SM: three (80
+// registers), or two (128 registers) on a tensor box up to N = 1024, where the
+// cells' 64-byte corners need more loads in flight than three CTAs of 80 registers
+// hold.  1.4e8 pixels of a 512^3 box at budgets 3 and 2: tensor N = 256 1.52 and
+// 1.41 ms, N = 1024 2.35 and 2.18, N = 2048 3.02 and 3.31; padded N = 256 1.07 and
+// 1.13, N = 2048 2.32 and 2.61 (budget 4 spills: 1.35 to 3.8 ms).
+constexpr int default_budget(int n_fft, int layout) { return layout == MK_BOX_TENSOR && n_fft <= 1024 ? 2 : 3; }
+
 // Whether a trilinear run reads its box through the cells of the sight line
 // (plan_cells in mk_pair.cuh) or gathers pixel by pixel.  Up to dr/cell = 0.1
 // (the paper's is 0.091) a pair's cells fit three rounds of one cell per thread
@@ -49,7 +57,7 @@ inline bool staged_pass(const void *pixtab, const float *delta, const float *eta
 }
 int stats_blocks_per_sm(int n_fft, int threads, int n_z, int n_k);
 // variant: box layout, plus kGauss7Variant for the Gaussian-kernel interpolation,
-// plus kPsNodesVariant for z-dependent P_s (built for register budget 3 only),
+// plus kPsNodesVariant for z-dependent P_s (built for the default register budget only),
 // plus kPixelGatherVariant (budget 3 only); cap: cells of a run (P.cell_cap);
 // minb: register budget of the instance, that of minb 256-thread CTAs per SM
 // (2, 3 or 4)

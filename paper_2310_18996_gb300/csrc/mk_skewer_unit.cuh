@@ -13,10 +13,10 @@ namespace mk {
 namespace skewer_unit_detail {
 
 // minb: register budget of the instance, that of minb 256-thread CTAs per SM;
-// psz: P_s tables at several redshifts (one instance per layout, budget 3)
+// psz: P_s tables at several redshifts (one instance per layout, of the default budget)
 template <int NN, int L, int INTERP, bool CELLS, typename F>
 cudaError_t with_budget(bool psz, int minb, F &&fn) {
-  if (psz) return fn(k_skewer<NN, L, 3, INTERP, true, CELLS>);
+  if (psz) return fn(k_skewer<NN, L, default_budget(NN, L), INTERP, true, CELLS>);
   if (minb >= 4) return fn(k_skewer<NN, L, 4, INTERP, false, CELLS>);
   if (minb == 3) return fn(k_skewer<NN, L, 3, INTERP, false, CELLS>);
   return fn(k_skewer<NN, L, 2, INTERP, false, CELLS>);
