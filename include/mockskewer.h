@@ -374,7 +374,9 @@ int mk_flux(mk_ctx *ctx, const mk_skewer_params *params, const mk_skewer *d_sk, 
    the segment.  Synchronous: fills *h_out.  MK_ERANGE (statistics not
    written) when a record's pixels run past the redshift tables of
    params->dr, as in mk_flux; mk_flux_stats and the tuning passes check the
-   same. */
+   same.  Flux may hold any value: one that is not finite makes the sums of its
+   pixel's z bin and, in a full segment, the P1D of that segment's z bin not
+   finite, and touches no other bin. */
 int mk_stats(mk_ctx *ctx, const mk_skewer_params *params, const mk_skewer *d_sk, int64_t n_sk,
              const int64_t *d_offsets_out, const float *d_flux, int32_t rebin,
              const float *d_delta, const float *d_eta, const mk_stat_bins *bins,

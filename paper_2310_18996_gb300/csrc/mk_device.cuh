@@ -132,6 +132,24 @@ __device__ __forceinline__ void team_sync(int team) {
   }
 }
 
+// true when pred holds on every thread of the team (a barrier of the team)
+template <int T>
+__device__ __forceinline__ bool team_all(int team, bool pred) {
+  if constexpr (T == 32) {
+    __syncwarp();
+    return __all_sync(0xffffffffu, pred);
+  } else {
+    uint32_t r;
+    asm volatile(
+        "{\n\t.reg .pred pi, po;\n\tsetp.ne.u32 pi, %1, 0;\n\tbar.red.and.pred po, %2, %3, pi;\n\t"
+        "selp.u32 %0, 1, 0, po;\n\t}"
+        : "=r"(r)
+        : "r"(static_cast<uint32_t>(pred)), "r"(team + 1), "r"(T)
+        : "memory");
+    return r != 0;
+  }
+}
+
 // ------------------------------------------------------------------ FFT plan
 template <int N>
 struct Fft {

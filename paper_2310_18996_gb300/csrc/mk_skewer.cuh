@@ -260,7 +260,8 @@ __global__ void __launch_bounds__(256, MINB) k_skewer(SkewerParams P) {
         team_sync<T>(team);
         load_modes<N>(buf, v, t);
       }
-      team_sync<T>(team);  // the modes are read; the cells are read
+      // (a barrier: the modes are read; the cells are read)
+      if (round == 0) team_sync<T>(team); else drop_nan<T>(v, za, zb, team);
       pair_fft<N>(buf, v, tws, P.tw, t, team);
       if (round == 1) break;
 
@@ -396,7 +397,7 @@ __global__ void __launch_bounds__(256, MINB) k_skewer(SkewerParams P) {
         for (int k = 0; k < 8; ++k) v[k] = make_float2(v[k].y, f8[k]);
       }
       // ---- P1D of the full segments
-      if (!((za >= 0 && za < P.n_z) || (zb >= 0 && zb < P.n_z))) {  // (always without statistics)
+      if (!(counted(za, P.n_z) || counted(zb, P.n_z))) {  // (always without statistics)
         za = -2;
         break;
       }
@@ -406,9 +407,10 @@ __global__ void __launch_bounds__(256, MINB) k_skewer(SkewerParams P) {
       pair_powers<N>(buf, v, t, team, ka, kb);
 #pragma unroll 1
       for (int h = 0; h < 2; ++h) {
-        if (za >= 0 && za < P.n_z) {
-          accumulate_p1d(W, P.n_k, bins, ka, 0.25f * P.p1d_scale, za);
-          if (t == 0) W.nseg[za] += 1u;
+        if (counted(za, P.n_z)) {
+          const int z = za & ~kPartFlag;
+          accumulate_p1d(W, P.n_k, bins, ka, za == z ? 0.25f * P.p1d_scale : __uint_as_float(0x7fffffffu), z);
+          if (t == 0) W.nseg[z] += 1u;
         }
         za = zb;
 #pragma unroll

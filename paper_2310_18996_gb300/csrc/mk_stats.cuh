@@ -17,7 +17,7 @@ struct StatSmem {
   static constexpr int STAGE = 2 * N + 4;  // floats per field and buffer (a pair plus its 16-byte misalignment)
   static_assert(2 * STAGE >= 2 * PairFft<N>::BUF, "a stage buffer holds the exchange buffer");
   static_assert((STAGE * sizeof(float)) % 16 == 0, "stage buffers start on 16 bytes");
-  static constexpr size_t HEAD = PairSmem<N>::HEAD;
+  static constexpr size_t HEAD = PairSmem<N>::HEAD + 8 * sizeof(uint2);  // and a slot per warp for part_segments
   static constexpr size_t TEAM = STAGED ? 4 * STAGE * sizeof(float) + 2 * sizeof(uint64_t) : sizeof(float2) * PairFft<N>::BUF;
   static size_t bytes(int threads, int n_z, int n_k) {
     return acc_bytes(threads, n_z, n_k, true) + HEAD + static_cast<size_t>(threads / (N / 8)) * TEAM;
@@ -65,23 +65,6 @@ __device__ __forceinline__ void bulk_g2s(void *dst, const void *src, uint32_t by
                : "memory");
 }
 
-// true when pred holds on every thread of the team (a barrier of the team)
-template <int T>
-__device__ __forceinline__ bool team_all(int team, bool pred) {
-  if constexpr (T == 32) {
-    return __all_sync(0xffffffffu, pred);
-  } else {
-    uint32_t r;
-    asm volatile(
-        "{\n\t.reg .pred pi, po;\n\tsetp.ne.u32 pi, %1, 0;\n\tbar.red.and.pred po, %2, %3, pi;\n\t"
-        "selp.u32 %0, 1, 0, po;\n\t}"
-        : "=r"(r)
-        : "r"(static_cast<uint32_t>(pred)), "r"(team + 1), "r"(T)
-        : "memory");
-    return r != 0;
-  }
-}
-
 // Where the kernel finds a pair of segments: its first index in the stored
 // arrays (fields, or flux), its output pixels, its first pixel-table index,
 // whether its pixels lie inside the tables; and, staged, the last (shift + npx)
@@ -125,6 +108,7 @@ __global__ void __launch_bounds__(256, 2) k_stats(StatParams P) {
   float2 *tws = reinterpret_cast<float2 *>(smem + nwarps * wbytes);
   int32_t *bin_end = reinterpret_cast<int32_t *>(tws + (PairFft<N>::TW_BYTES + 15) / 16 * 2);
   unsigned char *areas = smem + nwarps * wbytes + StatSmem<N, STAGED>::HEAD;
+  uint2 *slots = reinterpret_cast<uint2 *>(areas - 8 * sizeof(uint2)) + team * (T / 32);
   // stage buffers b = 0, 1: delta at stage_buf + 2 b STAGE, eta at stage_buf + (2 b + 1) STAGE
   float *stage_buf = reinterpret_cast<float *>(areas) + (STAGED ? team * 4 * STAGE : team * 2 * PairFft<N>::BUF);
   uint64_t *bars = reinterpret_cast<uint64_t *>(areas + static_cast<size_t>(teams) * 4 * STAGE * sizeof(float)) + 2 * team;
@@ -335,22 +319,31 @@ __global__ void __launch_bounds__(256, 2) k_stats(StatParams P) {
       for (int q = 0; q < 8; ++q) v[q] = make_float2(v[q].y, f8[q]);
     }
     // ---- P1D of the full segments
-    const bool pa = za >= 0 && za < P.n_z, pb = zb >= 0 && zb < P.n_z;
-    team_sync<T>(team);  // every field value is read before the transform overwrites the buffer
-    if (pa || pb) {
+    // a barrier on both ways: every field value is read before the transform overwrites the buffer
+    if (!(counted(za, P.n_z) || counted(zb, P.n_z))) {
+      team_sync<T>(team);
+    } else {
+      float2 e = f2mul(v[0], v[0]);
+#pragma unroll
+      for (int k = 1; k < 8; ++k) e = f2fma(v[k], v[k], e);
+      const uint2 energies = team_max<T>(make_uint2(__float_as_uint(e.x), __float_as_uint(e.y)), slots, t, team);
+      part_segments<T>(v, energies, za, zb, P.n_z, slots, t, team);
       pair_fft<N>(buf, v, tws, P.tw, t, team);
       float ka[4], kb[4];
       pair_powers<N>(buf, v, t, team, ka, kb);
 #pragma unroll 1
       for (int h = 0; h < 2; ++h) {
-        if (za >= 0 && za < P.n_z) {
-          accumulate_p1d(W, P.n_k, bins, ka, 0.25f * P.p1d_scale, za);
-          if (t == 0) W.nseg[za] += 1u;
+        if (counted(za, P.n_z)) {
+          const int z = za & ~kPartFlag;
+          const float up = za == z ? 1.f : __uint_as_float(h ? slots[0].y : slots[0].x);
+          accumulate_p1d(W, P.n_k, bins, ka, 0.25f * P.p1d_scale * up * up, z);
+          if (t == 0) W.nseg[z] += 1u;
         }
         za = zb;
 #pragma unroll
         for (int j = 0; j < 4; ++j) ka[j] = kb[j];
       }
+      if (T > 32 && (zb & kPartFlag)) team_sync<T>(team);  // slots[0] is read
     }
     cur = nxt;
   }
