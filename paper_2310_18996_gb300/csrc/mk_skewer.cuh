@@ -295,7 +295,7 @@ __global__ void __launch_bounds__(256, MINB) k_skewer(SkewerParams P) {
           int pend = N;  // segment pixel where bin zc ends
           if (P.do_stats) {
             const int z = h ? z0[1] : z0[0];
-            if (z != zc) {
+            if (z != zc || (h == 0 && u % kRunPairs == 0)) {
               if (zc != -2) flush_bin_sums<false>(W, P.n_z, zc, acc, lane);
               acc.zero();
               zc = z;

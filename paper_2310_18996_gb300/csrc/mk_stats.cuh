@@ -277,7 +277,7 @@ __global__ void __launch_bounds__(256, 2) k_stats(StatParams P) {
           }
         }
         // pixel sums
-        if (z0[0] != zc) {
+        if (z0[0] != zc || (h == 0 && u % kRunPairs == 0)) {
           if (zc != -2) flush_bin_sums<STAGED>(W, P.n_z, zc, acc, lane);
           acc.zero();
           zc = z0[0];
