@@ -337,20 +337,18 @@ __device__ __forceinline__ void load_modes(const float2 *buf, float2 (&v)[8], in
 // shared-memory reads and three packed FMAs instead of eight global loads and
 // seven lerps.
 //
-// Positions along a run are 2^-35 cells: frac + s q at pixel q, with s < 2^32 for
-// steps below 1/8 of a cell, one 32 x 32 + 64-bit multiply-add each; the step's
-// rounding moves a position by at most 2^-36 cells a pixel (the weights have 23
-// bits).  The same arithmetic decides which cell a pixel is in and where it is
-// inside it, so a pixel next to a face may take either cell but always with the
-// weight that belongs to it.  A decreasing coordinate runs on its complement,
-// which increases and crosses cells at the same pixels.
+// Positions along a run are the record's own, 2^-44 cells: frac + step q at pixel
+// q.  The same arithmetic decides which cell a pixel is in and where it is inside
+// it.  A decreasing coordinate runs on its complement, which increases and crosses
+// cells at the same pixels.  (2^-35 cells in 32 x 32-bit products were 65
+// instructions a pair less, and let the step's rounding grow to 2^-24 cells, as
+// much as the weight's own, by the end of a pair at N = 2048.)
 struct alignas(16) LineAxis {
-  uint64_t frac;  // position of pixel 0 inside its cell, plus the rounding of the weights
-  uint32_t s;     // |step|
+  uint64_t frac;  // position of pixel 0 inside its cell, in the direction of travel
+  uint64_t step;  // |step|
   int32_t c0;     // cell of pixel 0
-  float inv;      // 1 / s
+  float inv;      // 1 / step
   float slope;    // signed step in cells
-  int32_t sign;   // +1, or -1 for a decreasing coordinate
   int32_t n;      // crossings up to the last pixel
 };
 struct CellPlan {
@@ -371,21 +369,15 @@ __device__ __forceinline__ int plan_cells(const CellPlan &C, const mk_skewer *re
   constexpr int T = N / 8, WORDS = N / 16;
   if (t < WORDS) C.mask[t] = make_uint2(0u, 0u);
   if (t < 3) {
-    const int64_t step = rec->step[t], p = rec->p0[t] + j0 * step;
+    const int64_t step = rec->step[t], p = rec->p0[t] + kRoundQ + j0 * step;
     const bool neg = step < 0;
     LineAxis A;
-    A.frac = ((static_cast<uint64_t>(neg ? ~p : p) & ((uint64_t(1) << 44) - 1)) >> 9) + (1u << 11);
-    A.s = static_cast<uint32_t>(((neg ? -step : step) + 256) >> 9);
+    A.frac = static_cast<uint64_t>(neg ? ~p : p) & ((uint64_t(1) << 44) - 1);
+    A.step = static_cast<uint64_t>(neg ? -step : step);
     A.c0 = static_cast<int32_t>(p >> 44);
-    A.inv = __fdividef(1.0f, static_cast<float>(A.s));
+    A.inv = __fdividef(1.0f, __ull2float_rn(A.step));
     A.slope = static_cast<float>(step) * 0x1p-44f;
-    A.sign = neg ? -1 : 1;
-    A.n = static_cast<int>((A.frac + static_cast<uint64_t>(A.s) * (npx - 1)) >> 35);
-    if (A.frac >> 35) {  // rounded up to the next cell (weight 0)
-      A.frac -= uint64_t(1) << 35;
-      A.c0 += A.sign;
-      A.n -= 1;
-    }
+    A.n = static_cast<int>((A.frac + A.step * static_cast<uint32_t>(npx - 1)) >> 44);
     C.line[t] = A;
   }
   team_sync<T>(team);
@@ -398,14 +390,14 @@ __device__ __forceinline__ int plan_cells(const CellPlan &C, const mk_skewer *re
       const int ax = (i >= nx ? 1 : 0) + (i >= nxy ? 1 : 0);
       const uint32_t k = 1 + i - (i >= nxy ? nxy : (i >= nx ? nx : 0));
       const uint64_t frac = C.line[ax].frac;
-      const uint32_t s = C.line[ax].s;
-      // the smallest q with frac + q s >= k cells: the FP32 quotient is within
+      const uint64_t step = C.line[ax].step;
+      // the smallest q with frac + q step >= k cells: the FP32 quotient is within
       // 1e-3 of it, so q is its integer part or one or two more
       const uint32_t q0 =
-          static_cast<uint32_t>(__ull2float_rn((static_cast<uint64_t>(k) << 35) - frac) * C.line[ax].inv);
-      const uint64_t v = frac + static_cast<uint64_t>(s) * q0;
-      const int q = static_cast<int>(q0) + (static_cast<uint32_t>(v >> 35) < k ? 1 : 0) +
-                    (static_cast<uint32_t>((v + s) >> 35) < k ? 1 : 0);
+          static_cast<uint32_t>(__ull2float_rn((static_cast<uint64_t>(k) << 44) - frac) * C.line[ax].inv);
+      const uint64_t v = frac + step * q0;
+      const int q = static_cast<int>(q0) + (static_cast<uint32_t>(v >> 44) < k ? 1 : 0) +
+                    (static_cast<uint32_t>((v + step) >> 44) < k ? 1 : 0);
       at[i] = q;
       atomicOr(&C.mask[q >> 5].x, 1u << (q & 31));
     }
@@ -538,11 +530,10 @@ __device__ __forceinline__ void expand_cell(const CellPlan &C, int c, const floa
 #pragma unroll
   for (int k = 0; k < 3; ++k) {
     const LineAxis A = C.line[k];
-    const uint64_t v = A.frac + static_cast<uint64_t>(A.s) * q;
-    cell[k] = (A.c0 + A.sign * static_cast<int>(v >> 35)) & mask;
-    // weight in the direction of travel, 23 bits; 1 - it against the axis
-    const float f = __uint_as_float(0x3F800000u | (static_cast<uint32_t>(v >> 12) & 0x7FFFFFu)) - 1.0f;
-    w[k] = A.sign > 0 ? f : 1.0f - f;
+    const uint64_t v = A.frac + A.step * q;
+    const int crossed = static_cast<int>(v >> 44);
+    cell[k] = (A.slope < 0.f ? A.c0 - crossed : A.c0 + crossed) & mask;
+    w[k] = weight_of(static_cast<int64_t>(A.slope < 0.f ? ~v : v));
     sl[k] = A.slope;
   }
   const float wx = w[0], wy = w[1], wz = w[2], sx = sl[0], sy = sl[1], sz = sl[2];
