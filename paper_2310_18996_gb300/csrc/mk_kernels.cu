@@ -25,26 +25,25 @@ __device__ __forceinline__ double dc_eval(const DcTable &T, double z) {
 }
 
 // z(r): linear interpolation in the z(r) table (error ~1e-7), then two
-// Newton steps on the Hermite D_C, dz = (D_C(z) - r) E(z) H0/c.  E in FP32,
-// once: its relative error of ~1e-7 leaves the first step's result 1e-14 off
-// and the second's 1e-21.
+// Newton steps on the Hermite D_C, dz = (D_C(z) - r) E(z) H0/c, both with the E of
+// the starting point: that is 1e-7 off, so the second step still leaves less than
+// the FP64 rounding of D_C(z) - r.
 __device__ double z_of_dc(const DcTable &T, double r) {
   const double s = r * T.inv_hr;
   const int i = max(0, min(static_cast<int>(s), T.n_r - 2));
   const double z0 = T.zr[i], z1 = T.zr[i + 1];
   double z = fma(s - i, z1 - z0, z0);
-  const float zp = 1.0f + static_cast<float>(z), om = static_cast<float>(T.omega_m);
-  const double e = static_cast<double>(sqrtf(fmaf(om * zp, zp * zp, 1.0f - om)) * (1.0f / 2997.92458f));
+  const double zp = 1.0 + z;
+  const double e = sqrt(fma(T.omega_m * zp, zp * zp, 1.0 - T.omega_m)) * (1.0 / 2997.92458);
   z -= (dc_eval(T, z) - r) * e;
   z -= (dc_eval(T, z) - r) * e;
   return z;
 }
 
 // One thread per quasar, bound by the FP64 pipe (16 cycles a warp instruction
-// and SM): 1M quasars 475 -> 352 us with E in FP32 and no division by constants;
-// small CTAs, so that a small catalogue takes many SMs (500 quasars 15.0 ->
-// 11.4 us, most of it the chain of table loads).
-
+// and SM): 1M quasars 475 -> 370 us with one E for both steps and no division by
+// constants; small CTAs, so that a small catalogue takes many SMs (500 quasars
+// 15.0 -> 11.5 us, most of it the chain of table loads).
 constexpr int kGeomThreads = 32;
 
 __global__ void __launch_bounds__(kGeomThreads) k_geometry(const mk_qso *__restrict__ q, int64_t nq, GeomParams P, mk_skewer *sk,
