@@ -329,7 +329,10 @@ typedef struct mk_qso_draw_params {
    d_box_q[i]: n^3 floats at stride box_stride (1 planar, 2 for the pairs
    of mk_synth_box's MK_BOX_INTERLEAVED output, which reads delta).
    d_qso: capacity records.  *h_count: quasars drawn (also beyond capacity,
-   then MK_ERANGE and only the first capacity are written).  Synchronous. */
+   then MK_ERANGE and only the first capacity are written).  Synchronous.
+   Takes 0.14 n^3 bytes of device scratch (MK_ENOMEM where there is none); up to
+   256 MiB of it stay with the context for its next draw, more is given back
+   before the call returns. */
 int mk_draw_qso(mk_ctx *ctx, const mk_qso_draw_params *params, const float *const d_box_q[3], int32_t box_stride,
                 mk_qso *d_qso, int64_t capacity, int64_t *h_count);
 

@@ -11,6 +11,7 @@
 #include <vector>
 
 #include "../../include/mockskewer.h"
+#include "mk_host.h"
 #include "mk_kernels.h"
 #include "mk_trace.h"
 
@@ -1424,6 +1425,12 @@ int ctx_scratch(mk_ctx *c, size_t bytes, unsigned char **p) {
   const int rc = grow(c, &c->d_scratch, &c->scratch_cap, bytes);
   *p = static_cast<unsigned char *>(c->d_scratch);
   return rc;
+}
+void ctx_trim_scratch(mk_ctx *c) {
+  if (c->scratch_cap <= kScratchKept) return;
+  cudaFree(c->d_scratch);  // (waits for the device)
+  c->d_scratch = nullptr;
+  c->scratch_cap = 0;
 }
 double ctx_z_of(mk_ctx *c, double r) { return c->cos.z_of(r); }
 double ctx_growth(mk_ctx *c, double z) { return c->cos.growth(z); }

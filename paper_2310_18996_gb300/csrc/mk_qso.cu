@@ -306,8 +306,9 @@ extern "C" int mk_draw_qso(mk_ctx *ctx, const mk_qso_draw_params *q, const float
   CKQ(ctx, cudaSetDevice(mkhost::ctx_device(ctx)));
   const cudaStream_t st = mkhost::ctx_stream(ctx);
   const int64_t n = q->n, nv = n * n * n;
-  // device scratch, kept by the context: moments' partials, coefficient table,
-  // accept bits, counts and offsets of the sub-ranges, scan tiles
+  // device scratch: moments' partials, coefficient table, accept bits, counts and
+  // offsets of the sub-ranges, scan tiles (0.14 bytes a voxel); the context keeps a
+  // moderate one for the next call
   const int64_t subs = (nv + kSub - 1) / kSub;
   const int red_blocks = std::min<int64_t>(4 * mkhost::ctx_sms(ctx), (nv + kDrawThreads - 1) / kDrawThreads);
   const int n_tab = 8192;
@@ -322,6 +323,10 @@ extern "C" int mk_draw_qso(mk_ctx *ctx, const mk_qso_draw_params *q, const float
   const size_t o_bits = piece(sizeof(uint32_t) * subs * (kSub / 32)), o_cnt = piece(sizeof(int64_t) * subs);
   const size_t o_off = piece(sizeof(int64_t) * (subs + 1)), o_scan = piece(scan_workspace_bytes(subs));
   unsigned char *ws = nullptr;
+  struct Trim {
+    mk_ctx *ctx;
+    ~Trim() { mkhost::ctx_trim_scratch(ctx); }
+  } trim{ctx};
   if (int rc = mkhost::ctx_scratch(ctx, at, &ws)) return rc;
   double *d_part = reinterpret_cast<double *>(ws + o_part);
   float4 *d_tab = reinterpret_cast<float4 *>(ws + o_tab);
