@@ -7,7 +7,7 @@
 #include <cmath>
 #include <cstdio>
 #include <cstring>
-#include <system_error>
+#include <exception>
 #include <thread>
 #include <vector>
 
@@ -392,7 +392,7 @@ extern "C" int mk_draw_qso(mk_ctx *ctx, const mk_qso_draw_params *q, const float
         helper[t] = std::thread(fill, k0, k1);
         continue;
       }
-    } catch (const std::system_error &) {  // no thread to be had: this one does the share
+    } catch (const std::exception &) {  // no thread, or no memory for one: this one does the share
     }
     fill(k0, k1);
   }
