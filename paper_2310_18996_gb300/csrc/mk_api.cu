@@ -143,7 +143,7 @@ struct LaunchCfg {
 
 struct mk_ctx {
   int device = 0;
-  int sms = 0;
+  int sms = 0, sm_smem = 0;
   cudaStream_t stream = nullptr;
   mk_cosmo cosmo{};
   std::string err;
@@ -513,6 +513,13 @@ int skewer_grid(mk_ctx *ctx, int n_fft, int variant, int cap, LaunchCfg cfg, con
                                                      bins ? bins->n_z : 0, bins ? bins->n_k : 0, bins != nullptr));
 }
 
+// A shape of 256 threads with as many as the binning's accumulators let run.
+LaunchCfg shaped(mk_ctx *ctx, int n_fft, int cap, LaunchCfg cfg, const mk_stat_bins *bins) {
+  if (bins && cfg.threads == 256)
+    cfg.threads = skewer_threads(n_fft, cap, cfg.minb, ctx->sm_smem, bins->n_z, bins->n_k, true);
+  return cfg;
+}
+
 LaunchCfg default_cfg(int n_fft, int variant) {
   return LaunchCfg{256, default_budget(n_fft, variant & (kGauss7Variant - 1))};
 }
@@ -627,6 +634,7 @@ int mk_create(mk_ctx **out, int device, void *cuda_stream, const mk_cosmo *cosmo
     cudaDeviceProp prop;
     if (cudaGetDeviceProperties(&prop, device) != cudaSuccess) { rc = MK_ECUDA; break; }
     ctx->sms = prop.multiProcessorCount;
+    ctx->sm_smem = static_cast<int>(prop.sharedMemPerMultiprocessor);
     ctx->n_dc = static_cast<int>(ctx->cos.dc.size());
     std::vector<double2> tab(ctx->n_dc);
     for (int i = 0; i < ctx->n_dc; ++i) tab[i] = make_double2(ctx->cos.dc[i], ctx->cos.slope[i]);
@@ -887,7 +895,7 @@ int stats_pass(mk_ctx *ctx, const mk_skewer_params *params, const mk_skewer *d_s
       (rc = ensure_twiddles(ctx, bins->n_fft)) || (rc = ensure_zbin(ctx, bins, rebin)))
     return rc;
   if (nodes && (rc = ensure_pixtab(ctx, nodes))) return rc;
-  const int threads = 256;
+  const int threads = stats_threads(bins->n_fft, ctx->sm_smem, bins->n_z, bins->n_k);
   const StatLayout L{bins->n_z, bins->n_k};
   const int grid = stats_grid(ctx, bins, threads);
   if ((rc = grow(ctx, reinterpret_cast<void **>(&ctx->d_partials), &ctx->partials_cap,
@@ -1022,8 +1030,9 @@ int mk_run(mk_ctx *ctx, const mk_box *box, const mk_qso *d_qso, int64_t n_qso, c
     CK(cudaEventCreate(&a0));
     CK(cudaEventCreate(&a1));
     float best = 1e30f;
-    for (const LaunchCfg &c : cand) {
-      if (c.threads < params->n_fft / 8) continue;  // a team must fit in a CTA
+    for (const LaunchCfg &shape : cand) {
+      if (shape.threads < params->n_fft / 8) continue;  // a team must fit in a CTA
+      const LaunchCfg c = shaped(ctx, params->n_fft, S.cell_cap, shape, stats ? bins : nullptr);
       const int grid = skewer_grid(ctx, params->n_fft, variant, S.cell_cap, c, stats ? bins : nullptr);
       if ((rc = ensure_partials(grid))) break;
       if ((rc = enqueue_geometry(ctx, G, d_qso, n_qso, d_sk, d_offsets))) break;
@@ -1039,7 +1048,7 @@ int mk_run(mk_ctx *ctx, const mk_box *box, const mk_qso *d_qso, int64_t n_qso, c
       if (rc) break;
       if (ms < best) {
         best = ms;
-        cfg = c;
+        cfg = shape;
       }
     }
     cudaEventDestroy(a0);
@@ -1048,6 +1057,7 @@ int mk_run(mk_ctx *ctx, const mk_box *box, const mk_qso *d_qso, int64_t n_qso, c
     ctx->tuned[key] = cfg;
   }
 
+  cfg = shaped(ctx, params->n_fft, S.cell_cap, cfg, stats ? bins : nullptr);
   const int grid = skewer_grid(ctx, params->n_fft, variant, S.cell_cap, cfg, stats ? bins : nullptr);
   if ((rc = ensure_partials(grid))) return rc;
 
@@ -1165,6 +1175,7 @@ int mk_run_host(mk_ctx *ctx, const mk_box *box, const mk_qso *h_qso, int64_t n_q
   LaunchCfg cfg = default_cfg(params->n_fft, variant);
   auto it = ctx->tuned.find(tune_key(params->n_fft, variant, box->lgn, kflags));
   if (it != ctx->tuned.end()) cfg = it->second;
+  cfg = shaped(ctx, params->n_fft, run_cells(box, params), cfg, stats ? bins : nullptr);
   const int grid = skewer_grid(ctx, params->n_fft, variant, run_cells(box, params), cfg, stats ? bins : nullptr);
   const StatLayout L{stats ? bins->n_z : 0, stats ? bins->n_k : 0};
   if (stats && (rc = grow(ctx, reinterpret_cast<void **>(&ctx->d_partials), &ctx->partials_cap,
@@ -1378,7 +1389,7 @@ extern "C" int mk_stats_static(mk_ctx *ctx, const mk_skewer_params *params, cons
   double *d_part = reinterpret_cast<double *>(base + off_part);
   const size_t part_doubles = (MK_STATIC_SCRATCH_BYTES - off_part) / sizeof(double);
 
-  const int threads = 256;
+  const int threads = stats_threads(bins->n_fft, ctx->sm_smem, bins->n_z, bins->n_k);
   const StatLayout L{bins->n_z, bins->n_k};
   int grid = stats_grid(ctx, bins, threads);
   if (static_cast<size_t>(grid) * L.size() > part_doubles) grid = static_cast<int>(part_doubles / L.size());

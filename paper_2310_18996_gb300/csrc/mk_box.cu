@@ -141,10 +141,6 @@ __device__ __forceinline__ void cp_async_wait_all() {
   asm volatile("cp.async.commit_group;\ncp.async.wait_group 0;\n" ::: "memory");
 }
 
-// Start a line on its way to L2: the next group's rows are requested while the
-// current group transforms, so that its copies then wait for L2, not for DRAM.
-__device__ __forceinline__ void prefetch_l2(const void *p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
-
 __device__ __forceinline__ int wrap_index(int j, int n) { return j < n / 2 ? j : j - n; }
 
 // Filter pair p of the Sec. 2.1 boxes at wave vector k (k2 = |k|^2 > 0):
@@ -261,6 +257,8 @@ __global__ void __launch_bounds__(BoxSmem<N2, REG>::THREADS, 2) k_box_pass(BoxPa
       float2 *base = P.work + off(P.az, static_cast<int>(g / blocks)) + off(P.ax, static_cast<int>(g % blocks) * kLines);
       for (int i = threadIdx.x; i < kLines * M; i += THREADS)  // 8-byte copies, 64 B per row
         cp_async8(lines + (i % kLines) * LS + i / kLines, base + off(P.ay, i / kLines) + i % kLines);
+      // the next group's rows are requested while this one transforms, so that its
+      // copies then wait for L2, not for DRAM
       if (const int64_t gn = g + gridDim.x; gn < static_cast<int64_t>(M) * blocks) {
         const float2 *next = P.work + off(P.az, static_cast<int>(gn / blocks)) + off(P.ax, static_cast<int>(gn % blocks) * kLines);
         for (int e = threadIdx.x; e < M; e += THREADS) prefetch_l2(next + off(P.ay, e));

@@ -411,6 +411,9 @@ __device__ __forceinline__ void gauss7_run(float2 *out, uint16_t *list, const fl
   }
 }
 
+// Start a line on its way to L2.
+__device__ __forceinline__ void prefetch_l2(const void *p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
+
 // Prefetch into L2 the four voxel rows (y0|y1, z0|z1) that the trilinear
 // stencil at (px, py, pz) reads, for the paired layouts (each row's two
 // corners x0, x0 + 1 are adjacent).
@@ -440,7 +443,7 @@ __device__ __forceinline__ void prefetch_stencil(const float *__restrict__ d, in
   }
   const char *base = reinterpret_cast<const char *>(d);
 #pragma unroll
-  for (int r = 0; r < 4; ++r) asm volatile("prefetch.global.L2 [%0];" ::"l"(base + kRecord * row[r]));
+  for (int r = 0; r < 4; ++r) prefetch_l2(base + kRecord * row[r]);
 }
 
 // ------------------------------------------------------------------ FGPA
@@ -456,22 +459,35 @@ __device__ __forceinline__ float fgpa(float4 tab, float delta, float eta) {
 }
 
 // ------------------------------------------------------------------ statistics
-// Per-warp accumulators in shared memory, FP32 with Kahan compensation
-// (each slot has one writer lane), flushed to FP64 at the end of the kernel:
-//   sums[n_z][NSUM] (float2 {sum, compensation}), p1d[n_z][n_k] (float2),
-//   nseg[n_z] (uint32)
-struct WarpAcc {
-  float2 *sums, *p1d;
+// Accumulators of a team of N/256 warps in shared memory, FP32 with Kahan
+// compensation (float2 {sum, compensation}; each slot has one writer lane),
+// flushed to FP64 at the end of the kernel:
+//   sums[warps][n_z][NSUM], p1d[n_z][slots], nseg[n_z] (uint32)
+// A warp holds N/2 / warps = 128 of a segment's modes, so with n_k >= warps bins a
+// bin's modes lie in one warp and the team shares one set of slots; with fewer
+// bins every warp has a slot of its own.  (A set per warp took 8 n_z n_k bytes for
+// every warp of the team: at N = 1024 and 16 x 32 bins that left one CTA per SM.)
+template <int N>
+struct TeamAcc {
+  static constexpr int WARPS = N / 256;
+  float2 *sums, *p1d;  // sums: this warp's
   uint32_t *nseg;
+  __host__ __device__ static int slots(int n_k) { return WARPS == 1 || n_k > WARPS ? n_k : WARPS; }
   __host__ __device__ static size_t bytes(int n_z, int n_k) {
-    return ((sizeof(float2) * n_z * (MK_NSUM + n_k) + sizeof(uint32_t) * n_z) + 15) / 16 * 16;
+    return ((sizeof(float2) * n_z * (WARPS * MK_NSUM + slots(n_k)) + sizeof(uint32_t) * n_z) + 15) / 16 * 16;
   }
-  __device__ static WarpAcc at(unsigned char *base, int n_z, int n_k) {
-    WarpAcc a;
-    a.sums = reinterpret_cast<float2 *>(base);
-    a.p1d = a.sums + n_z * MK_NSUM;
-    a.nseg = reinterpret_cast<uint32_t *>(a.p1d + n_z * n_k);
+  __device__ static TeamAcc at(unsigned char *base, int warp_of_team, int n_z, int n_k) {
+    TeamAcc a;
+    float2 *s = reinterpret_cast<float2 *>(base);
+    a.sums = s + warp_of_team * n_z * MK_NSUM;
+    a.p1d = s + WARPS * n_z * MK_NSUM;
+    a.nseg = reinterpret_cast<uint32_t *>(a.p1d + n_z * slots(n_k));
     return a;
+  }
+  // every thread of the team; a barrier has to follow
+  __device__ static void zero(unsigned char *base, int n_z, int n_k, int t) {
+    float *f = reinterpret_cast<float *>(base);
+    for (size_t i = t; i < bytes(n_z, n_k) / sizeof(float); i += N / 8) f[i] = 0.f;
   }
 };
 
@@ -521,8 +537,8 @@ struct PixelSums {
 // for bit.  The staged statistics kernel gains (4.57 -> 4.36 ms a pass of 1M
 // skewers); the fused kernel (11.10 -> 11.26 ms a step) and the direct statistics
 // kernel (1.07 -> 1.25 ms a call) lose more to instruction fetches.
-template <bool HALVE>
-__device__ __forceinline__ void flush_bin_sums(const WarpAcc &W, int n_z, int zb, const PixelSums &a, int lane) {
+template <bool HALVE, int N>
+__device__ __forceinline__ void flush_bin_sums(const TeamAcc<N> &W, int n_z, int zb, const PixelSums &a, int lane) {
   float v[MK_NSUM] = {a.n, a.f, a.ff, a.m1.x, a.m1.y, a.m2.x, a.m2.y, a.de, a.fm.x, a.fm.y};
   if constexpr (HALVE) {
     static_assert(MK_NSUM == 10, "the halving steps");
@@ -558,31 +574,23 @@ __device__ __forceinline__ void flush_bin_sums(const WarpAcc &W, int n_z, int zb
   }
 }
 
-// P1D bins of a thread's 4 modes 4t+1 .. 4t+4 (m modes, n_k equal bins), worked
-// out once per kernel.
-struct P1dBins {
-  int per_bin, group, slot;  // modes per bin, threads of a warp that share a bin (0: several bins per thread), bin of mode 4t+1
-  bool writer;
-  __device__ __forceinline__ P1dBins(int m, int n_k, int t) {
-    per_bin = m / max(n_k, 1);
-    group = per_bin >= 4 ? min(per_bin / 4, 32) : 0;
-    slot = (4 * t) / max(per_bin, 1);
-    writer = group > 0 && (t & (group - 1)) == 0;
-  }
-};
-
-// Add the 4 mode powers of thread t (modes 4t+1..4t+4) to the P1D bins of z
-// bin zb (warp-uniform call).  Every bin slot of a warp has one writer.
-__device__ __forceinline__ void accumulate_p1d(const WarpAcc &W, int n_k, const P1dBins &B, const float (&pk)[4],
-                                               float scale, int zb) {
-  float2 *row = W.p1d + zb * n_k;
-  if (B.group > 0) {
+// Add the 4 mode powers of thread t (modes 4t+1..4t+4) to the P1D slots of z
+// bin zb (warp-uniform call).  A bin holds N/2 / n_k modes and a slot at most the
+// 128 of a warp, both powers of two.  Every slot has one writer.
+template <int N>
+__device__ __forceinline__ void accumulate_p1d(const TeamAcc<N> &W, int n_k, int t, const float (&pk)[4], float scale,
+                                               int zb) {
+  constexpr int kLgModes = N == 256 ? 7 : N == 512 ? 8 : N == 1024 ? 9 : 10;
+  const int lg = min(kLgModes + 1 - __ffs(n_k), 7);  // of a slot's modes
+  float2 *row = W.p1d + zb * TeamAcc<N>::slots(n_k) + ((4 * t) >> lg);
+  if (lg >= 2) {
     float s = (pk[0] + pk[1]) + (pk[2] + pk[3]);
-    for (int o = 1; o < B.group; o <<= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    if (B.writer) kahan_add(row[B.slot], s * scale);
+    const int group = 1 << (lg - 2);  // threads that share a slot
+    for (int o = 1; o < group; o <<= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if ((t & (group - 1)) == 0) kahan_add(row[0], s * scale);
   } else {
 #pragma unroll
-    for (int r = 0; r < 4; ++r) kahan_add(row[B.slot + r / B.per_bin], pk[r] * scale);
+    for (int r = 0; r < 4; ++r) kahan_add(row[r >> lg], pk[r] * scale);
   }
 }
 

@@ -48,6 +48,11 @@ cudaError_t launch_pick(const int64_t *off, int64_t n, int k, int64_t *out, cuda
 cudaError_t launch_bin_end(const int16_t *zbin, int32_t j_max, int n_z, int32_t *bin_end, cudaStream_t st);
 cudaError_t launch_out_counts(const mk_skewer *sk, int64_t n, int rebin, int64_t *cnt, cudaStream_t st);
 cudaError_t launch_seg_counts(const int64_t *off, int64_t n, int n_fft, int64_t *cnt, cudaStream_t st);
+// Threads of a CTA, at most 256, that keep the most warps on an SM of sm_smem bytes
+// of shared memory: 256 unless the accumulators of a large binning leave fewer CTAs
+// of them than the register budget would (see best_threads).
+int skewer_threads(int n_fft, int cap, int minb, int sm_smem, int n_z, int n_k, bool stats);
+int stats_threads(int n_fft, int sm_smem, int n_z, int n_k);
 int skewer_blocks_per_sm(int n_fft, int variant, int cap, int minb, int threads, int n_z, int n_k, bool stats);
 // Whether a statistics pass is a tuning pass whose fields can be staged with
 // bulk copies (FGPA table set, rebin 1, 16-byte aligned fields).
@@ -70,6 +75,8 @@ template <int N>
 struct SkewerUnit {
   static int blocks_per_sm(int variant, int cap, int minb, int threads, int n_z, int n_k, bool stats);
   static cudaError_t launch(const SkewerParams &P, int variant, int minb, int grid, int threads, cudaStream_t st);
+  static int skewer_threads(int cap, int minb, int sm_smem, int n_z, int n_k, bool stats);
+  static int stats_threads(int sm_smem, int n_z, int n_k);
   static int stats_blocks_per_sm(int threads, int n_z, int n_k);
   static cudaError_t launch_stats(const StatParams &P, int grid, int threads, cudaStream_t st);
 };

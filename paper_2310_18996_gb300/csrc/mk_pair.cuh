@@ -189,9 +189,7 @@ __device__ __forceinline__ void pair_powers(float2 *buf, const float2 (&v)[8], i
 // ------------------------------------------------------------------ what two segments must not share
 // One transform carries both segments, so a value that is not finite would reach
 // every mode of both, and a segment of much larger values would round its
-// partner's modes away.  Each segment stands for itself: a segment with a value
-// that is not finite enters the transform as zeros and its powers are NaN, and
-// segments that differ too much enter scaled by powers of two.
+// partner's modes away.  Each segment stands for itself.
 //
 // The z bin of a segment's power (za, zb of the kernels) carries a flag for it,
 // which costs no register through the transform.
@@ -201,10 +199,10 @@ __device__ __forceinline__ bool counted(int z, int n_z) {
   return static_cast<unsigned>(z & ~kPartFlag) < static_cast<unsigned>(n_z);
 }
 
-// Flux that comes from the FGPA lies in [0, 1] or is NaN: only the NaN has to be
-// found (a packed sum of the thread's values and a vote; then, rarely, a vote per
-// segment).  A segment that has one becomes zeros and its z bin is flagged.  A
-// barrier of the team.
+// The fused kernel's flux comes from the FGPA and lies in [0, 1] or is NaN: only the
+// NaN has to be found (a packed sum of the thread's values and a vote; then,
+// rarely, a vote per segment).  A segment that has one becomes zeros and its z bin
+// is flagged.  A barrier of the team.
 template <int T>
 __device__ __forceinline__ void drop_nan(float2 (&v)[8], int &za, int &zb, int team) {
   float2 s = v[0];
@@ -218,44 +216,40 @@ __device__ __forceinline__ void drop_nan(float2 (&v)[8], int &za, int &zb, int t
   zb |= b ? kPartFlag : 0;
 }
 
-// Maximum of two values (as unsigned words) over a team.  slots: one per warp of
-// the team, written here; no barrier follows the reads, so the caller needs one
-// before the next call.  A barrier of the team.
+// Stored flux may hold anything (and the tuning pass works as the statistics of its
+// stored flux would).  Where every thread's square sums
+// of the two lie within 2^8 of each other (amplitudes within 16: the transform's
+// rounding stays at the level of the smaller one's own; only a counted segment can
+// be too small), they pass as they are, for 16 instructions and a vote.  Otherwise
+// each counted segment is scaled by the power of two that takes its largest value
+// to [1, 2), one with a value that is not finite becomes zeros, both z bins are
+// flagged and *factors gets what undoes the scale in the powers (twice each), NaN
+// for what is not finite.  buf: the exchange buffer, whose readers are done at the
+// next barrier.  A barrier of the team; the transform's barriers order *factors.
 template <int T>
-__device__ __forceinline__ uint2 team_max(uint2 m, uint2 *slots, int t, int team) {
-  m = make_uint2(__reduce_max_sync(0xffffffffu, m.x), __reduce_max_sync(0xffffffffu, m.y));
-  if constexpr (T == 32) {
-    __syncwarp();
-  } else {
-    if ((t & 31) == 0) slots[t >> 5] = m;
-    team_sync<T>(team);
-#pragma unroll
-    for (int w = 0; w < T / 32; ++w) m = make_uint2(max(m.x, slots[w].x), max(m.y, slots[w].y));
-  }
-  return m;
-}
-
-// Stored flux may hold anything.  Segments whose largest square sums of a thread
-// lie within 2^8 of each other (amplitudes within ~16: the transform's rounding
-// stays at the level of the smaller one's own) pass as they are.  Otherwise each
-// counted segment is scaled by the power of two that takes its largest value to
-// [1, 2), its z bin is flagged and slots[0] gets the factors that undo the scale
-// in the powers (twice each), NaN where a value is not finite.  energies:
-// team_max of the threads' square sums.  The transform's barriers order slots[0].
-template <int T>
-__device__ __forceinline__ void part_segments(float2 (&v)[8], uint2 energies, int &za, int &zb, int n_z, uint2 *slots,
+__device__ __forceinline__ void part_segments(float2 (&v)[8], int &za, int &zb, int n_z, float2 *buf, uint2 *factors,
                                               int t, int team) {
   constexpr uint32_t kInf = 0x7f800000u;
-  const int apart = static_cast<int>(energies.x >> 23) - static_cast<int>(energies.y >> 23);
+  float2 e = f2mul(v[0], v[0]);
+#pragma unroll
+  for (int k = 1; k < 8; ++k) e = f2fma(v[k], v[k], e);
+  const uint32_t ea = __float_as_uint(e.x), eb = __float_as_uint(e.y);
+  const int apart = static_cast<int>(ea >> 23) - static_cast<int>(eb >> 23);
   const bool pa = counted(za, n_z), pb = counted(zb, n_z);
-  if (max(energies.x, energies.y) < kInf && !(pb && apart > 8) && !(pa && apart < -8)) return;
+  if (team_all<T>(team, max(ea, eb) < kInf && !(pb && apart > 8) && !(pa && apart < -8))) return;
   uint2 m = make_uint2(0u, 0u);
 #pragma unroll
   for (int k = 0; k < 8; ++k)
     m = make_uint2(max(m.x, __float_as_uint(v[k].x) & 0x7fffffffu), max(m.y, __float_as_uint(v[k].y) & 0x7fffffffu));
-  team_sync<T>(team);  // the energies are read
-  m = team_max<T>(m, slots, t, team);
-  team_sync<T>(team);  // the maxima are read
+  m = make_uint2(__reduce_max_sync(0xffffffffu, m.x), __reduce_max_sync(0xffffffffu, m.y));
+  if constexpr (T > 32) {
+    uint2 *warps = reinterpret_cast<uint2 *>(buf);
+    if ((t & 31) == 0) warps[t >> 5] = m;
+    team_sync<T>(team);
+#pragma unroll
+    for (int w = 0; w < T / 32; ++w) m = make_uint2(max(m.x, warps[w].x), max(m.y, warps[w].y));
+    team_sync<T>(team);  // (the transform writes there)
+  }
   // 2^-e of the largest value's exponent e; zeros and subnormals stay (their
   // powers are 0 in either case)
   auto down = [](uint32_t w) {
@@ -267,7 +261,7 @@ __device__ __forceinline__ void part_segments(float2 (&v)[8], uint2 energies, in
   for (int k = 0; k < 8; ++k) v[k] = make_float2(a ? v[k].x * da : 0.f, b ? v[k].y * db : 0.f);
   if (t == 0) {
     const uint32_t nan = 0x7fffffffu;
-    slots[0] = make_uint2(m.x < kInf ? __float_as_uint(1.f / da) : nan, m.y < kInf ? __float_as_uint(1.f / db) : nan);
+    *factors = make_uint2(m.x < kInf ? __float_as_uint(1.f / da) : nan, m.y < kInf ? __float_as_uint(1.f / db) : nan);
   }
   za |= kPartFlag;
   zb |= kPartFlag;

@@ -8,11 +8,12 @@
 namespace mk {
 
 // =================================================================== shared-memory plan
+template <int N>
 __host__ __device__ inline size_t acc_bytes(int threads, int n_z, int n_k, bool stats) {
-  return stats ? static_cast<size_t>(threads / 32) * WarpAcc::bytes(n_z, n_k) : 0;
+  return stats ? static_cast<size_t>(threads / (N / 8)) * TeamAcc<N>::bytes(n_z, n_k) : 0;
 }
 
-// Fused kernel, per CTA: per-warp accumulators (when statistics are on), the
+// Fused kernel, per CTA: the teams' accumulators (when statistics are on), the
 // twiddles, the ends of the z bins, then per team one area that is the FFT's
 // exchange buffer and, between the two transforms, the cubics of the pair's
 // cells; a stash of N floats; the skewer's record; and the line, the masks and
@@ -26,13 +27,13 @@ struct PairSmem {
     return f > c ? f : c;
   }
   static constexpr size_t HEAD = (PairFft<N>::TW_BYTES + 15) / 16 * 16 + (sizeof(int32_t) * (MK_MAX_ZBINS + 2) + 15) / 16 * 16;
-  static constexpr int REC = 10;  // 8-byte words: the record, then the end of its pairs
+  static constexpr int REC = 10;  // 8-byte words kept for the record
   __host__ __device__ static size_t team_bytes(int cap) {
     return area_bytes(cap) + sizeof(float) * N + sizeof(uint64_t) * REC +
            (cap > 0 ? CellPlan::kLineBytes + sizeof(uint2) * (N / 16) + sizeof(float) * cap : 0);
   }
   __host__ __device__ static size_t bytes(int threads, int n_z, int n_k, bool stats, int cap) {
-    return acc_bytes(threads, n_z, n_k, stats) + HEAD + static_cast<size_t>(threads / T) * team_bytes(cap);
+    return acc_bytes<N>(threads, n_z, n_k, stats) + HEAD + static_cast<size_t>(threads / T) * team_bytes(cap);
   }
 };
 
@@ -46,31 +47,30 @@ __device__ __forceinline__ int64_t upper_index(const int64_t *a, int64_t n, int6
   return lo;
 }
 
-__device__ __forceinline__ void zero_warp_acc(unsigned char *base, size_t wbytes) {
-  float *f = reinterpret_cast<float *>(base);
-  for (size_t i = threadIdx.x & 31; i < wbytes / sizeof(float); i += 32) f[i] = 0.f;
-  __syncwarp();
-}
-
-// Sum the warps' compensated FP32 accumulators in FP64 and write this CTA's
-// partials in the StatLayout order.
-__device__ __forceinline__ void flush_warp_partials(unsigned char *smem, int nwarps, size_t wbytes, int n_z, int n_k,
-                                    double *partials) {
+// Sum the CTA's compensated FP32 accumulators in FP64, warp after warp, and write
+// its partials in the StatLayout order.
+template <int N>
+__device__ __forceinline__ void flush_partials(unsigned char *smem, int teams, int n_z, int n_k, double *partials) {
+  using A = TeamAcc<N>;
   __syncthreads();
   const StatLayout L{n_z, n_k};
-  const int ns = n_z * MK_NSUM, np = n_z * n_k;
+  const size_t tbytes = A::bytes(n_z, n_k);
+  const int ns = n_z * MK_NSUM, np = n_z * n_k, slots = A::slots(n_k);
+  auto value = [](float2 v) { return static_cast<double>(v.x) - static_cast<double>(v.y); };
   for (int idx = threadIdx.x; idx < L.size(); idx += blockDim.x) {
     double s = 0.0;
-    for (int w = 0; w < nwarps; ++w) {
-      const WarpAcc A = WarpAcc::at(smem + w * wbytes, n_z, n_k);
+#pragma unroll 1
+    for (int team = 0; team < teams; ++team) {
+      const A a = A::at(smem + team * tbytes, 0, n_z, n_k);
       if (idx < ns) {
-        const float2 v = A.sums[idx];
-        s += static_cast<double>(v.x) - static_cast<double>(v.y);
+#pragma unroll 1
+        for (int w = 0; w < A::WARPS; ++w) s += value(a.sums[w * ns + idx]);
       } else if (idx < ns + np) {
-        const float2 v = A.p1d[idx - ns];
-        s += static_cast<double>(v.x) - static_cast<double>(v.y);
+        const int z = (idx - ns) / n_k, k = (idx - ns) % n_k;
+#pragma unroll 1
+        for (int q = k * slots / n_k; q < (k + 1) * slots / n_k; ++q) s += value(a.p1d[z * slots + q]);
       } else {
-        s += static_cast<double>(A.nseg[idx - ns - np]);
+        s += static_cast<double>(a.nseg[idx - ns - np]);
       }
     }
     partials[static_cast<size_t>(blockIdx.x) * L.size() + idx] = s;
@@ -109,14 +109,13 @@ __global__ void __launch_bounds__(256, MINB) k_skewer(SkewerParams P) {
   constexpr int T = N / 8;
   constexpr int kRows = 2;  // rows of T pixels per round of the pixel loop
   const int teams = blockDim.x / T;
-  const int team = threadIdx.x / T, t = threadIdx.x % T, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int team = threadIdx.x / T, t = threadIdx.x % T, lane = threadIdx.x & 31;
   const int wlo0 = t & ~31;  // first team pixel of this warp
-  const int nwarps = blockDim.x >> 5;
   extern __shared__ __align__(16) unsigned char smem[];
-  const size_t wbytes = P.do_stats ? WarpAcc::bytes(P.n_z, P.n_k) : 0;
-  float2 *tws = reinterpret_cast<float2 *>(smem + nwarps * wbytes);
+  const size_t tbytes = P.do_stats ? TeamAcc<N>::bytes(P.n_z, P.n_k) : 0;
+  float2 *tws = reinterpret_cast<float2 *>(smem + teams * tbytes);
   int32_t *bin_end = reinterpret_cast<int32_t *>(tws + (PairFft<N>::TW_BYTES + 15) / 16 * 2);
-  unsigned char *mine = smem + nwarps * wbytes + PairSmem<N>::HEAD + team * PairSmem<N>::team_bytes(P.cell_cap);
+  unsigned char *mine = smem + teams * tbytes + PairSmem<N>::HEAD + team * PairSmem<N>::team_bytes(P.cell_cap);
   float2 *buf = reinterpret_cast<float2 *>(mine);
   CellPlan C;
   C.a = reinterpret_cast<float4 *>(mine);
@@ -127,9 +126,9 @@ __global__ void __launch_bounds__(256, MINB) k_skewer(SkewerParams P) {
   C.line = reinterpret_cast<LineAxis *>(recw + PairSmem<N>::REC);
   C.mask = reinterpret_cast<uint2 *>(C.line + 3);
   C.first = reinterpret_cast<float *>(C.mask + N / 16);
-  const WarpAcc W = WarpAcc::at(smem + warp * wbytes, P.n_z, P.n_k);
+  const TeamAcc<N> W = TeamAcc<N>::at(smem + team * tbytes, t >> 5, P.n_z, P.n_k);
   if (P.do_stats) {
-    zero_warp_acc(smem + warp * wbytes, wbytes);
+    W.zero(smem + team * tbytes, P.n_z, P.n_k, t);
     for (int k = threadIdx.x; k < P.n_z + 2; k += blockDim.x) bin_end[k] = P.bin_end[k];
   }
   fill_pair_twiddles<N>(tws, P.tw);  // (ends with a CTA barrier)
@@ -144,38 +143,36 @@ __global__ void __launch_bounds__(256, MINB) k_skewer(SkewerParams P) {
   int64_t i = u < uend ? upper_index(P.segoff, P.n_sk, u) : 0;
 
   // The skewer's record waits in shared memory, and the next skewer's in a
-  // register of each of ten threads (thread t: word t; t = 9: the end of its
-  // pairs), so that a new skewer costs no round trip to memory.
-  static_assert(sizeof(mk_skewer) == 72, "nine words");
+  // register of each of nine threads (thread t: word t), so that a new skewer costs
+  // no round trip to memory.
+  constexpr int kRecWords = 9;
+  static_assert(sizeof(mk_skewer) == kRecWords * sizeof(uint64_t), "the record's words");
   auto fetch = [&](int64_t q) -> uint64_t {
-    if (q >= P.n_sk) return 0;
-    if (t < 9) return reinterpret_cast<const uint64_t *>(P.sk + q)[t];
-    return t == 9 ? static_cast<uint64_t>(P.segoff[q + 1]) : 0;
+    return q < P.n_sk && t < kRecWords ? reinterpret_cast<const uint64_t *>(P.sk + q)[t] : 0;
   };
   uint64_t next = fetch(i);
-  int64_t base = P.segoff[i], end = base;  // pairs of skewer i - 1 end where i's begin
+  int pair = static_cast<int>(u - P.segoff[i]), left = 0;  // next pair of the skewer, pairs left from it on
   --i;
 
   PixelSums acc;
   acc.zero();
   int zc = -2;  // z bin of acc (warp-uniform), -2 before the first segment
   const uint32_t lanes_le = 0xffffffffu >> (31 - lane);
-  const P1dBins bins(N / 2, P.n_k, t);
   // inner node of this lane, for the search by ballot
   const float ps_node = PSZ && lane >= 1 && lane < P.ps_nodes - 1 ? P.ps_z[lane < MK_MAX_NODES ? lane : 0] : INFINITY;
   const bool put_fields = P.delta_out != nullptr, put_flux = P.flux_out != nullptr;
 
   for (; u < uend; ++u) {
-    while (u >= end) {  // (the last pair ended with a barrier)
-      base = end;
+    while (left == 0) {  // (the last pair ended with a barrier)
       ++i;
-      if (t < PairSmem<N>::REC) recw[t] = next;
+      if (t < kRecWords) recw[t] = next;
       next = fetch(i + 1);
       team_sync<T>(team);
-      end = static_cast<int64_t>(recw[9]);
-      if (u >= end) team_sync<T>(team);  // an empty skewer
+      left = (rec->n + 2 * N - 1) / (2 * N) - pair;
+      if (left == 0) team_sync<T>(team);  // an empty skewer
     }
-    const int s = 2 * static_cast<int>(u - base);
+    const int s = 2 * pair++;
+    if (--left == 0) pair = 0;
     const int64_t offset = rec->offset;
     const int n = rec->n;
     const int j0 = s * N;              // first pixel of the pair
@@ -261,7 +258,8 @@ __global__ void __launch_bounds__(256, MINB) k_skewer(SkewerParams P) {
         load_modes<N>(buf, v, t);
       }
       // (a barrier: the modes are read; the cells are read)
-      if (round == 0) team_sync<T>(team); else drop_nan<T>(v, za, zb, team);
+      if (round == 0) team_sync<T>(team);
+      else drop_nan<T>(v, za, zb, team);
       pair_fft<N>(buf, v, tws, P.tw, t, team);
       if (round == 1) break;
 
@@ -405,12 +403,17 @@ __global__ void __launch_bounds__(256, MINB) k_skewer(SkewerParams P) {
     if (za != -2) {
       float ka[4], kb[4];
       pair_powers<N>(buf, v, t, team, ka, kb);
+      // (N = 512, 1024: the accumulators' place is worked out here; held through the
+      // loop it costs registers, 88 bytes of spills and 3 % at N = 1024)
+      int tm = team, wt = t >> 5;
+      if constexpr (N == 512 || N == 1024) asm volatile("" : "+r"(tm), "+r"(wt));
+      const TeamAcc<N> A = TeamAcc<N>::at(smem + tm * tbytes, wt, P.n_z, P.n_k);
 #pragma unroll 1
       for (int h = 0; h < 2; ++h) {
         if (counted(za, P.n_z)) {
           const int z = za & ~kPartFlag;
-          accumulate_p1d(W, P.n_k, bins, ka, za == z ? 0.25f * P.p1d_scale : __uint_as_float(0x7fffffffu), z);
-          if (t == 0) W.nseg[z] += 1u;
+          accumulate_p1d(A, P.n_k, t, ka, za == z ? 0.25f * P.p1d_scale : __uint_as_float(0x7fffffffu), z);
+          if (t == 0) A.nseg[z] += 1u;
         }
         za = zb;
 #pragma unroll
@@ -422,7 +425,7 @@ __global__ void __launch_bounds__(256, MINB) k_skewer(SkewerParams P) {
   }
   if (P.do_stats) {
     if (zc != -2) flush_bin_sums<false>(W, P.n_z, zc, acc, lane);
-    flush_warp_partials(smem, nwarps, wbytes, P.n_z, P.n_k, P.partials);
+    flush_partials<N>(smem, teams, P.n_z, P.n_k, P.partials);
   }
 }
 

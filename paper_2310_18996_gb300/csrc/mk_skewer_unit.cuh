@@ -4,6 +4,8 @@
 // unit of its own (mk_skewer_<N>.cu), so that the lengths compile in parallel.
 #pragma once
 
+#include <algorithm>
+
 #include "mk_kernels.h"
 #include "mk_skewer.cuh"
 #include "mk_stats.cuh"
@@ -42,6 +44,26 @@ cudaError_t with_skewer_kernel(int variant, int minb, F &&fn) {
   return with_layout<NN, MK_BOX_PLANAR>(psz, cells, minb, fn);
 }
 
+// Shared memory is what a large binning runs out of, team by team (8 n_z (10 +
+// n_k) bytes of accumulators at N = 256), so that two CTAs of 256 threads may not
+// fit where two of 224 do.  Of the multiples of a team up to 256 threads: the one
+// that keeps the most threads resident, the largest of equals; regs: the threads
+// that the register budget holds.  12 x 64 bins at N = 256: tuning pass 1.92 ms with
+// one CTA of 256 threads, 1.53 with two of 224 (12 x 32 bins: 1.29; 300k skewers).
+template <typename F>
+int best_threads(int team, int regs, int sm_smem, F bytes) {
+  constexpr int kReserved = 1024;  // of a CTA, for the system
+  int best = 256, most = 0;
+  for (int threads = 256; threads >= team; threads -= team) {
+    const int ctas = std::min(regs / threads, static_cast<int>(sm_smem / (bytes(threads) + kReserved)));
+    if (ctas * threads > most) {
+      most = ctas * threads;
+      best = threads;
+    }
+  }
+  return best;
+}
+
 template <typename K>
 int occupancy(K kern, int threads, size_t smem) {
   cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
@@ -50,6 +72,19 @@ int occupancy(K kern, int threads, size_t smem) {
   return v;
 }
 }  // namespace skewer_unit_detail
+
+template <int NN>
+int SkewerUnit<NN>::skewer_threads(int cap, int minb, int sm_smem, int n_z, int n_k, bool stats) {
+  return skewer_unit_detail::best_threads(NN / 8, 256 * minb, sm_smem,
+                                          [&](int threads) { return PairSmem<NN>::bytes(threads, n_z, n_k, stats, cap); });
+}
+
+// The same for both variants, which then agree bit for bit.
+template <int NN>
+int SkewerUnit<NN>::stats_threads(int sm_smem, int n_z, int n_k) {
+  return skewer_unit_detail::best_threads(NN / 8, 512, sm_smem,
+                                          [&](int threads) { return StatSmem<NN, true>::bytes(threads, n_z, n_k); });
+}
 
 template <int NN>
 int SkewerUnit<NN>::blocks_per_sm(int variant, int cap, int minb, int threads, int n_z, int n_k, bool stats) {
@@ -74,7 +109,6 @@ cudaError_t SkewerUnit<NN>::launch(const SkewerParams &P, int variant, int minb,
   });
 }
 
-// The same for both variants, which then agree bit for bit.
 template <int NN>
 int SkewerUnit<NN>::stats_blocks_per_sm(int threads, int n_z, int n_k) {
   const int a = skewer_unit_detail::occupancy(k_stats<NN, true>, threads, StatSmem<NN, true>::bytes(threads, n_z, n_k));

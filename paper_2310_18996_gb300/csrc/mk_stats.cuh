@@ -8,7 +8,7 @@
 namespace mk {
 
 // =================================================================== shared memory
-// Per CTA: per-warp accumulators, the twiddles, the ends of the z bins, then per
+// Per CTA: the teams' accumulators, the twiddles, the ends of the z bins, then per
 // team two stage buffers of delta and eta (a pair's transform runs in its own
 // stage buffer once its fields are read) and one mbarrier per buffer, or, when
 // nothing is staged, the transform's exchange buffer.
@@ -17,10 +17,10 @@ struct StatSmem {
   static constexpr int STAGE = 2 * N + 4;  // floats per field and buffer (a pair plus its 16-byte misalignment)
   static_assert(2 * STAGE >= 2 * PairFft<N>::BUF, "a stage buffer holds the exchange buffer");
   static_assert((STAGE * sizeof(float)) % 16 == 0, "stage buffers start on 16 bytes");
-  static constexpr size_t HEAD = PairSmem<N>::HEAD + 8 * sizeof(uint2);  // and a slot per warp for part_segments
+  static constexpr size_t HEAD = PairSmem<N>::HEAD + 8 * sizeof(uint2);  // and the teams' factors of part_segments
   static constexpr size_t TEAM = STAGED ? 4 * STAGE * sizeof(float) + 2 * sizeof(uint64_t) : sizeof(float2) * PairFft<N>::BUF;
   static size_t bytes(int threads, int n_z, int n_k) {
-    return acc_bytes(threads, n_z, n_k, true) + HEAD + static_cast<size_t>(threads / (N / 8)) * TEAM;
+    return acc_bytes<N>(threads, n_z, n_k, true) + HEAD + static_cast<size_t>(threads / (N / 8)) * TEAM;
   }
 };
 
@@ -86,7 +86,9 @@ struct StatPair {
 // z over R pixels (zbin, bin_end) for every R.  (With R > 1 the bin once came
 // from an FP64 division per pixel, and this GPU's FP64 pipe was the bound: flux
 // and statistics of 1.4e8 fine pixels at R = 3 took 3.28 ms then and 1.19 ms with
-// the tables.)
+// the tables.)  Without staging, the next pair's lines are requested into L2 while
+// one is processed: this kernel alone, 2.9e8 fine pixels at R = 3, 1.11 -> 0.82 ms,
+// of it 0.12 from one copy of the bin loop's flush instead of eight.
 //
 // STAGED: a tuning pass (rebin 1, fields and FGPA table set; delta, eta 16-byte
 // aligned): the next pair's fields are copied into shared memory by the bulk-copy
@@ -100,20 +102,19 @@ __global__ void __launch_bounds__(256, 2) k_stats(StatParams P) {
   constexpr int T = N / 8;
   constexpr int STAGE = StatSmem<N, STAGED>::STAGE;
   const int teams = blockDim.x / T;
-  const int team = threadIdx.x / T, t = threadIdx.x % T, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int team = threadIdx.x / T, t = threadIdx.x % T, lane = threadIdx.x & 31;
   const int wlo0 = t & ~31;  // first team pixel of this warp
-  const int nwarps = blockDim.x >> 5;
   extern __shared__ __align__(16) unsigned char smem[];
-  const size_t wbytes = WarpAcc::bytes(P.n_z, P.n_k);
-  float2 *tws = reinterpret_cast<float2 *>(smem + nwarps * wbytes);
+  const size_t tbytes = TeamAcc<N>::bytes(P.n_z, P.n_k);
+  float2 *tws = reinterpret_cast<float2 *>(smem + teams * tbytes);
   int32_t *bin_end = reinterpret_cast<int32_t *>(tws + (PairFft<N>::TW_BYTES + 15) / 16 * 2);
-  unsigned char *areas = smem + nwarps * wbytes + StatSmem<N, STAGED>::HEAD;
-  uint2 *slots = reinterpret_cast<uint2 *>(areas - 8 * sizeof(uint2)) + team * (T / 32);
+  unsigned char *areas = smem + teams * tbytes + StatSmem<N, STAGED>::HEAD;
+  uint2 *factors = reinterpret_cast<uint2 *>(areas - 8 * sizeof(uint2)) + team;
   // stage buffers b = 0, 1: delta at stage_buf + 2 b STAGE, eta at stage_buf + (2 b + 1) STAGE
   float *stage_buf = reinterpret_cast<float *>(areas) + (STAGED ? team * 4 * STAGE : team * 2 * PairFft<N>::BUF);
   uint64_t *bars = reinterpret_cast<uint64_t *>(areas + static_cast<size_t>(teams) * 4 * STAGE * sizeof(float)) + 2 * team;
-  const WarpAcc W = WarpAcc::at(smem + warp * wbytes, P.n_z, P.n_k);
-  zero_warp_acc(smem + warp * wbytes, wbytes);
+  const TeamAcc<N> W = TeamAcc<N>::at(smem + team * tbytes, t >> 5, P.n_z, P.n_k);
+  W.zero(smem + team * tbytes, P.n_z, P.n_k, t);
   for (int k = threadIdx.x; k < P.n_z + 2; k += blockDim.x) bin_end[k] = P.bin_end[k];
   if (STAGED && t == 0) {
     mbar_init(bars);
@@ -131,7 +132,6 @@ __global__ void __launch_bounds__(256, 2) k_stats(StatParams P) {
   PixelSums acc;
   acc.zero();
   int zc = -2;  // z bin of acc (warp-uniform), -2 before the first segment
-  const P1dBins bins(N / 2, P.n_k, t);
 
   // describe pair uu (of skewer inext, advanced as needed); team-uniform
   auto describe = [&](int64_t uu) -> StatPair {
@@ -168,6 +168,16 @@ __global__ void __launch_bounds__(256, 2) k_stats(StatParams P) {
       }
     }
   };
+  auto prefetch = [&](const StatPair &d) {
+    if (!d.ok) return;
+    if (!P.pixtab)
+      for (int i = 32 * t; i < d.npx; i += 32 * T) prefetch_l2(P.flux + d.flux + i);
+    if (P.delta)
+      for (int i = 32 * t; i < d.npx * R; i += 32 * T) {
+        prefetch_l2(P.delta + d.field + i);
+        prefetch_l2(P.eta + d.field + i);
+      }
+  };
   uint32_t parity = 0;  // bit b: parity of stage buffer b's next phase
   StatPair cur{0, 0, 0, 0, false, 0.f, 0.f};
   if (u_first < uend) {
@@ -181,7 +191,7 @@ __global__ void __launch_bounds__(256, 2) k_stats(StatParams P) {
     StatPair nxt = cur;
     if (u + 1 < uend) {
       nxt = describe(u + 1);
-      if (STAGED) stage(nxt, b ^ 1);
+      if (STAGED) stage(nxt, b ^ 1); else prefetch(nxt);
     }
     const int npair = cur.npx, jb0 = cur.jb;
     // z bins of the two segments' first pixels and of the full segments,
@@ -232,11 +242,11 @@ __global__ void __launch_bounds__(256, 2) k_stats(StatParams P) {
       if (npx > 0) {
         const int jb = jb0 + h * N * R;
         float2 x8[8];
-        if (STAGED || P.pixtab) {  // FGPA of the fields (pixels past the end: the last one's table entry, masked)
+        if (STAGED || P.pixtab) {  // FGPA of the fields (pixels past the end: masked; the table has entries for them)
           float4 tb[8];
           const float4 *tp = P.pixtab + jb + t;
 #pragma unroll
-          for (int q = 0; q < 8; ++q) tb[q] = __ldg(tp + min(T * q, rem - 1));
+          for (int q = 0; q < 8; ++q) tb[q] = __ldg(tp + T * q);
 #pragma unroll
           for (int q = 0; q < 8; ++q) {
             const bool on = T * q < rem;
@@ -286,31 +296,25 @@ __global__ void __launch_bounds__(256, 2) k_stats(StatParams P) {
           const int d = bin_end[zc + 1] - jb;
           return R == 1 ? d : (d + R - 1) / R;
         };
-        int pend = bin_stop();
-        // warp-uniform: this warp's pixels of the segment all lie before pend
-        if (min(T * 7 + wlo0 + 32, npx) <= pend) {
-          // (F and the fields of pixels past the end are 0)
+        int pend = bin_stop(), done = 0;
+        const int whi = min(T * 7 + wlo0 + 32, npx);  // end of this warp's pixels
+        if (whi <= pend) {  // (F and the fields of pixels past the end are 0)
 #pragma unroll
           for (int q = 0; q < 8; ++q) acc.add_sums(f8[q], x8[q]);
           acc.n += static_cast<float>(max(0, min(8, (rem + T - 1) / T)));
-        } else {
+        } else {  // bin after bin (one copy of the flush: unrolled over the pixels it was 900 instructions more)
+#pragma unroll 1
+          for (;;) {
+            const int stop = min(pend, npx) - t;
 #pragma unroll
-          for (int q = 0; q < 8; ++q) {
-            const int p = t + T * q;
-            // this warp's pixels at q: T q + wlo0 + lane; flush while they pass pend
-            const int hi = min(T * q + wlo0 + 32, npx);
-            bool todo = p < npx;
-            while (hi > pend) {
-              if (todo && p < pend) {
-                acc.add(f8[q], x8[q]);
-                todo = false;
-              }
-              flush_bin_sums<STAGED>(W, P.n_z, zc, acc, lane);
-              acc.zero();
-              ++zc;
-              pend = bin_stop();
-            }
-            if (todo) acc.add(f8[q], x8[q]);
+            for (int q = 0; q < 8; ++q)
+              if (T * q >= done - t && T * q < stop) acc.add(f8[q], x8[q]);
+            if (whi <= pend) break;
+            flush_bin_sums<STAGED>(W, P.n_z, zc, acc, lane);
+            acc.zero();
+            ++zc;
+            done = pend;
+            pend = bin_stop();
           }
         }
       }
@@ -323,11 +327,7 @@ __global__ void __launch_bounds__(256, 2) k_stats(StatParams P) {
     if (!(counted(za, P.n_z) || counted(zb, P.n_z))) {
       team_sync<T>(team);
     } else {
-      float2 e = f2mul(v[0], v[0]);
-#pragma unroll
-      for (int k = 1; k < 8; ++k) e = f2fma(v[k], v[k], e);
-      const uint2 energies = team_max<T>(make_uint2(__float_as_uint(e.x), __float_as_uint(e.y)), slots, t, team);
-      part_segments<T>(v, energies, za, zb, P.n_z, slots, t, team);
+      part_segments<T>(v, za, zb, P.n_z, buf, factors, t, team);
       pair_fft<N>(buf, v, tws, P.tw, t, team);
       float ka[4], kb[4];
       pair_powers<N>(buf, v, t, team, ka, kb);
@@ -335,20 +335,20 @@ __global__ void __launch_bounds__(256, 2) k_stats(StatParams P) {
       for (int h = 0; h < 2; ++h) {
         if (counted(za, P.n_z)) {
           const int z = za & ~kPartFlag;
-          const float up = za == z ? 1.f : __uint_as_float(h ? slots[0].y : slots[0].x);
-          accumulate_p1d(W, P.n_k, bins, ka, 0.25f * P.p1d_scale * up * up, z);
+          const float up = za == z ? 1.f : __uint_as_float(h ? factors->y : factors->x);
+          accumulate_p1d(W, P.n_k, t, ka, 0.25f * P.p1d_scale * up * up, z);
           if (t == 0) W.nseg[z] += 1u;
         }
         za = zb;
 #pragma unroll
         for (int j = 0; j < 4; ++j) ka[j] = kb[j];
       }
-      if (T > 32 && (zb & kPartFlag)) team_sync<T>(team);  // slots[0] is read
+      if (T > 32 && (zb & kPartFlag)) team_sync<T>(team);  // *factors is read
     }
     cur = nxt;
   }
   if (zc != -2) flush_bin_sums<STAGED>(W, P.n_z, zc, acc, lane);
-  flush_warp_partials(smem, nwarps, wbytes, P.n_z, P.n_k, P.partials);
+  flush_partials<N>(smem, teams, P.n_z, P.n_k, P.partials);
 }
 
 }  // namespace mk
