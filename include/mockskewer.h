@@ -460,9 +460,9 @@ int mk_run_host(mk_ctx *ctx, const mk_box *box, const mk_qso *h_qso, int64_t n_q
    per SM (2, 3 or 4).  layout: the box layout, plus 16 for MK_INTERP_GAUSS7,
    plus 32 for P_S tables at several redshifts (p_s_nodes >= 2; that
    instance has one register budget: 2 for MK_BOX_TENSOR up to N = 1024, else
-   3), plus 64 for trilinear interpolation
-   with pixels longer than 0.1 cell (p_s_nodes and length as before; that
-   instance has one register budget too).
+   3), plus 64 for the kernel that takes single segments, which a trilinear run
+   uses where its pixels are longer than 0.115 to 0.25 cells (by N and layout)
+   or no skewer has two segments (n_max <= n_fft); it has one register budget, 3.
    MK_OK when the autotuner chose it, MK_ERANGE when it is the default
    (still written). */
 int mk_launch_config(mk_ctx *ctx, int32_t n_fft, int32_t layout, int32_t big_box, uint32_t flags,

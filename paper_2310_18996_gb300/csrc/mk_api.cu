@@ -514,30 +514,30 @@ int skewer_grid(mk_ctx *ctx, int n_fft, int variant, int cap, LaunchCfg cfg, con
 }
 
 // A shape of 256 threads with as many as the binning's accumulators let run.
-LaunchCfg shaped(mk_ctx *ctx, int n_fft, int cap, LaunchCfg cfg, const mk_stat_bins *bins) {
+LaunchCfg shaped(mk_ctx *ctx, int n_fft, int variant, int cap, LaunchCfg cfg, const mk_stat_bins *bins) {
   if (bins && cfg.threads == 256)
-    cfg.threads = skewer_threads(n_fft, cap, cfg.minb, ctx->sm_smem, bins->n_z, bins->n_k, true);
+    cfg.threads = skewer_threads(n_fft, variant, cap, cfg.minb, ctx->sm_smem, bins->n_z, bins->n_k, true);
   return cfg;
 }
 
 LaunchCfg default_cfg(int n_fft, int variant) {
-  return LaunchCfg{256, default_budget(n_fft, variant & (kGauss7Variant - 1))};
+  return LaunchCfg{256, variant & kSegmentVariant ? 3 : default_budget(n_fft, variant & (kGauss7Variant - 1))};
 }
 
 // kernel variant: the box layout, plus kGauss7Variant for the Gaussian kernel,
-// plus kPsNodesVariant for P_s tables at several redshifts, plus
-// kPixelGatherVariant where pixels are too long for the cells
+// plus kPsNodesVariant for P_s tables at several redshifts, plus kSegmentVariant
+// where pairs of segments do not pay
 int kernel_variant(const mk_box *box, const mk_skewer_params *p) {
+  const bool segment = p->interp == MK_INTERP_TRILINEAR &&
+                       !use_pairs(p->n_fft, box->desc.layout, p->dr / box->desc.cell, p->n_max);
   return box->desc.layout | (p->interp == MK_INTERP_GAUSS7 ? kGauss7Variant : 0) |
-         (p->p_s_nodes >= 2 ? kPsNodesVariant : 0) |
-         (p->interp == MK_INTERP_TRILINEAR && !use_cells(p->dr, box->desc.cell) ? kPixelGatherVariant : 0);
+         (p->p_s_nodes >= 2 ? kPsNodesVariant : 0) | (segment ? kSegmentVariant : 0);
 }
 
-// cells the sight line of a pair of segments may cross (0: the kernel gathers per pixel)
+// cells the sight line of a pair of segments may cross (0: not by cells)
 int run_cells(const mk_box *box, const mk_skewer_params *p) {
-  return p->interp == MK_INTERP_TRILINEAR && use_cells(p->dr, box->desc.cell)
-             ? cell_capacity(p->n_fft, p->dr / box->desc.cell)
-             : 0;
+  return kernel_variant(box, p) & (kGauss7Variant | kSegmentVariant) ? 0
+                                                                     : cell_capacity(p->n_fft, p->dr / box->desc.cell);
 }
 
 int check_interp(mk_ctx *ctx, const mk_box *box, const mk_skewer_params *p) {
@@ -569,7 +569,7 @@ GeomParams geom_params(mk_ctx *ctx, const mk_box *box, const mk_skewer_params *p
   for (int d = 0; d < 3; ++d) G.origin[d] = box->desc.origin[d];
   G.inv_cell = 1.0 / box->desc.cell;
   G.j_max = ctx->j_max;
-  G.unit_px = 2 * p->n_fft;
+  G.unit_px = kernel_variant(box, p) & kSegmentVariant ? p->n_fft : 2 * p->n_fft;
   return G;
 }
 
@@ -1032,7 +1032,7 @@ int mk_run(mk_ctx *ctx, const mk_box *box, const mk_qso *d_qso, int64_t n_qso, c
     float best = 1e30f;
     for (const LaunchCfg &shape : cand) {
       if (shape.threads < params->n_fft / 8) continue;  // a team must fit in a CTA
-      const LaunchCfg c = shaped(ctx, params->n_fft, S.cell_cap, shape, stats ? bins : nullptr);
+      const LaunchCfg c = shaped(ctx, params->n_fft, variant, S.cell_cap, shape, stats ? bins : nullptr);
       const int grid = skewer_grid(ctx, params->n_fft, variant, S.cell_cap, c, stats ? bins : nullptr);
       if ((rc = ensure_partials(grid))) break;
       if ((rc = enqueue_geometry(ctx, G, d_qso, n_qso, d_sk, d_offsets))) break;
@@ -1057,7 +1057,7 @@ int mk_run(mk_ctx *ctx, const mk_box *box, const mk_qso *d_qso, int64_t n_qso, c
     ctx->tuned[key] = cfg;
   }
 
-  cfg = shaped(ctx, params->n_fft, S.cell_cap, cfg, stats ? bins : nullptr);
+  cfg = shaped(ctx, params->n_fft, variant, S.cell_cap, cfg, stats ? bins : nullptr);
   const int grid = skewer_grid(ctx, params->n_fft, variant, S.cell_cap, cfg, stats ? bins : nullptr);
   if ((rc = ensure_partials(grid))) return rc;
 
@@ -1175,7 +1175,7 @@ int mk_run_host(mk_ctx *ctx, const mk_box *box, const mk_qso *h_qso, int64_t n_q
   LaunchCfg cfg = default_cfg(params->n_fft, variant);
   auto it = ctx->tuned.find(tune_key(params->n_fft, variant, box->lgn, kflags));
   if (it != ctx->tuned.end()) cfg = it->second;
-  cfg = shaped(ctx, params->n_fft, run_cells(box, params), cfg, stats ? bins : nullptr);
+  cfg = shaped(ctx, params->n_fft, variant, run_cells(box, params), cfg, stats ? bins : nullptr);
   const int grid = skewer_grid(ctx, params->n_fft, variant, run_cells(box, params), cfg, stats ? bins : nullptr);
   const StatLayout L{stats ? bins->n_z : 0, stats ? bins->n_k : 0};
   if (stats && (rc = grow(ctx, reinterpret_cast<void **>(&ctx->d_partials), &ctx->partials_cap,

@@ -427,8 +427,8 @@ __device__ __forceinline__ void prefetch_stencil(const float *__restrict__ d, in
   int64_t row[4];
   if constexpr (LAYOUT == MK_BOX_PADDED || LAYOUT == MK_BOX_HALO || LAYOUT == MK_BOX_TENSOR) {
     constexpr int h = LAYOUT == MK_BOX_HALO ? 3 : 0;
-    const int64_t n1 = mask + 1 + (LAYOUT == MK_BOX_HALO ? 6 : 1);
-    row[0] = ((z0 + h) * n1 + (y0 + h)) * n1 + (x0 + h);
+    const uint32_t n1 = mask + 1 + (LAYOUT == MK_BOX_HALO ? 6 : 1);
+    row[0] = static_cast<uint64_t>((z0 + h) * n1 + (y0 + h)) * n1 + (x0 + h);
     row[1] = row[0] + n1;
     row[2] = row[0] + n1 * n1;
     row[3] = row[2] + n1;

@@ -568,8 +568,8 @@ cudaError_t launch_skewer(const SkewerParams &P, int n_fft, int variant, int min
   MK_SWITCH(launch(P, variant, minb, grid, threads, st), cudaErrorInvalidValue)
 }
 
-int skewer_threads(int n_fft, int cap, int minb, int sm_smem, int n_z, int n_k, bool stats) {
-  MK_SWITCH(skewer_threads(cap, minb, sm_smem, n_z, n_k, stats), 256)
+int skewer_threads(int n_fft, int variant, int cap, int minb, int sm_smem, int n_z, int n_k, bool stats) {
+  MK_SWITCH(skewer_threads(variant, cap, minb, sm_smem, n_z, n_k, stats), 256)
 }
 
 int stats_threads(int n_fft, int sm_smem, int n_z, int n_k) { MK_SWITCH(stats_threads(sm_smem, n_z, n_k), 256) }

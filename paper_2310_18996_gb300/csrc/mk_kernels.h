@@ -9,7 +9,7 @@ namespace mk {
 
 constexpr int kGauss7Variant = 16;   // kernel variant bit of MK_INTERP_GAUSS7
 constexpr int kPsNodesVariant = 32;  // kernel variant bit of P_s tables at several redshifts
-constexpr int kPixelGatherVariant = 64;  // kernel variant bit of trilinear gathers per pixel (see use_cells)
+constexpr int kSegmentVariant = 64;  // kernel variant bit of k_segment (see use_pairs)
 
 // Default register budget of the fused kernel, in 256-thread CTAs per SM: three (80
 // registers), or two (128 registers) on a tensor box up to N = 1024, where the
@@ -19,13 +19,26 @@ constexpr int kPixelGatherVariant = 64;  // kernel variant bit of trilinear gath
 // 1.13, N = 2048 2.32 and 2.61 (budget 4 spills: 1.35 to 3.8 ms).
 constexpr int default_budget(int n_fft, int layout) { return layout == MK_BOX_TENSOR && n_fft <= 1024 ? 2 : 3; }
 
-// Whether a trilinear run reads its box through the cells of the sight line
-// (plan_cells in mk_pair.cuh) or gathers pixel by pixel.  Up to dr/cell = 0.1
-// (the paper's is 0.091) a pair's cells fit three rounds of one cell per thread
-// and the shared memory of three CTAs per SM.  At 0.091 the fused kernel takes
-// 1.07 ms per 1.37e8 pixels through the cells and 1.46 ms gathering (N = 256;
-// 1.53 and 2.60 ms on a tensor box, 1.78 and 2.17 ms at N = 1024).
-inline bool use_cells(double dr, double cell) { return dr <= 0.1 * cell; }
+// Whether a trilinear run takes pairs of segments and the cells of its sight line
+// (k_skewer) or single segments and a gather per pixel (k_segment).
+// - Pixel length in cells: a pair's cells grow with it, and past these limits fewer
+//   CTAs fit an SM (12 x 32 bins; the tensor box runs two CTAs anyway and gains more
+//   from reading a corner once).  60k quasars of a 512^3 box, pairs and single
+//   segments in ms: padded N = 256 0.66 and 0.76 at 0.111, 0.80 and 0.76 at 0.133;
+//   N = 1024 1.06 and 1.10 at 0.133, 1.33 and 1.10 at 0.2; N = 2048 1.50 and 1.51 at
+//   0.2; tensor N = 256 1.13 and 1.39 at 0.2, 1.30 and 1.42 at 0.25, 1.60 and 1.45 at
+//   0.3.  (The paper's pixels are 0.091 cells.)
+// - Skewers of one segment at most (n_max) leave half of every pair empty: padded
+//   N = 512, n_max 400: 0.31 and 0.28, N = 1024, n_max 700: 0.61 and 0.54; planar and
+//   tensor boxes, whose corners cost more, and N = 2048 still gain from the cells
+//   (planar N = 1024: 0.63 and 0.66).
+inline bool use_pairs(int n_fft, int layout, double dr_over_cell, int n_max) {
+  if (n_max > 0 && n_max <= n_fft && n_fft <= 1024 && layout != MK_BOX_PLANAR && layout != MK_BOX_TENSOR)
+    return false;
+  const double limit = layout == MK_BOX_TENSOR ? (n_fft <= 1024 ? 0.25 : 0.2)
+                                               : (n_fft == 256 ? 0.115 : n_fft <= 1024 ? 0.14 : 0.2);
+  return dr_over_cell <= limit;
+}
 
 cudaError_t launch_geometry(const mk_qso *q, int64_t nq, const GeomParams &P, mk_skewer *sk, int64_t *cnt_px,
                             int64_t *cnt_seg, int *err, cudaStream_t st);
@@ -51,7 +64,7 @@ cudaError_t launch_seg_counts(const int64_t *off, int64_t n, int n_fft, int64_t 
 // Threads of a CTA, at most 256, that keep the most warps on an SM of sm_smem bytes
 // of shared memory: 256 unless the accumulators of a large binning leave fewer CTAs
 // of them than the register budget would (see best_threads).
-int skewer_threads(int n_fft, int cap, int minb, int sm_smem, int n_z, int n_k, bool stats);
+int skewer_threads(int n_fft, int variant, int cap, int minb, int sm_smem, int n_z, int n_k, bool stats);
 int stats_threads(int n_fft, int sm_smem, int n_z, int n_k);
 int skewer_blocks_per_sm(int n_fft, int variant, int cap, int minb, int threads, int n_z, int n_k, bool stats);
 // Whether a statistics pass is a tuning pass whose fields can be staged with
@@ -63,7 +76,7 @@ inline bool staged_pass(const void *pixtab, const float *delta, const float *eta
 int stats_blocks_per_sm(int n_fft, int threads, int n_z, int n_k);
 // variant: box layout, plus kGauss7Variant for the Gaussian-kernel interpolation,
 // plus kPsNodesVariant for z-dependent P_s (built for the default register budget only),
-// plus kPixelGatherVariant (budget 3 only); cap: cells of a run (P.cell_cap);
+// plus kSegmentVariant (k_segment, budget 3 only); cap: cells of a run (P.cell_cap);
 // minb: register budget of the instance, that of minb 256-thread CTAs per SM
 // (2, 3 or 4)
 cudaError_t launch_skewer(const SkewerParams &P, int n_fft, int variant, int minb, int grid, int threads,
@@ -75,7 +88,7 @@ template <int N>
 struct SkewerUnit {
   static int blocks_per_sm(int variant, int cap, int minb, int threads, int n_z, int n_k, bool stats);
   static cudaError_t launch(const SkewerParams &P, int variant, int minb, int grid, int threads, cudaStream_t st);
-  static int skewer_threads(int cap, int minb, int sm_smem, int n_z, int n_k, bool stats);
+  static int skewer_threads(int variant, int cap, int minb, int sm_smem, int n_z, int n_k, bool stats);
   static int stats_threads(int sm_smem, int n_z, int n_k);
   static int stats_blocks_per_sm(int threads, int n_z, int n_k);
   static cudaError_t launch_stats(const StatParams &P, int grid, int threads, cudaStream_t st);

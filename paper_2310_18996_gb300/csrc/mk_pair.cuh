@@ -356,7 +356,7 @@ struct CellPlan {
 // Cell plan of a run of npx pixels from pixel j0 of a skewer: lines, masks and
 // first pixels; returns the number of cells (the same in every thread).  Starts
 // with the plan's memory free and ends with a team barrier.  A run has at most
-// cell_capacity() <= 3 T cells (see use_cells).
+// cell_capacity() cells.
 template <int N>
 __device__ __forceinline__ int plan_cells(const CellPlan &C, const mk_skewer *rec, int j0, int npx, int t,
                                           int team) {
@@ -377,9 +377,9 @@ __device__ __forceinline__ int plan_cells(const CellPlan &C, const mk_skewer *re
   team_sync<T>(team);
   const int nx = C.line[0].n, nxy = nx + C.line[1].n, total = nxy + C.line[2].n;
   int *at = reinterpret_cast<int *>(C.a);  // (free until the cubics) first pixel past each crossing
-#pragma unroll (N == 256 ? 1 : 3)
-  for (int e = 0; e < 3; ++e) {
-    const int i = t + T * e;
+#pragma unroll 1
+  for (int i0 = 0; i0 < total; i0 += T) {
+    const int i = t + i0;
     if (i < total) {
       const int ax = (i >= nx ? 1 : 0) + (i >= nxy ? 1 : 0);
       const uint32_t k = 1 + i - (i >= nxy ? nxy : (i >= nx ? nx : 0));
@@ -422,9 +422,9 @@ __device__ __forceinline__ int plan_cells(const CellPlan &C, const mk_skewer *re
   }
   if (t == 0) C.first[0] = 0.f;
   team_sync<T>(team);
-#pragma unroll (N == 256 ? 1 : 3)
-  for (int e = 0; e < 3; ++e) {
-    const int i = t + T * e;
+#pragma unroll 1
+  for (int i0 = 0; i0 < total; i0 += T) {
+    const int i = t + i0;
     if (i < total) {
       const int q = at[i];
       const uint2 m = C.mask[q >> 5];
@@ -462,8 +462,8 @@ __device__ __forceinline__ void load_corners(const float *__restrict__ d, const 
   const int mask = (1 << lgn) - 1;
   if constexpr (LAYOUT == MK_BOX_PADDED || LAYOUT == MK_BOX_HALO || LAYOUT == MK_BOX_TENSOR) {
     constexpr int h = LAYOUT == MK_BOX_HALO ? 3 : 0;
-    const int64_t n1 = mask + 1 + (LAYOUT == MK_BOX_HALO ? 6 : 1);
-    const int64_t i00 = ((z0 + h) * n1 + (y0 + h)) * n1 + (x0 + h);
+    const uint32_t n1 = mask + 1 + (LAYOUT == MK_BOX_HALO ? 6 : 1);  // (one 32 x 32 + 64-bit product a point)
+    const int64_t i00 = static_cast<uint64_t>((z0 + h) * n1 + (y0 + h)) * n1 + (x0 + h);
     const int64_t row[4] = {i00, i00 + n1, i00 + n1 * n1, i00 + n1 * n1 + n1};
     if constexpr (LAYOUT == MK_BOX_TENSOR) {
       const float4 *b = reinterpret_cast<const float4 *>(d);
@@ -480,36 +480,26 @@ __device__ __forceinline__ void load_corners(const float *__restrict__ d, const 
       for (int k = 0; k < 8; ++k) v[k] = __ldg(b + row[k >> 1] + (k & 1));
     }
   } else {
-    const int x1 = (x0 + 1) & mask, y1 = (y0 + 1) & mask, z1 = (z0 + 1) & mask;
-    const size_t zz[2] = {static_cast<size_t>(z0) << (2 * lgn), static_cast<size_t>(z1) << (2 * lgn)};
-    const size_t yy[2] = {static_cast<size_t>(y0) << lgn, static_cast<size_t>(y1) << lgn};
+    // (row pointers by a 32 x 32 + 64-bit product each)
+    const uint32_t n = mask + 1, xa = x0, xb = (x0 + 1) & mask, y1 = (y0 + 1) & mask, z1 = (z0 + 1) & mask;
 #pragma unroll
-    for (int k = 0; k < 8; ++k) {
-      const size_t i = zz[k >> 2] | yy[(k >> 1) & 1] | static_cast<size_t>((k & 1) ? x1 : x0);
-      v[k] = LAYOUT == MK_BOX_INTERLEAVED ? __ldg(reinterpret_cast<const float2 *>(d) + i)
-                                          : make_float2(__ldg(d + i), __ldg(e + i));
+    for (int k = 0; k < 4; ++k) {
+      const uint32_t zy = (k & 2 ? z1 : z0) * n + (k & 1 ? y1 : y0);
+      if constexpr (LAYOUT == MK_BOX_INTERLEAVED) {
+        const float2 *row = reinterpret_cast<const float2 *>(reinterpret_cast<const char *>(d) + static_cast<uint64_t>(zy) * (8u * n));
+        v[2 * k] = __ldg(row + xa);
+        v[2 * k + 1] = __ldg(row + xb);
+      } else {
+        const uint64_t i = static_cast<uint64_t>(zy) * n;
+        v[2 * k] = make_float2(__ldg(d + (i | xa)), __ldg(e + (i | xa)));
+        v[2 * k + 1] = make_float2(__ldg(d + (i | xb)), __ldg(e + (i | xb)));
+      }
     }
   }
 }
 
 __device__ __forceinline__ float2 f2fma1(float a, float2 b, float2 c) { return f2fma(make_float2(a, a), b, c); }
 __device__ __forceinline__ float2 f2mul1(float a, float2 b) { return f2mul(make_float2(a, a), b); }
-
-// Trilinear (delta, eta) at one fixed-point position, for pixels too long for
-// the cells of a run to pay: lerps in x, then y, then z, the pair packed.
-template <int LAYOUT>
-__device__ __forceinline__ float2 gather(const float *__restrict__ d, const float *__restrict__ e, int lgn, int64_t px,
-                                         int64_t py, int64_t pz, const int64_t (&st)[3]) {
-  const int mask = (1 << lgn) - 1;
-  float2 v[8];
-  float uu[6];
-  tensor_weights<LAYOUT>(static_cast<float>(st[0]), static_cast<float>(st[1]), static_cast<float>(st[2]), uu);
-  load_corners<LAYOUT>(d, e, lgn, cell_of(px, mask), cell_of(py, mask), cell_of(pz, mask), uu, v);
-  const float tx = weight_of(px), ty = weight_of(py), tz = weight_of(pz);
-  const float2 c0 = f2lerp(v[0], v[1], tx), c1 = f2lerp(v[2], v[3], tx);
-  const float2 c2 = f2lerp(v[4], v[5], tx), c3 = f2lerp(v[6], v[7], tx);
-  return f2lerp(f2lerp(c0, c1, ty), f2lerp(c2, c3, ty), tz);
-}
 
 // The cubic of cell c: the trilinear interpolant of the corners along the line,
 // expanded in the pixel number from the cell's first pixel.  At that pixel it

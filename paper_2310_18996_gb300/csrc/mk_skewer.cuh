@@ -59,7 +59,7 @@ __device__ __forceinline__ void flush_partials(unsigned char *smem, int teams, i
   auto value = [](float2 v) { return static_cast<double>(v.x) - static_cast<double>(v.y); };
   for (int idx = threadIdx.x; idx < L.size(); idx += blockDim.x) {
     double s = 0.0;
-#pragma unroll 1
+#pragma unroll 4
     for (int team = 0; team < teams; ++team) {
       const A a = A::at(smem + team * tbytes, 0, n_z, n_k);
       if (idx < ns) {
@@ -98,15 +98,15 @@ __device__ __forceinline__ void flush_partials(unsigned char *smem, int teams, i
 // pixel loops were unrolled further (4400 to 6000 instructions instead of 3600)
 // ran 10 to 50 % slower, stalled on fetches.
 //
-// CELLS: the trilinear interpolant from the cubics of the line's cells (needs
-// P.cell_cap).  Otherwise INTERP == MK_INTERP_GAUSS7 (LAYOUT must be
-// MK_BOX_HALO): the averages of a segment are computed ahead of its pixel loop
-// into the exchange buffer (gauss7_run); or trilinear with pixels too long for
-// the cells to pay (see use_cells), each pixel gathering for itself.
+// INTERP == MK_INTERP_TRILINEAR: from the cubics of the line's cells (needs
+// P.cell_cap).  MK_INTERP_GAUSS7 (LAYOUT must be MK_BOX_HALO): the averages of a
+// segment are computed ahead of its pixel loop into the exchange buffer
+// (gauss7_run).  Long pixels and catalogues of single segments: k_segment.
 // PSZ: P_s given at several redshifts (P.ps_nodes >= 2), interpolated per segment
-template <int N, int LAYOUT, int MINB, int INTERP, bool PSZ, bool CELLS>
+template <int N, int LAYOUT, int MINB, int INTERP, bool PSZ>
 __global__ void __launch_bounds__(256, MINB) k_skewer(SkewerParams P) {
   constexpr int T = N / 8;
+  constexpr bool CELLS = INTERP == MK_INTERP_TRILINEAR;
   constexpr int kRows = 2;  // rows of T pixels per round of the pixel loop
   const int teams = blockDim.x / T;
   const int team = threadIdx.x / T, t = threadIdx.x % T, lane = threadIdx.x & 31;
@@ -194,7 +194,7 @@ __global__ void __launch_bounds__(256, MINB) k_skewer(SkewerParams P) {
     }
     // ---- start the box rows of the pair's stencils on their way to L2, where
     // the loads are many (the tensor's 64 bytes a corner row, 1.57 -> 1.48 ms
-    // per 1.4e8 pixels; gathers per pixel): lane t samples pixel 16t + 8.  The
+    // per 1.4e8 pixels; the Gaussian kernel's): lane t samples pixel 16t + 8.  The
     // 8-byte layouts read each cell once and gain nothing from it.
     if constexpr (!CELLS || LAYOUT == MK_BOX_TENSOR) {
       const int64_t q = j0 + min(npair - 1, 16 * t + 8);
@@ -315,14 +315,8 @@ __global__ void __launch_bounds__(256, MINB) k_skewer(SkewerParams P) {
           auto interpolate = [&](int d, int k) -> float2 {
             if constexpr (CELLS) {
               return eval_cell(C, mp[k * (T / 32)], qf + static_cast<float>(T * k), lanes_le);
-            } else if constexpr (INTERP == MK_INTERP_GAUSS7) {
-              return buf[t + d + T * k];
             } else {
-              const int q = j0 + h * N + t + d + T * k;
-              const int64_t st[3] = {rec->step[0], rec->step[1], rec->step[2]};
-              const int64_t px = rec->p0[0] + kRoundQ + q * st[0], py = rec->p0[1] + kRoundQ + q * st[1],
-                            pz = rec->p0[2] + kRoundQ + q * st[2];
-              return gather<LAYOUT>(P.box_d, P.box_e, P.lgn, px, py, pz, st);
+              return buf[t + d + T * k];
             }
           };
           auto flux_of = [&](float2 de, float4 tb, float ds, float2 &x) -> float {

@@ -7,6 +7,7 @@
 #include <algorithm>
 
 #include "mk_kernels.h"
+#include "mk_segment.cuh"
 #include "mk_skewer.cuh"
 #include "mk_stats.cuh"
 
@@ -16,32 +17,37 @@ namespace skewer_unit_detail {
 
 // minb: register budget of the instance, that of minb 256-thread CTAs per SM;
 // psz: P_s tables at several redshifts (one instance per layout, of the default budget)
-template <int NN, int L, int INTERP, bool CELLS, typename F>
+template <int NN, int L, int INTERP, typename F>
 cudaError_t with_budget(bool psz, int minb, F &&fn) {
-  if (psz) return fn(k_skewer<NN, L, default_budget(NN, L), INTERP, true, CELLS>);
-  if (minb >= 4) return fn(k_skewer<NN, L, 4, INTERP, false, CELLS>);
-  if (minb == 3) return fn(k_skewer<NN, L, 3, INTERP, false, CELLS>);
-  return fn(k_skewer<NN, L, 2, INTERP, false, CELLS>);
+  if (psz) return fn(k_skewer<NN, L, default_budget(NN, L), INTERP, true>);
+  if (minb >= 4) return fn(k_skewer<NN, L, 4, INTERP, false>);
+  if (minb == 3) return fn(k_skewer<NN, L, 3, INTERP, false>);
+  return fn(k_skewer<NN, L, 2, INTERP, false>);
 }
 
 template <int NN, int L, typename F>
-cudaError_t with_layout(bool psz, bool cells, int minb, F &&fn) {
-  if (cells) return with_budget<NN, L, MK_INTERP_TRILINEAR, true>(psz, minb, fn);
-  return psz ? fn(k_skewer<NN, L, 3, MK_INTERP_TRILINEAR, true, false>)
-             : fn(k_skewer<NN, L, 3, MK_INTERP_TRILINEAR, false, false>);
+cudaError_t with_layout(bool psz, bool segment, int minb, F &&fn) {
+  if (!segment) return with_budget<NN, L, MK_INTERP_TRILINEAR>(psz, minb, fn);
+  return psz ? fn(k_segment<NN, L, 3, true>) : fn(k_segment<NN, L, 3, false>);
 }
 
 // Calls fn with the kernel instance for (kernel variant, register budget).
 template <int NN, typename F>
 cudaError_t with_skewer_kernel(int variant, int minb, F &&fn) {
-  const bool psz = (variant & kPsNodesVariant) != 0, cells = (variant & kPixelGatherVariant) == 0;
+  const bool psz = (variant & kPsNodesVariant) != 0, segment = (variant & kSegmentVariant) != 0;
   const int layout = variant & (kGauss7Variant - 1);
-  if (variant & kGauss7Variant) return with_budget<NN, MK_BOX_HALO, MK_INTERP_GAUSS7, false>(psz, minb, fn);
-  if (layout == MK_BOX_HALO) return with_layout<NN, MK_BOX_HALO>(psz, cells, minb, fn);
-  if (layout == MK_BOX_TENSOR) return with_layout<NN, MK_BOX_TENSOR>(psz, cells, minb, fn);
-  if (layout == MK_BOX_PADDED) return with_layout<NN, MK_BOX_PADDED>(psz, cells, minb, fn);
-  if (layout == MK_BOX_INTERLEAVED) return with_layout<NN, MK_BOX_INTERLEAVED>(psz, cells, minb, fn);
-  return with_layout<NN, MK_BOX_PLANAR>(psz, cells, minb, fn);
+  if (variant & kGauss7Variant) return with_budget<NN, MK_BOX_HALO, MK_INTERP_GAUSS7>(psz, minb, fn);
+  if (layout == MK_BOX_HALO) return with_layout<NN, MK_BOX_HALO>(psz, segment, minb, fn);
+  if (layout == MK_BOX_TENSOR) return with_layout<NN, MK_BOX_TENSOR>(psz, segment, minb, fn);
+  if (layout == MK_BOX_PADDED) return with_layout<NN, MK_BOX_PADDED>(psz, segment, minb, fn);
+  if (layout == MK_BOX_INTERLEAVED) return with_layout<NN, MK_BOX_INTERLEAVED>(psz, segment, minb, fn);
+  return with_layout<NN, MK_BOX_PLANAR>(psz, segment, minb, fn);
+}
+
+template <int NN>
+size_t skewer_smem(int variant, int threads, int n_z, int n_k, bool stats, int cap) {
+  return variant & kSegmentVariant ? SegmentSmem<NN>::bytes(threads, n_z, n_k, stats)
+                                   : PairSmem<NN>::bytes(threads, n_z, n_k, stats, cap);
 }
 
 // Shared memory is what a large binning runs out of, team by team (8 n_z (10 +
@@ -74,9 +80,10 @@ int occupancy(K kern, int threads, size_t smem) {
 }  // namespace skewer_unit_detail
 
 template <int NN>
-int SkewerUnit<NN>::skewer_threads(int cap, int minb, int sm_smem, int n_z, int n_k, bool stats) {
-  return skewer_unit_detail::best_threads(NN / 8, 256 * minb, sm_smem,
-                                          [&](int threads) { return PairSmem<NN>::bytes(threads, n_z, n_k, stats, cap); });
+int SkewerUnit<NN>::skewer_threads(int variant, int cap, int minb, int sm_smem, int n_z, int n_k, bool stats) {
+  return skewer_unit_detail::best_threads(NN / 8, 256 * minb, sm_smem, [&](int threads) {
+    return skewer_unit_detail::skewer_smem<NN>(variant, threads, n_z, n_k, stats, cap);
+  });
 }
 
 // The same for both variants, which then agree bit for bit.
@@ -88,7 +95,7 @@ int SkewerUnit<NN>::stats_threads(int sm_smem, int n_z, int n_k) {
 
 template <int NN>
 int SkewerUnit<NN>::blocks_per_sm(int variant, int cap, int minb, int threads, int n_z, int n_k, bool stats) {
-  const size_t smem = PairSmem<NN>::bytes(threads, n_z, n_k, stats, cap);
+  const size_t smem = skewer_unit_detail::skewer_smem<NN>(variant, threads, n_z, n_k, stats, cap);
   int b = 1;
   skewer_unit_detail::with_skewer_kernel<NN>(variant, minb, [&](auto kern) {
     b = skewer_unit_detail::occupancy(kern, threads, smem);
@@ -100,7 +107,7 @@ int SkewerUnit<NN>::blocks_per_sm(int variant, int cap, int minb, int threads, i
 template <int NN>
 cudaError_t SkewerUnit<NN>::launch(const SkewerParams &P, int variant, int minb, int grid, int threads,
                                    cudaStream_t st) {
-  const size_t smem = PairSmem<NN>::bytes(threads, P.n_z, P.n_k, P.do_stats != 0, P.cell_cap);
+  const size_t smem = skewer_unit_detail::skewer_smem<NN>(variant, threads, P.n_z, P.n_k, P.do_stats != 0, P.cell_cap);
   return skewer_unit_detail::with_skewer_kernel<NN>(variant, minb, [&](auto kern) {
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
     if (e != cudaSuccess) return e;
