@@ -463,6 +463,8 @@ int mk_run_host(mk_ctx *ctx, const mk_box *box, const mk_qso *h_qso, int64_t n_q
    3), plus 64 for the kernel that takes single segments, which a trilinear run
    uses where its pixels are longer than 0.115 to 0.25 cells (by N and layout)
    or no skewer has two segments (n_max <= n_fft); it has one register budget, 3.
+   A shape of 256 threads runs with fewer where the accumulators of a large
+   binning would leave room for fewer warps with 256.
    MK_OK when the autotuner chose it, MK_ERANGE when it is the default
    (still written). */
 int mk_launch_config(mk_ctx *ctx, int32_t n_fft, int32_t layout, int32_t big_box, uint32_t flags,

@@ -521,7 +521,7 @@ LaunchCfg shaped(mk_ctx *ctx, int n_fft, int variant, int cap, LaunchCfg cfg, co
 }
 
 LaunchCfg default_cfg(int n_fft, int variant) {
-  return LaunchCfg{256, variant & kSegmentVariant ? 3 : default_budget(n_fft, variant & (kGauss7Variant - 1))};
+  return LaunchCfg{256, budget_of(n_fft, variant, default_budget(n_fft, variant & (kGauss7Variant - 1)))};
 }
 
 // kernel variant: the box layout, plus kGauss7Variant for the Gaussian kernel,
@@ -546,6 +546,7 @@ int check_interp(mk_ctx *ctx, const mk_box *box, const mk_skewer_params *p) {
   return MK_OK;
 }
 
+// (boxes above 1024^3 keep shapes of their own, as mk_launch_config's big_box says)
 uint64_t tune_key(int n_fft, int variant, int lgn, uint32_t flags) {
   return (static_cast<uint64_t>(n_fft) << 32) | (static_cast<uint64_t>(variant) << 16) |
          (static_cast<uint64_t>(lgn > 10) << 8) | (flags & (MK_STORE_FIELDS | MK_STORE_FLUX | MK_STATS));
@@ -1032,6 +1033,7 @@ int mk_run(mk_ctx *ctx, const mk_box *box, const mk_qso *d_qso, int64_t n_qso, c
     float best = 1e30f;
     for (const LaunchCfg &shape : cand) {
       if (shape.threads < params->n_fft / 8) continue;  // a team must fit in a CTA
+      if (budget_of(params->n_fft, variant, shape.minb) != shape.minb) continue;  // no such instance
       const LaunchCfg c = shaped(ctx, params->n_fft, variant, S.cell_cap, shape, stats ? bins : nullptr);
       const int grid = skewer_grid(ctx, params->n_fft, variant, S.cell_cap, c, stats ? bins : nullptr);
       if ((rc = ensure_partials(grid))) break;

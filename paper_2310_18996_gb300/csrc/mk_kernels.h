@@ -19,6 +19,16 @@ constexpr int kSegmentVariant = 64;  // kernel variant bit of k_segment (see use
 // 1.13, N = 2048 2.32 and 2.61 (budget 4 spills: 1.35 to 3.8 ms).
 constexpr int default_budget(int n_fft, int layout) { return layout == MK_BOX_TENSOR && n_fft <= 1024 ? 2 : 3; }
 
+// Register budget of the instance that runs when a variant is asked for budget
+// `minb` (2, 3 or 4): k_segment and the P_s-node instances exist for one.
+constexpr int budget_of(int n_fft, int variant, int minb) {
+  return variant & kSegmentVariant   ? 3
+         : variant & kPsNodesVariant ? default_budget(n_fft, variant & (kGauss7Variant - 1))
+         : minb < 3                  ? 2
+         : minb > 3                  ? 4
+                                     : 3;
+}
+
 // Whether a trilinear run takes pairs of segments and the cells of its sight line
 // (k_skewer) or single segments and a gather per pixel (k_segment).
 // - Pixel length in cells: a pair's cells grow with it, and past these limits fewer
@@ -75,10 +85,9 @@ inline bool staged_pass(const void *pixtab, const float *delta, const float *eta
 }
 int stats_blocks_per_sm(int n_fft, int threads, int n_z, int n_k);
 // variant: box layout, plus kGauss7Variant for the Gaussian-kernel interpolation,
-// plus kPsNodesVariant for z-dependent P_s (built for the default register budget only),
-// plus kSegmentVariant (k_segment, budget 3 only); cap: cells of a run (P.cell_cap);
-// minb: register budget of the instance, that of minb 256-thread CTAs per SM
-// (2, 3 or 4)
+// plus kPsNodesVariant for z-dependent P_s, plus kSegmentVariant (k_segment); cap: cells
+// of a run (P.cell_cap); minb: register budget asked for, that of minb 256-thread
+// CTAs per SM (see budget_of)
 cudaError_t launch_skewer(const SkewerParams &P, int n_fft, int variant, int minb, int grid, int threads,
                           cudaStream_t st);
 // The fused skewer kernel and the statistics kernel for FFT length N: launch

@@ -15,11 +15,11 @@ namespace mk {
 
 namespace skewer_unit_detail {
 
-// minb: register budget of the instance, that of minb 256-thread CTAs per SM;
-// psz: P_s tables at several redshifts (one instance per layout, of the default budget)
+// minb: register budget of the instance (from budget_of); psz: P_s tables at several
+// redshifts
 template <int NN, int L, int INTERP, typename F>
 cudaError_t with_budget(bool psz, int minb, F &&fn) {
-  if (psz) return fn(k_skewer<NN, L, default_budget(NN, L), INTERP, true>);
+  if (psz) return fn(k_skewer<NN, L, budget_of(NN, L | kPsNodesVariant, 0), INTERP, true>);
   if (minb >= 4) return fn(k_skewer<NN, L, 4, INTERP, false>);
   if (minb == 3) return fn(k_skewer<NN, L, 3, INTERP, false>);
   return fn(k_skewer<NN, L, 2, INTERP, false>);
@@ -28,7 +28,8 @@ cudaError_t with_budget(bool psz, int minb, F &&fn) {
 template <int NN, int L, typename F>
 cudaError_t with_layout(bool psz, bool segment, int minb, F &&fn) {
   if (!segment) return with_budget<NN, L, MK_INTERP_TRILINEAR>(psz, minb, fn);
-  return psz ? fn(k_segment<NN, L, 3, true>) : fn(k_segment<NN, L, 3, false>);
+  constexpr int kBudget = budget_of(NN, L | kSegmentVariant, 0);
+  return psz ? fn(k_segment<NN, L, kBudget, true>) : fn(k_segment<NN, L, kBudget, false>);
 }
 
 // Calls fn with the kernel instance for (kernel variant, register budget).
