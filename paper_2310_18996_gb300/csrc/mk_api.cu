@@ -605,7 +605,6 @@ SkewerParams skewer_params(mk_ctx *ctx, const mk_box *box, const mk_skewer *d_sk
   S.zwin = ctx->d_zwin;
   S.tw = ctx->d_tw[tw_slot(p->n_fft)];
   S.seed = p->seed;
-  S.j_max = ctx->j_max;
   S.segzbin = ctx->zt[0].segzbin;
   S.bin_end = ctx->zt[0].bin_end;
   S.err = ctx->d_err;

@@ -60,24 +60,6 @@ __device__ constexpr float kW32[22][2] = {
     {-1.0f, 0.0f}, {-0.980785251f, -0.195090324f}, {-0.923879504f, -0.382683426f},
     {-0.831469595f, -0.555570245f}, {-0.707106769f, -0.707106769f}, {-0.555570245f, -0.831469595f}};
 
-// 8-point DFT in place, natural order
-template <int SIGN>
-__device__ __forceinline__ void dft8(float2 &v0, float2 &v1, float2 &v2, float2 &v3, float2 &v4, float2 &v5, float2 &v6,
-                                     float2 &v7) {
-  constexpr float kH = 0.70710678118654752f;
-  float2 a0 = f2add(v0, v4), b0 = f2sub(v0, v4), a1 = f2add(v1, v5), b1 = f2sub(v1, v5);
-  float2 a2 = f2add(v2, v6), b2 = f2sub(v2, v6), a3 = f2add(v3, v7), b3 = f2sub(v3, v7);
-  // b1 (1 + SIGN i) / sqrt 2, SIGN i b2, b3 (-1 + SIGN i) / sqrt 2
-  const float2 r1 = cmul_i<SIGN>(b1), r3 = cmul_i<SIGN>(b3);
-  b1 = f2mul(make_float2(b1.x + r1.x, b1.y + r1.y), make_float2(kH, kH));
-  b3 = f2mul(make_float2(r3.x - b3.x, r3.y - b3.y), make_float2(kH, kH));
-  b2 = cmul_i<SIGN>(b2);
-  dft4<SIGN>(a0, a1, a2, a3);
-  dft4<SIGN>(b0, b1, b2, b3);
-  v0 = a0; v2 = a1; v4 = a2; v6 = a3;
-  v1 = b0; v3 = b1; v5 = b2; v7 = b3;
-}
-
 // Place of X[k] after dft32.
 __host__ __device__ constexpr int pos32(int k) { return 4 * (k & 7) + (k >> 3); }
 

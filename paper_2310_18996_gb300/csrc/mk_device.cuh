@@ -53,8 +53,6 @@ __device__ __forceinline__ float2 unit_phase(uint32_t x) {
 __device__ __forceinline__ float sqrt_pos(float x) { return x * rsqrtf(x); }  // x > 0
 
 // ------------------------------------------------------------------ complex helpers
-__device__ __forceinline__ float2 cadd(float2 a, float2 b) { return make_float2(a.x + b.x, a.y + b.y); }
-__device__ __forceinline__ float2 csub(float2 a, float2 b) { return make_float2(a.x - b.x, a.y - b.y); }
 __device__ __forceinline__ float2 cmul(float2 a, float2 b) {
   return make_float2(fmaf(a.x, b.x, -a.y * b.y), fmaf(a.x, b.y, a.y * b.x));
 }
@@ -213,6 +211,24 @@ __device__ __forceinline__ void dft4(float2 &v0, float2 &v1, float2 &v2, float2 
   const float2 d = cmul_i<SIGN>(e);
   v1 = make_float2(b.x + d.x, b.y + d.y);
   v3 = make_float2(b.x - d.x, b.y - d.y);
+}
+
+// 8-point DFT in place, natural order
+template <int SIGN>
+__device__ __forceinline__ void dft8(float2 &v0, float2 &v1, float2 &v2, float2 &v3, float2 &v4, float2 &v5, float2 &v6,
+                                     float2 &v7) {
+  constexpr float kH = 0.70710678118654752f;
+  float2 a0 = f2add(v0, v4), b0 = f2sub(v0, v4), a1 = f2add(v1, v5), b1 = f2sub(v1, v5);
+  float2 a2 = f2add(v2, v6), b2 = f2sub(v2, v6), a3 = f2add(v3, v7), b3 = f2sub(v3, v7);
+  // b1 (1 + SIGN i) / sqrt 2, SIGN i b2, b3 (-1 + SIGN i) / sqrt 2
+  const float2 r1 = cmul_i<SIGN>(b1), r3 = cmul_i<SIGN>(b3);
+  b1 = f2mul(make_float2(b1.x + r1.x, b1.y + r1.y), make_float2(kH, kH));
+  b3 = f2mul(make_float2(r3.x - b3.x, r3.y - b3.y), make_float2(kH, kH));
+  b2 = cmul_i<SIGN>(b2);
+  dft4<SIGN>(a0, a1, a2, a3);
+  dft4<SIGN>(b0, b1, b2, b3);
+  v0 = a0; v2 = a1; v4 = a2; v6 = a3;
+  v1 = b0; v3 = b1; v5 = b2; v7 = b3;
 }
 
 // Stockham passes after pass 0 (whose butterfly j = t outputs are in v[]).

@@ -58,23 +58,6 @@ __device__ __forceinline__ void fill_pair_twiddles(float2 *tws, const float2 *__
   __syncthreads();
 }
 
-// 8-point forward DFT in place, natural order
-__device__ __forceinline__ void dft8(float2 (&v)[8]) {
-  constexpr float kH = 0.70710678118654752f;
-  float2 a0 = f2add(v[0], v[4]), b0 = f2sub(v[0], v[4]);
-  float2 a1 = f2add(v[1], v[5]), b1 = f2sub(v[1], v[5]);
-  float2 a2 = f2add(v[2], v[6]), b2 = f2sub(v[2], v[6]);
-  float2 a3 = f2add(v[3], v[7]), b3 = f2sub(v[3], v[7]);
-  // b1 (1 - i) / sqrt 2, -i b2, b3 (-1 - i) / sqrt 2
-  b1 = f2mul(make_float2(b1.x + b1.y, b1.y - b1.x), make_float2(kH, kH));
-  b3 = f2mul(make_float2(b3.y - b3.x, -b3.x - b3.y), make_float2(kH, kH));
-  b2 = cmul_i<-1>(b2);
-  dft4<-1>(a0, a1, a2, a3);
-  dft4<-1>(b0, b1, b2, b3);
-  v[0] = a0; v[2] = a1; v[4] = a2; v[6] = a3;
-  v[1] = b0; v[3] = b1; v[5] = b2; v[7] = b3;
-}
-
 // N-point forward complex FFT of a team, v[r] at index t + T r on both ends, natural
 // order.  buf: BUF complex slots, free when the call starts after a team
 // barrier; its contents are undefined on return, and a barrier is needed before
@@ -86,7 +69,7 @@ __device__ __forceinline__ void pair_fft(float2 *buf, float2 (&v)[8], const floa
                                          const float2 *__restrict__ tab, int t, int team) {
   using P = PairFft<N>;
   constexpr int T = P::T;
-  dft8(v);
+  dft8<-1>(v[0], v[1], v[2], v[3], v[4], v[5], v[6], v[7]);
   {
     float2 *w = buf + 8 * t + (t >> 1);
 #pragma unroll
@@ -103,7 +86,7 @@ __device__ __forceinline__ void pair_fft(float2 *buf, float2 (&v)[8], const floa
     const float2 w = tws[P::TW1 + 8 * (r - 1) + (t & 7)];
     v[r] = cmul(v[r], w);
   }
-  dft8(v);
+  dft8<-1>(v[0], v[1], v[2], v[3], v[4], v[5], v[6], v[7]);
   team_sync<T>(team);
   {
     float2 *w = buf + (t >> 3) * 72 + (t & 7);
@@ -126,7 +109,7 @@ __device__ __forceinline__ void pair_fft(float2 *buf, float2 (&v)[8], const floa
       const float2 w = tws[P::TW2 + 64 * (r - 1) + (t & 63)];
       v[r] = cmul(v[r], w);
     }
-    dft8(v);  // N = 512: index t + 64 r, done
+    dft8<-1>(v[0], v[1], v[2], v[3], v[4], v[5], v[6], v[7]);  // N = 512: index t + 64 r, done
     if constexpr (P::F > 1) {
       team_sync<T>(team);
       float2 *w = buf + (t >> 6) * 512 + (t & 63);

@@ -106,7 +106,6 @@ struct SkewerParams {
   const float *zwin;       // per J: mean z of pixels J .. J+N-1 (with ps_nodes >= 2)
   const float2 *tw;      // e^{-2 pi i k/N}, k < N
   uint32_t seed;
-  int32_t j_max;
   // outputs
   float *delta_out, *eta_out, *flux_out;
   int64_t capacity;
