@@ -544,15 +544,15 @@ struct PixelSums {
   }
 };
 
-// Add the warp's PixelSums of bin zb to the warp accumulators (warp-uniform
-// call; bins outside [0, n_z) are dropped).  It runs about once a pair of
-// segments, and its code shares the instruction cache with the segment loop it
-// interrupts: a rolled butterfly of the ten sums (60 instructions, 50 shuffles).
-// HALVE: two steps that halve the values a lane holds (10, 5, 3), then a rolled
-// butterfly of three: 17 shuffles in more code.  Both add in the same order, bit
-// for bit.  The staged statistics kernel gains (4.57 -> 4.36 ms a pass of 1M
-// skewers); the fused kernel (11.10 -> 11.26 ms a step) and the direct statistics
-// kernel (1.07 -> 1.25 ms a call) lose more to instruction fetches.
+// Add the warp's PixelSums of bin zb to its accumulators (warp-uniform call; bins
+// outside [0, n_z) are dropped).  It runs about once a pair of segments.  HALVE: two
+// steps that halve the values a lane holds (10, 5, 3), then a rolled butterfly of
+// three: 17 shuffles.  Otherwise a rolled butterfly of the ten sums, 50 shuffles in 60
+// instructions.  Both add in the same order, bit for bit.  k_skewer, whose loop fills
+// the instruction cache, loses more to fetches than it gains (11.10 -> 11.26 ms a
+// step); the statistics kernels gain (tuning pass of 1M skewers 4.57 -> 4.36 ms,
+// stored flux of 200k at N = 1024 2.24 -> 2.06), and k_segment from N = 512 on (N =
+// 1024: 0.57 -> 0.54 ms).
 template <bool HALVE, int N>
 __device__ __forceinline__ void flush_bin_sums(const TeamAcc<N> &W, int n_z, int zb, const PixelSums &a, int lane) {
   float v[MK_NSUM] = {a.n, a.f, a.ff, a.m1.x, a.m1.y, a.m2.x, a.m2.y, a.de, a.fm.x, a.fm.y};

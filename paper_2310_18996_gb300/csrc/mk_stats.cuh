@@ -288,7 +288,7 @@ __global__ void __launch_bounds__(256, 2) k_stats(StatParams P) {
         }
         // pixel sums
         if (z0[0] != zc || (h == 0 && u % kRunPairs == 0)) {
-          if (zc != -2) flush_bin_sums<STAGED>(W, P.n_z, zc, acc, lane);
+          if (zc != -2) flush_bin_sums<true>(W, P.n_z, zc, acc, lane);
           acc.zero();
           zc = z0[0];
         }
@@ -310,7 +310,7 @@ __global__ void __launch_bounds__(256, 2) k_stats(StatParams P) {
             for (int q = 0; q < 8; ++q)
               if (T * q >= done - t && T * q < stop) acc.add(f8[q], x8[q]);
             if (whi <= pend) break;
-            flush_bin_sums<STAGED>(W, P.n_z, zc, acc, lane);
+            flush_bin_sums<true>(W, P.n_z, zc, acc, lane);
             acc.zero();
             ++zc;
             done = pend;
@@ -347,7 +347,7 @@ __global__ void __launch_bounds__(256, 2) k_stats(StatParams P) {
     }
     cur = nxt;
   }
-  if (zc != -2) flush_bin_sums<STAGED>(W, P.n_z, zc, acc, lane);
+  if (zc != -2) flush_bin_sums<true>(W, P.n_z, zc, acc, lane);
   flush_partials<N>(smem, teams, P.n_z, P.n_k, P.partials);
 }
 
