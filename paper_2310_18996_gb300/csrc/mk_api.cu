@@ -1070,7 +1070,8 @@ int mk_run(mk_ctx *ctx, const mk_box *box, const mk_qso *d_qso, int64_t n_qso, c
     std::memcpy(kp, &G, sizeof(G));
     std::memcpy(kp + sizeof(G), &S, sizeof(S));
     const int64_t extra[8] = {reinterpret_cast<int64_t>(d_qso), n_qso, reinterpret_cast<int64_t>(d_offsets),
-                              static_cast<int64_t>(ctx->generation), grid, cfg.threads * 16 + cfg.minb,
+                              static_cast<int64_t>(ctx->generation), grid,
+                              (variant * 4096 + cfg.threads) * 16 + cfg.minb,  // which kernel
                               static_cast<int64_t>(flags & ~MK_AUTOTUNE),
                               stats ? (bins->n_z * 4096 + bins->n_k * 8 + (bins->n_fft >> 8)) : 0};
     std::memcpy(kp + sizeof(G) + sizeof(S), extra, sizeof(extra));
