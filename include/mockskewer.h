@@ -324,8 +324,9 @@ typedef struct mk_qso_draw_params {
    high), counter (v low, v high, 0x51534F, 0): accepted when
    (w0 + 1/2) 2^-32 < P, at origin + (x + u1, y + u2, z + u3) cell with
    u = (w + 1/2) 2^-32; id = v.  The catalogue lists accepted voxels in
-   increasing v.  The coefficients are tabulated in r (host FP64, 8192
-   points over the box's distance range, linear in between).
+   increasing v.  The coefficients are tabulated in r (FP64, E[p] and the norm on
+   the device, the rest on the host; 8192 points over the box's distance range,
+   kept in FP32, linear in between).
    d_box_q[i]: n^3 floats at stride box_stride (1 planar, 2 for the pairs
    of mk_synth_box's MK_BOX_INTERLEAVED output, which reads delta).
    d_qso: capacity records.  *h_count: quasars drawn (also beyond capacity,

@@ -515,10 +515,10 @@ __device__ __forceinline__ void kahan_add(float2 &acc, float x) {
 }
 
 // Pairs of segments after which a thread's FP32 pixel sums go to the compensated
-// accumulators even if its z bin goes on: 128 pixels a thread at most.  (One wide
+// accumulators even if its z bin goes on: 256 pixels a thread at most.  (One wide
 // bin would otherwise collect 1e5 and more: errors of 1e-6 in the sums, and past
 // 2^24 pixels a wrong count.)  With bins of ordinary width they went before that.
-constexpr int kRunPairs = 8;
+constexpr int kRunPairs = 16;
 
 // Pixel sums of one thread for one z bin, in the StatLayout order
 // n, F, F^2, d, e, d^2, e^2, d e, F d, F e; the (d, e) pairs run packed.

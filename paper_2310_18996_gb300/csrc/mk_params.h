@@ -88,13 +88,13 @@ __host__ __device__ inline void finalize_bin_p1d(mk_stats_bin *b, int k, double 
 // Everything the fused / split skewer kernels read.
 struct SkewerParams {
   const mk_skewer *sk;
-  const int64_t *segoff;  // exclusive prefix of pairs of segments per skewer, n_sk + 1
+  const int64_t *segoff;  // exclusive prefix of pairs of segments (k_segment: segments) per skewer, n_sk + 1
   int64_t n_sk;
   // box
   const float *box_d;  // planar delta, or (delta, eta) pairs (interleaved, padded)
   const float *box_e;  // planar eta or NULL
   int32_t lgn;
-  int32_t cell_cap;  // cells a pair's sight line may cross (0: gathers per pixel)
+  int32_t cell_cap;  // cells a pair's sight line may cross (0: not by cells)
   // tables
   const float4 *pixtab;  // per global pixel J: {G, a log2e, b log2e, c}
   const int16_t *zbin;     // per J: z bin, -1 below, n_z above

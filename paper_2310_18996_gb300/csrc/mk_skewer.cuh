@@ -1,5 +1,5 @@
 // Template of the fused skewer kernel and what it shares with the statistics
-// kernels (mk_stats.cuh); each FFT length is instantiated in its own translation
+// (mk_stats.cuh) and single-segment (mk_segment.cuh) kernels; each FFT length is instantiated in its own translation
 // unit (mk_skewer_<N>.cu).
 #pragma once
 
@@ -17,8 +17,7 @@ __host__ __device__ inline size_t acc_bytes(int threads, int n_z, int n_k, bool 
 // twiddles, the ends of the z bins, then per team one area that is the FFT's
 // exchange buffer and, between the two transforms, the cubics of the pair's
 // cells; a stash of N floats; the skewer's record; and the line, the masks and
-// the cells' first pixels (cap, a multiple of 4, is 0 where pixels gather for
-// themselves).
+// the cells' first pixels (cap, a multiple of 4, is 0 for the Gaussian kernel).
 template <int N>
 struct PairSmem {
   static constexpr int T = N / 8;
@@ -88,15 +87,16 @@ __device__ __forceinline__ void flush_partials(unsigned char *smem, int teams, i
 // accumulators when its pixels reach the end of the bin (bin_end) or a
 // segment starts in another bin.
 //
-// Bound by instruction issue: 6.6 warp instructions a pixel at 68 % of the issue
-// slots, DRAM ~10 B a pixel.  One radix-8 transform for two segments and one set
-// of corner loads per cell of the sight line take 1.07 ms per 1.37e8 pixels
-// (512^3 box, 100k quasars, N = 256) where a radix-4 transform per segment and a
-// gather of eight corners per pixel took 1.25 ms, and 1.53 against 2.19 ms on a
-// tensor box; a step of the 1024^3 box with 1M quasars went from 13.0 to 11.2 ms.
+// Bound by instruction issue: 6.5 warp instructions a pixel at 67 % of the issue
+// slots, DRAM ~10 B a pixel.  60k quasars (8.2e7 pixels, 512^3 box): one radix-8
+// transform for two segments and one set of corner loads per cell of the sight line
+// take 0.66 ms at N = 256 where a radix-4 transform per segment and a gather of
+// eight corners per pixel took 0.74, 0.83 against 1.33 on a tensor box, 1.03 against
+// 1.12 at N = 1024; a step of the 1024^3 box with 1M quasars went from 13.0 to 11.2 ms.
 // The loop over pairs has to fit the instruction cache: variants of it whose
 // pixel loops were unrolled further (4400 to 6000 instructions instead of 3600)
-// ran 10 to 50 % slower, stalled on fetches.
+// ran 10 to 50 % slower, stalled on fetches.  Registers are as scarce: with the cells
+// of one segment at a time (to hold fewer of them) it spilled and was 10 % slower.
 //
 // INTERP == MK_INTERP_TRILINEAR: from the cubics of the line's cells (needs
 // P.cell_cap).  MK_INTERP_GAUSS7 (LAYOUT must be MK_BOX_HALO): the averages of a

@@ -93,8 +93,10 @@ struct StatPair {
 // STAGED: a tuning pass (rebin 1, fields and FGPA table set; delta, eta 16-byte
 // aligned): the next pair's fields are copied into shared memory by the bulk-copy
 // (TMA) engine while the current one is processed.  It reads 8 bytes a pixel and
-// is bound by latency and issue: 2.4 warp instructions a pixel, 4.21 ms per
-// 1.45e9 pixels, where one radix-4 transform per segment took 3.1 and 5.67 ms.
+// is bound by latency and issue: 4.25 ms per 1.45e9 pixels, where one radix-4
+// transform per segment took 5.67 ms; 16 warps an SM by registers.  (Buffers of a
+// segment instead of a pair hold larger binnings at 16 warps, but 1.50 ms where
+// these take 1.29: 300k skewers.)
 // Both variants work through the same pairs in the same order with the same
 // grid, so a tuning pass and the statistics of its stored flux agree bit for bit.
 template <int N, bool STAGED>
